@@ -477,6 +477,7 @@ int run_brute(qa_model* m, const qa_raster* r, int closed, int bound, int8_t* ou
   L.ni = ni;
   L.n_max = closed ? -1 : bound;
   L.nouter = (unsigned long long)(outer + 0.5);
+  L.num_sms = m->num_sms;
   cudaError_t e = qa::launch_brute(L, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "brute-force launch");
   return QA_OK;

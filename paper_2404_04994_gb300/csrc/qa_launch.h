@@ -90,6 +90,10 @@ struct BruteLaunch {
   int ni;
   int n_max;                   // open: box bound reported by kBruteAtBox
   unsigned long long nouter;   // radix^(nfree - ni)
+  int num_sms;
+  // set by launch_brute
+  unsigned long long nhi;      // states of the digits above the last two
+  int team, pix;               // lanes per pixel, pixels per block
 };
 enum : unsigned { kBruteNearTie = 1u, kBruteAtBox = 2u, kBruteNone = 4u };
 cudaError_t launch_brute(const BruteLaunch& L, cudaStream_t st);

@@ -388,7 +388,8 @@ __device__ __forceinline__ double pixel_c_f64(const ModelData* md, int ng,
                                               long long p, int i) {
   double a = 0.0;
   if (sc.kind == 0) {
-    const long long iy = p / sc.W, ix = p - iy * sc.W;
+    // a raster has at most 2^31 - 1 pixels: 32-bit division
+    const unsigned iy = (unsigned)p / (unsigned)sc.W, ix = (unsigned)p - iy * (unsigned)sc.W;
     const double xs = sc.x0 + (int)ix * sc.dx, ys = sc.y0 + (int)iy * sc.dy;
     for (int g = 0; g < ng; ++g) a += md->Cgd[i * ng + g] * (sc.V0[g] + xs * sc.u[g] + ys * sc.w[g]);
   } else {

@@ -117,3 +117,37 @@ def test_brute_force_errors(qa):
         big.brute_force_open(inputs.raster(16, gx, gy, np.zeros(16), W=2, H=2), 127)
     assert e.value.code == -5
     big.close()
+
+
+# The FP32 line search against the oracle where it can go wrong: one state, one
+# line, the largest digit range, many leading digits, closed simplices whose
+# leading digits leave nothing, and exact ties (uncoupled dots at half
+# charges, 2^N of equal energy), which the FP64 shortlist settles.
+@pytest.mark.parametrize("n,closed,bound,W,H", [
+    (1, False, 0, 7, 1), (1, False, 127, 33, 3), (1, True, 0, 3, 1), (2, False, 127, 9, 5),
+    (3, False, 1, 5, 129), (6, False, 3, 7, 3), (10, False, 1, 3, 2), (2, True, 127, 9, 3),
+    (5, True, 6, 11, 3), (6, True, 2, 1, 33)])
+def test_line_search_edges(qa, n, closed, bound, W, H):
+    r = np.random.Generator(np.random.PCG64(500 + n))
+    Cdd, Cgd = inputs.random_model(r, n)
+    gx, gy = (0, 0) if n == 1 else inputs.swept_gates(n)
+    ras = inputs.raster(n, gx, gy, inputs.offsets(r, n, (gx, gy)), W=W, H=H,
+                        hi=140.0 if bound == 127 else 5.0)
+    _check(qa, Cdd, Cgd, ras, closed, bound, f"N={n} closed={closed} bound={bound}")
+
+
+@pytest.mark.parametrize("n", [2, 4])
+@pytest.mark.parametrize("closed", [False, True])
+def test_line_search_exact_ties(qa, n, closed):
+    # every dot at c = 1.5 (open: 2^n equal energies; closed with 2 n - n / 2
+    # charges: n over n / 2 of them): a near tie, the lexicographically
+    # smallest state
+    ras = inputs.raster(n, 0, 1, np.full(n, 1.5), W=1, H=1)
+    ras["V0"][:] = 1.5
+    ras["u"][:] = 0.0
+    ras["w"][:] = 0.0
+    nh = n + n // 2
+    nn, U, f = _brute_gpu(qa, np.eye(n), np.eye(n), ras, closed, nh if closed else 4)
+    want = [1] * (n - n // 2) + [2] * (n // 2) if closed else [1] * n
+    np.testing.assert_array_equal(nn[0], want)
+    assert f[0] & 1 and abs(U[0] - 0.125 * n) < 1e-14
