@@ -39,29 +39,6 @@ struct TeamSlots {
   float ustar_kT;      // U(n*) / kT  (rounded from double-float)
 };
 
-// D(b) = E(b) - E(b*) from the slots that differ from b*: the first-order
-// terms gp / gm of each and the pair terms between them, read from the team's
-// slot-ordered copy of M (Ms[s * KMAX + s2] = M of the dots of slots s, s2).
-template <int KMAX>
-__device__ __forceinline__ float delta_energy(const TeamSlots& ts, const float* Ms,
-                                              unsigned b) {
-  const unsigned d = b ^ ts.bstar;
-  float D = 0.f;
-  for (unsigned m = d; m; m &= m - 1u) {
-    const int s = __ffs(m) - 1;
-    const bool add = (b >> s) & 1u;
-    D += add ? ts.gp[s] : ts.gm[s];
-    const float* row = Ms + s * KMAX;
-    for (unsigned q = d & ((1u << s) - 1u); q; q &= q - 1u) {
-      const int s2 = __ffs(q) - 1;
-      const bool add2 = (b >> s2) & 1u;
-      const float v = row[s2];
-      D += (add == add2) ? v : -v;
-    }
-  }
-  return D;
-}
-
 // v[s] for a runtime s, the array staying in registers.
 template <int K>
 __device__ __forceinline__ float pick(const float (&v)[K], int s) {
@@ -72,15 +49,15 @@ __device__ __forceinline__ float pick(const float (&v)[K], int s) {
   return r;
 }
 
-// Fit step: the pixel's <n> from the slot weight sums accb (slot order) and
+// Fit step: the pixel's <n> from the slot weight sums accb(s) (slot order) and
 // Z, then the MSE gradient g = dL/d<n> into gsh[0, n); returns the pixel's
 // squared residual (summed over the team).  Sum target: r = sum_i <n_i> -
 // target_p and g_i = scale r for every dot; per-dot target: r_i = <n_i> -
 // target_pi and g_i = scale r_i.  The team's lanes take the dots; all lanes
 // of the warp call.
-template <int K>
+template <typename Acc>
 __device__ __forceinline__ float fit_loss_grad_team(const SoftLaunch& a, const TeamSlots& ts,
-                                                    const float (&accb)[K], float Z,
+                                                    const Acc& accb, float Z,
                                                     long long p, float* gsh, int lt, int T,
                                                     bool active) {
   const int n = a.n;
@@ -88,7 +65,7 @@ __device__ __forceinline__ float fit_loss_grad_team(const SoftLaunch& a, const T
   if (active)
     for (int i = lt; i < n; i += T) {
       float v = (float)ts.base[i];
-      if ((ts.mask >> i) & 1u) v += pick<K>(accb, __popc(ts.mask & ((1u << i) - 1u))) / Z;
+      if ((ts.mask >> i) & 1u) v += accb(__popc(ts.mask & ((1u << i) - 1u))) / Z;
       if (a.out_mean) a.out_mean[p * n + i] = v;
       if (a.fit_per_dot) {
         const float r = v - a.fit_target[p * n + i];
@@ -317,186 +294,6 @@ __device__ inline void soft_contrib(const SoftLaunch& a, TeamSlots& ts, const fl
     for (int q = 0; q < teams; ++q) sacc = df_add(sacc, {s_contrib[q * L + e], 0.f});
     out[(size_t)e * gridDim.x + blockIdx.x] = make_float2(sacc.hi, sacc.lo);
   }
-}
-
-// Soft occupation (forward) and, with BWD, the per-block gradient partials.
-template <int L1, int L2, bool CLOSED, bool BWD, int KMAX>
-__global__ void __launch_bounds__(kSoftThreads) k_soft(SoftLaunch a) {
-  __shared__ ModelConsts cs;
-  __shared__ TeamSlots tsm[kSoftThreads / 4 > 0 ? kSoftThreads / 4 : 1];
-  // slot-ordered M per team (teams of >= 4 lanes for KMAX 8, 32 lanes beyond)
-  constexpr int kMaxTeams = kSoftThreads / (KMAX > 8 ? 32 : 4);
-  __shared__ float slotM[kMaxTeams][KMAX * KMAX];
-  __shared__ float sQa[BWD ? kMaxTeams : 1][tri(KMAX) + KMAX + 1];  // Qa, va, sa of a team
-  __shared__ float sGf[BWD ? kMaxTeams : 1][kMaxDot];                 // fit step: g of a team
-  extern __shared__ float s_contrib[];  // BWD: [teams][contrib_len]
-  const int n = a.n;
-  stage_consts(&a.md->k, &cs);
-  __syncthreads();
-  const float* sM = cs.Mhi;
-  const float* sMlo = cs.Mlo;
-  const int T = a.cfg.T;  // >= 4
-  const int team = threadIdx.x / T, lt = threadIdx.x % T;
-  const int teams = blockDim.x / T;
-  const long long p = (long long)blockIdx.x * teams + team;
-  const bool active = p < a.sc.P;
-  TeamSlots& ts = tsm[team];
-  const float kT = (float)a.kT;
-
-  soft_setup_team<CLOSED>(a, ts, p, lt, T, active);
-  float* Ms = slotM[team];
-  if (active)
-    for (int e = lt; e < KMAX * KMAX; e += T) {
-      const int s = e / KMAX, s2 = e % KMAX;
-      Ms[e] = (s < ts.k && s2 < ts.k) ? sM[ts.dot[s] * kLdM + ts.dot[s2]] : 0.f;
-    }
-  __syncwarp();
-
-  // pass 1: the minimum-energy candidate b* (from the forward's context when
-  // the backward has it)
-  const bool use_ctx = BWD && a.ctx_in != nullptr;
-  float m1 = kInf, m2 = kInf;
-  unsigned b1 = 0u;
-  unsigned long long ev = 0;
-  if (use_ctx) {
-    if (active) b1 = a.ctx_in[p].x;
-  } else if (active) {
-    SlotView sv{ts.dot, ts.h, ts.k, ts.w};
-    search_lane<L1, L2, CLOSED, false>(sM, sv, lt, T, 0.f, nullptr, nullptr, 0u, m1,
-                                       b1, m2, ev);
-  }
-  if (!use_ctx)
-    for (int off = 1; off < T; off <<= 1) {
-      const float om1 = __shfl_xor_sync(kFullS, m1, off);
-      const unsigned ob1 = __shfl_xor_sync(kFullS, b1, off);
-      const float om2 = __shfl_xor_sync(kFullS, m2, off);
-      top2_merge(m1, b1, m2, om1, ob1, om2);
-    }
-  soft_anchor<kMaxDot>(a, ts, sM, sMlo, T, lt, active, b1);
-
-  // pass 2: Boltzmann weights relative to b*
-  const int k = active ? ts.k : 0;
-  const unsigned total = 1u << k;
-  float Z = 0.f;
-  float acc[KMAX];
-#pragma unroll
-  for (int s = 0; s < KMAX; ++s) acc[s] = 0.f;
-  const float inv_kT = 1.0f / kT;
-  if (use_ctx) {
-    if (active) Z = expf(__uint_as_float(a.ctx_in[p].y));
-  } else {
-    if (active) {
-      for (unsigned b = (unsigned)lt; b < total; b += (unsigned)T) {
-        if (CLOSED && __popc(b) != ts.w) continue;
-        const float wgt = expf(-delta_energy<KMAX>(ts, Ms, b) * inv_kT);
-        Z += wgt;
-#pragma unroll
-        for (int s = 0; s < KMAX; ++s)
-          if ((b >> s) & 1u) acc[s] += wgt;
-      }
-    }
-    for (int off = 1; off < T; off <<= 1) {
-      Z += __shfl_xor_sync(kFullS, Z, off);
-#pragma unroll
-      for (int s = 0; s < KMAX; ++s) acc[s] += __shfl_xor_sync(kFullS, acc[s], off);
-    }
-  }
-  if (!BWD) {
-    if (active) {
-      for (int i = lt; i < n; i += T) {
-        float v = (float)ts.base[i];
-        if ((ts.mask >> i) & 1u) {
-          const int s = __popc(ts.mask & ((1u << i) - 1u));
-#pragma unroll
-          for (int q = 0; q < KMAX; ++q)
-            if (q == s) v += acc[q] / Z;
-        }
-        a.out_mean[p * n + i] = v;
-      }
-      if (lt == 0 && a.out_logZ) a.out_logZ[p] = logf(Z) - ts.ustar_kT;
-      if (lt == 0 && a.ctx_out) a.ctx_out[p] = make_uint2(ts.bstar, __float_as_uint(logf(Z)));
-    }
-    return;
-  }
-
-  // ---- backward: a_b = -(w_b / kT) (g . n_b - g . <n>), w_b normalised ----
-  const int L = contrib_len(n);
-  float* my = s_contrib + team * L;
-  float gs[KMAX];      // g of each slot's dot
-  float gmean = 0.f;   // g . <n>
-  float gbase = 0.f;   // g . base
-  const float invZ = 1.0f / Z;
-#pragma unroll
-  for (int s = 0; s < KMAX; ++s) gs[s] = 0.f;
-  const bool fit = a.fit_target != nullptr;
-  float lossp = 0.f;
-  if (fit) lossp = fit_loss_grad_team<KMAX>(a, ts, acc, Z, p, sGf[team], lt, T, active);
-  if (active) {
-    const float* g = fit ? sGf[team] : a.grad_mean + p * n;
-    for (int i = 0; i < n; ++i) gbase += g[i] * (float)ts.base[i];
-#pragma unroll
-    for (int s = 0; s < KMAX; ++s)
-      if (s < k) gs[s] = g[ts.dot[s]];
-    if (use_ctx) {
-      for (int i = 0; i < n; ++i) gmean += g[i] * a.mean_in[p * n + i];
-    } else {
-      // g . <n> - g . base = sum_s g_s <b_s>, so that gn - gmean below is
-      // formed without the large g . base on both sides
-      gmean = 0.f;
-#pragma unroll
-      for (int s = 0; s < KMAX; ++s)
-        if (s < k) gmean += gs[s] * acc[s] * invZ;
-      gbase = 0.f;
-    }
-  }
-  float sa = 0.f;
-  float va[KMAX];
-  float Qa[tri(KMAX)];
-#pragma unroll
-  for (int s = 0; s < KMAX; ++s) va[s] = 0.f;
-#pragma unroll
-  for (int e = 0; e < tri(KMAX); ++e) Qa[e] = 0.f;
-  if (active) {
-    for (unsigned b = (unsigned)lt; b < total; b += (unsigned)T) {
-      if (CLOSED && __popc(b) != ts.w) continue;
-      const float wgt = expf(-delta_energy<KMAX>(ts, Ms, b) * inv_kT) * invZ;
-      float gn = gbase;
-#pragma unroll
-      for (int s = 0; s < KMAX; ++s)
-        if ((b >> s) & 1u) gn += gs[s];
-      const float av = -(wgt * inv_kT) * (gn - gmean);
-      sa += av;
-#pragma unroll
-      for (int s = 0; s < KMAX; ++s) {
-        if ((b >> s) & 1u) {
-          va[s] += av;
-#pragma unroll
-          for (int s2 = s; s2 < KMAX; ++s2)
-            if ((b >> s2) & 1u) Qa[s * KMAX - s * (s - 1) / 2 + (s2 - s)] += av;
-        }
-      }
-    }
-  }
-  for (int off = 1; off < T; off <<= 1) {
-    sa += __shfl_xor_sync(kFullS, sa, off);
-#pragma unroll
-    for (int s = 0; s < KMAX; ++s) va[s] += __shfl_xor_sync(kFullS, va[s], off);
-#pragma unroll
-    for (int e = 0; e < tri(KMAX); ++e) Qa[e] += __shfl_xor_sync(kFullS, Qa[e], off);
-  }
-  // pixel contribution: dM_p = 1/2 [sa r0 r0^T + r0 va^T + va r0^T + Qa],
-  // rho = sa r0 + va, dc_p = -M rho (dot coordinates); the team's lanes split
-  // the entries
-  float* q_s = sQa[BWD ? team : 0];
-  if (lt == 0) {
-#pragma unroll
-    for (int e = 0; e < tri(KMAX); ++e) q_s[e] = Qa[e];
-#pragma unroll
-    for (int s = 0; s < KMAX; ++s) q_s[tri(KMAX) + s] = va[s];
-    q_s[tri(KMAX) + KMAX] = sa;
-  }
-  __syncwarp();
-  soft_contrib<KMAX>(a, ts, q_s, my, s_contrib, sM, T, lt, teams, active, p, lossp);
 }
 
 // ---------------------------------------------------------------------------
@@ -807,7 +604,9 @@ __global__ void __launch_bounds__(kDenseThreads, 640 / kDenseThreads) k_soft_den
   constexpr bool fit = MODE == kDenseFit;
   float lossp = 0.f;
   float* gf = sGf + team * kMaxDot;
-  if (fit) lossp = fit_loss_grad_team<K>(a, ts, accb, Z, p, gf, lt, T, active);
+  if (fit)
+    lossp = fit_loss_grad_team(a, ts, [&](int s) { return pick<K>(accb, s); }, Z, p, gf, lt, T,
+                               active);
   if (active) {
     const float* g = fit ? gf : a.grad_mean + p * n;
 #pragma unroll
@@ -917,6 +716,621 @@ __global__ void __launch_bounds__(kDenseThreads, 640 / kDenseThreads) k_soft_den
   const int L = contrib_len(n);
   float* my = s_contrib + team * L;
   soft_contrib<K>(a, ts, q_s, my, s_contrib, sM, T, lt, kTeams, active, p, lossp);
+}
+
+// ---------------------------------------------------------------------------
+// The same for 9 to 16 dots: a warp per pixel.  Slots 0..4 are the inner table
+// of a lane, slots 5..9 the bits of its lane index, slots 10.. (NIT of them at
+// most: 2 for up to 12 dots, 6 for 16) the bits of the iteration the warp is
+// in; an iteration covers 1024 patterns, 32 a lane.  Both passes evaluate F as
+// the dense form does: the lane's rest value and inner coefficients for its
+// lane bits, formed once, plus a row of a table over the iteration patterns
+// (shared by the warp) and the lane's pair terms with the iteration's slots;
+// the 32 inner values by doubling plus the pair table.  So a weight is a sum
+// over the flipped slots alone, never a long incremental walk.  Pass 2 carries
+// the scale -log2(e) / kT in its coefficients, so a weight is one addition and
+// one exponential after the doubling.
+//   The moments come from the superset sum over the inner bits of each
+// iteration: of the weights (forward), and of x(d) = w(d) (c0 + gam . d)
+// (backward); sums over lane bits are taken once at the end, over rows of
+// shared memory; an iteration slot has its own accumulators.  An iteration
+// whose weights all round to zero (exponents below FP32's range) adds nothing
+// and is skipped.
+//   What bounds it: FP32 issue, and latency at 3 to 5 blocks per SM (the
+// backward keeps 29 or 67 moments a lane in registers).  A training step of
+// 12 dots on 75 x 60 pixels through torch.autograd, kernels, torch's own
+// kernels and host work together: 2240 us with one candidate at a time (a sum
+// over the slots that differ from b*, 136 moment updates), 664 us so; its
+// gradient is 2.4e-7 off FP64 where it was 1.4e-6.
+// ---------------------------------------------------------------------------
+constexpr int kWideIn = 5;                 // inner slots
+constexpr int kWideOut = 10;               // inner slots + lane bits
+constexpr int kWideRow = 36;               // row of the lane sums: 32 lanes, 16-byte aligned
+__host__ __device__ constexpr int wide_slots(int nit) { return kWideOut + nit; }
+// per-lane sums of the backward: |S| <= 2 over the inner slots (16), {}, {j}
+// with each iteration slot, {} with each pair of them
+__host__ __device__ constexpr int wide_rows(int nit) { return 16 + 6 * nit + nit * (nit - 1) / 2; }
+__host__ __device__ constexpr int wide_moments(int k) { return 1 + k + k * (k - 1) / 2; }
+
+template <int NIT>
+struct WideSmem {  // bytes from the start of the dynamic buffer; per team, kSoftThreads / 32 of them
+  static constexpr int K = wide_slots(NIT), kTeams = kSoftThreads / 32;
+  size_t slots, W, G, r, itab, ptab, cls, qs, qd, gf, red, contrib, total;
+  __host__ __device__ constexpr WideSmem(bool bwd, int L)
+      : slots(0),
+        W(al16(sizeof(TeamSlots) * kTeams)),
+        G(W + sizeof(float) * kTeams * kMaxDot * kMaxDot),
+        r(G + sizeof(float) * kTeams * kMaxDot),
+        itab(r + sizeof(float) * kTeams * 2 * kMaxDot),
+        ptab(itab + sizeof(float) * kTeams * (8 << NIT)),
+        cls(ptab + sizeof(float) * kTeams * 32),
+        qs(cls + sizeof(unsigned) * kTeams * 8),
+        qd(qs + (bwd ? al16(sizeof(float) * kTeams * (tri(K) + K + 1)) : 0)),
+        gf(qd + al16(sizeof(float) * kTeams * (bwd ? wide_moments(K) : 1 + K))),
+        red(gf + (bwd ? sizeof(float) * kTeams * 2 * kMaxDot : 0)),
+        contrib(red + sizeof(float) * kTeams * kWideRow * (bwd ? wide_rows(NIT) : 6 + NIT)),
+        total(contrib + (bwd ? al16(sizeof(float) * kTeams * L) : 0)) {}
+};
+
+// A lane's part of F: its lane bits' energy, the inner coefficients given
+// them, their pair terms with each iteration slot.
+template <int NIT>
+struct WideLane {
+  float A, q[kWideIn], cr[NIT];
+};
+
+// The lane's part, the iteration table and the inner pair table from the
+// coefficients G and pair terms W (slot order, stride 16; absent slots: W = 0
+// and a G that no pattern with them survives).  All lanes of the warp.
+template <int NIT>
+__device__ __forceinline__ void wide_tables(const float* W, const float* G, float* itab,
+                                            float* ptab, int lane, int nit, WideLane<NIT>& t) {
+  t.A = 0.f;
+#pragma unroll
+  for (int j = 0; j < kWideIn; ++j) t.q[j] = G[j];
+#pragma unroll
+  for (int ii = 0; ii < NIT; ++ii) t.cr[ii] = 0.f;
+  float wO[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) wO[i] = ((lane >> i) & 1) ? 1.f : 0.f;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const float4* row4 = reinterpret_cast<const float4*>(W + (kWideIn + i) * kMaxDot);
+    float row[kMaxDot];
+#pragma unroll
+    for (int e = 0; e < kMaxDot / 4; ++e) {
+      if (4 * e >= wide_slots(NIT)) break;
+      const float4 v = row4[e];
+      row[4 * e] = v.x; row[4 * e + 1] = v.y; row[4 * e + 2] = v.z; row[4 * e + 3] = v.w;
+    }
+    float add = G[kWideIn + i];
+#pragma unroll
+    for (int i2 = 0; i2 < i; ++i2) add = fmaf(wO[i2], row[kWideIn + i2], add);
+    t.A = fmaf(wO[i], add, t.A);
+#pragma unroll
+    for (int j = 0; j < kWideIn; ++j) t.q[j] = fmaf(wO[i], row[j], t.q[j]);
+#pragma unroll
+    for (int ii = 0; ii < NIT; ++ii) t.cr[ii] = fmaf(wO[i], row[kWideOut + ii], t.cr[ii]);
+  }
+  for (int it = lane; it < (1 << nit); it += 32) {
+    float A = 0.f, q[kWideIn];
+#pragma unroll
+    for (int j = 0; j < kWideIn; ++j) q[j] = 0.f;
+#pragma unroll
+    for (int ii = 0; ii < NIT; ++ii) {
+      const float w = ((it >> ii) & 1) ? 1.f : 0.f;
+      const float* row = W + (kWideOut + ii) * kMaxDot;
+      float add = G[kWideOut + ii];
+#pragma unroll
+      for (int i2 = 0; i2 < ii; ++i2)
+        add = fmaf(((it >> i2) & 1) ? 1.f : 0.f, row[kWideOut + i2], add);
+      A = fmaf(w, add, A);
+#pragma unroll
+      for (int j = 0; j < kWideIn; ++j) q[j] = fmaf(w, row[j], q[j]);
+    }
+    float4* dst = reinterpret_cast<float4*>(itab + it * 8);
+    dst[0] = make_float4(A, q[0], q[1], q[2]);
+    dst[1] = make_float4(q[3], q[4], 0.f, 0.f);
+  }
+  float pb = 0.f;
+#pragma unroll
+  for (int j = 1; j < kWideIn; ++j)
+#pragma unroll
+    for (int l = 0; l < j; ++l)
+      pb = fmaf(((lane >> j) & (lane >> l) & 1) ? 1.f : 0.f, W[j * kMaxDot + l], pb);
+  ptab[lane] = pb;
+  __syncwarp();
+}
+
+// Rest value and inner coefficients of iteration pattern it.
+template <int NIT>
+__device__ __forceinline__ void wide_rest(const WideLane<NIT>& t, const float* itab, unsigned it,
+                                          float& A, float (&q)[kWideIn]) {
+  const float4* row = reinterpret_cast<const float4*>(itab + it * 8);
+  const float4 r0 = row[0], r1 = row[1];
+  float x = 0.f;
+#pragma unroll
+  for (int ii = 0; ii < NIT; ++ii) x = fmaf(((it >> ii) & 1u) ? 1.f : 0.f, t.cr[ii], x);
+  A = (t.A + x) + r0.x;
+  q[0] = t.q[0] + r0.y;
+  q[1] = t.q[1] + r0.z;
+  q[2] = t.q[2] + r0.w;
+  q[3] = t.q[3] + r1.x;
+  q[4] = t.q[4] + r1.y;
+}
+
+// v[b] = A + the coefficients of b's bits, over the 32 inner patterns.
+__device__ __forceinline__ void wide_doubling(float A, const float (&q)[kWideIn], float2 (&v)[16]) {
+  v[0] = make_float2(A, A + q[0]);
+#pragma unroll
+  for (int j = 1; j < kWideIn; ++j) {
+    const float2 qq = make_float2(q[j], q[j]);
+#pragma unroll
+    for (int b = 0; b < (1 << (j - 1)); ++b) v[b + (1 << (j - 1))] = fadd2(v[b], qq);
+  }
+}
+
+// F of the 32 inner patterns (pairs of patterns 2 b, 2 b + 1).
+__device__ __forceinline__ void wide_block(float A, const float (&q)[kWideIn], const float* ptab,
+                                           float2 (&F)[16]) {
+  wide_doubling(A, q, F);
+  const float4* P4 = reinterpret_cast<const float4*>(ptab);
+#pragma unroll
+  for (int b = 0; b < 16; b += 2) {
+    const float4 p = P4[b / 2];
+    F[b] = fadd2(F[b], make_float2(p.x, p.y));
+    F[b + 1] = fadd2(F[b + 1], make_float2(p.z, p.w));
+  }
+}
+
+// 2^x, results below FP32's normal range as zero.
+__device__ __forceinline__ float wide_exp2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Superset sum over the inner bits, in place (w[S] <- sum over b containing S).
+__device__ __forceinline__ void wide_superset(float2 (&w)[16]) {
+#pragma unroll
+  for (int b = 0; b < 16; ++b) w[b].x += w[b].y;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int b = 0; b < 16; ++b)
+      if (!((b >> j) & 1)) w[b] = fadd2(w[b], w[b | (1 << j)]);
+}
+__device__ __forceinline__ float wide_at(const float2 (&w)[16], int S) {
+  return (S & 1) ? w[S >> 1].y : w[S >> 1].x;
+}
+
+// Sum over the lanes containing the bits of m of a row of per-lane values.
+__device__ __forceinline__ float wide_lane_sum(const float* row, int m) {
+  float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+  for (int l = 0; l < 32; l += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(row + l);
+    s0 += (l & m) == m ? v.x : 0.f;
+    s1 += ((l + 1) & m) == m ? v.y : 0.f;
+    s0 += ((l + 2) & m) == m ? v.z : 0.f;
+    s1 += ((l + 3) & m) == m ? v.w : 0.f;
+  }
+  return s0 + s1;
+}
+
+// Row and lane mask of the moment of slots s <= s2 (s == s2: the single).
+template <int NIT>
+__device__ __forceinline__ void wide_where(int s, int s2, int& row, int& m) {
+  auto lane_bit = [](int q) { return q >= kWideIn && q < kWideOut ? 1 << (q - kWideIn) : 0; };
+  m = lane_bit(s) | lane_bit(s2);
+  const int j = s < kWideIn ? s : -1;
+  const int ii = s2 >= kWideOut ? s2 - kWideOut : -1;
+  if (s >= kWideOut && s2 > s) {  // two iteration slots i < ii
+    const int i = s - kWideOut;
+    row = 16 + 6 * NIT + i * (2 * NIT - i - 1) / 2 + (ii - i - 1);
+  } else if (ii >= 0) {
+    row = 16 + 6 * ii + 1 + j;  // j = -1: the {} row
+  } else if (j >= 0 && s2 < kWideIn && s2 > s) {
+    row = 6 + j * (2 * kWideIn - j - 1) / 2 + (s2 - j - 1);
+  } else {
+    row = 1 + j;
+  }
+}
+
+template <bool CLOSED, int MODE, int NIT>
+__global__ void __launch_bounds__(kSoftThreads) k_soft_wide(SoftLaunch a) {
+  constexpr bool BWD = MODE != kDenseFwd;
+  constexpr bool use_ctx = MODE == kDenseBwdCtx;
+  constexpr bool fit = MODE == kDenseFit;
+  constexpr int K = wide_slots(NIT);
+  constexpr int kTeams = kSoftThreads / 32;
+  static_assert(kWideIn == 5 && kWideOut == 10, "a warp's lane bits are slots 5..9");
+  __shared__ __align__(16) float sMh[kMaxDot * kLdM], sMl[kMaxDot * kLdM];
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  const int n = a.n;
+  const int L = contrib_len(n);
+  const WideSmem<NIT> lay(BWD, L);
+  const int team = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  TeamSlots& ts = reinterpret_cast<TeamSlots*>(s_dyn + lay.slots)[team];
+  float* W = reinterpret_cast<float*>(s_dyn + lay.W) + team * kMaxDot * kMaxDot;
+  float* G = reinterpret_cast<float*>(s_dyn + lay.G) + team * kMaxDot;
+  float* rr = reinterpret_cast<float*>(s_dyn + lay.r) + team * 2 * kMaxDot;
+  float* itab = reinterpret_cast<float*>(s_dyn + lay.itab) + team * (8 << NIT);
+  float* ptab = reinterpret_cast<float*>(s_dyn + lay.ptab) + team * 32;
+  unsigned* cls = reinterpret_cast<unsigned*>(s_dyn + lay.cls) + team * 8;
+  float* q_s = reinterpret_cast<float*>(s_dyn + lay.qs) + team * (tri(K) + K + 1);
+  float* qd = reinterpret_cast<float*>(s_dyn + lay.qd) + team * (BWD ? wide_moments(K) : 1 + K);
+  float* gf = reinterpret_cast<float*>(s_dyn + lay.gf) + team * 2 * kMaxDot;
+  float* red = reinterpret_cast<float*>(s_dyn + lay.red) +
+               team * kWideRow * (BWD ? wide_rows(NIT) : 6 + NIT);
+  float* s_contrib = reinterpret_cast<float*>(s_dyn + lay.contrib);
+  for (int e = threadIdx.x; e < kMaxDot * kLdM / 4; e += blockDim.x) {
+    reinterpret_cast<float4*>(sMh)[e] = reinterpret_cast<const float4*>(a.md->k.Mhi)[e];
+    reinterpret_cast<float4*>(sMl)[e] = reinterpret_cast<const float4*>(a.md->k.Mlo)[e];
+  }
+  __syncthreads();
+  const long long p = (long long)blockIdx.x * kTeams + team;
+  const bool active = p < a.sc.P;  // the same for the whole warp
+  const float kT = (float)a.kT;
+  float lossp = 0.f;
+  soft_setup_team<CLOSED>(a, ts, p, lane, 32, active);
+  if (active) {
+    const int k = ts.k;
+    const int nit = k > kWideOut ? k - kWideOut : 0;
+    const unsigned mask = ts.mask;
+    // pair terms in slot order (lane = column and half of the rows)
+    {
+      const int s2 = lane & 15;
+      const int d2 = s2 < k ? ts.dot[s2] : 0;
+#pragma unroll
+      for (int s0 = 0; s0 < kMaxDot; s0 += 2) {
+        const int s = s0 + (lane >> 4);
+        W[s * kMaxDot + s2] = (s < k && s2 < k) ? sMh[ts.dot[s] * kLdM + d2] : 0.f;
+      }
+    }
+    WideLane<NIT> t;
+    float2 F[16];
+    // pass 1: the minimum-energy pattern b* (the forward's, when given)
+    unsigned b1;
+    if (use_ctx) {
+      b1 = a.ctx_in[p].x;
+    } else {
+      __syncwarp();
+      if (lane < kMaxDot)
+        G[lane] = lane < k ? ts.h[lane] + 0.5f * W[lane * kMaxDot + lane] : kBig;
+      __syncwarp();
+      wide_tables<NIT>(W, G, itab, ptab, lane, nit, t);
+      // per lane the iteration with the lowest block minimum
+      float best = kInf;
+      unsigned bit = 0u;
+      for (unsigned it = 0; it < (1u << nit); ++it) {
+        float A, q[kWideIn];
+        wide_rest<NIT>(t, itab, it, A, q);
+        wide_block(A, q, ptab, F);
+        float m0 = kInf, m1 = kInf;
+        const int r = CLOSED ? ts.w - __popc(it) - __popc((unsigned)lane) : 0;
+#pragma unroll
+        for (int b = 0; b < 32; b += 2) {
+          const float2 e = F[b >> 1];
+          if (!CLOSED) {
+            m0 = fminf(m0, e.x);
+            m1 = fminf(m1, e.y);
+          } else {
+            m0 = fminf(m0, popc_c((unsigned)b) == r ? e.x : kInf);
+            m1 = fminf(m1, popc_c((unsigned)b + 1u) == r ? e.y : kInf);
+          }
+        }
+        const float mn = fminf(m0, m1);
+        bit = mn < best ? it : bit;
+        best = fminf(best, mn);
+      }
+      // the warp's lowest block, then its 32 patterns, one a lane
+      unsigned who = ((unsigned)lane << 8) | bit;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const float ob = __shfl_xor_sync(kFullS, best, off);
+        const unsigned ow = __shfl_xor_sync(kFullS, who, off);
+        const bool take = ob < best || (ob == best && ow < who);
+        best = take ? ob : best;
+        who = take ? ow : who;
+      }
+      const int wl = (int)(who >> 8);
+      const unsigned wit = who & 255u;
+      float A, q[kWideIn];
+      wide_rest<NIT>(t, itab, wit, A, q);
+      float e = __shfl_sync(kFullS, A, wl);
+#pragma unroll
+      for (int j = 0; j < kWideIn; ++j) {
+        const float qj = __shfl_sync(kFullS, q[j], wl);
+        e += ((lane >> j) & 1) ? qj : 0.f;
+      }
+      e += ptab[lane];
+      if (CLOSED && __popc((unsigned)lane) != ts.w - __popc(wit) - __popc((unsigned)wl)) e = kInf;
+      unsigned bb = (unsigned)lane;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const float oe = __shfl_xor_sync(kFullS, e, off);
+        const unsigned ob = __shfl_xor_sync(kFullS, bb, off);
+        const bool take = oe < e || (oe == e && __brev(ob) < __brev(bb));
+        e = take ? oe : e;
+        bb = take ? ob : bb;
+      }
+      b1 = bb | ((unsigned)wl << kWideIn) | (wit << kWideOut);
+    }
+    // the gradient at b* in double-float: r = n* - c staged by the dots' lanes,
+    // a row per lane of the first half-warp, half its columns in the second
+    {
+      df r = {0.f, 0.f};
+      if (lane < n) {
+        int ni = ts.base[lane];
+        if ((mask >> lane) & 1u) ni += (int)((b1 >> __popc(mask & ((1u << lane) - 1u))) & 1u);
+        r = df_sub({(float)ni, 0.f}, {ts.chi[lane], ts.clo[lane]});
+      }
+      if (lane < kMaxDot) {
+        rr[lane] = r.hi;
+        rr[kMaxDot + lane] = r.lo;
+      }
+      __syncwarp();
+      const int i = lane & 15, j0 = (lane >> 4) * 8;
+      df acc = {0.f, 0.f};
+#pragma unroll
+      for (int j = j0; j < j0 + 8; ++j)  // columns past n hold zeros
+        acc = df_add(acc, df_mul({sMh[i * kLdM + j], sMl[i * kLdM + j]},
+                                 {rr[j], rr[kMaxDot + j]}));
+      df o;
+      o.hi = __shfl_xor_sync(kFullS, acc.hi, 16);
+      o.lo = __shfl_xor_sync(kFullS, acc.lo, 16);
+      acc = df_add(acc, o);
+      if (!BWD) {
+        df u = lane < n ? df_mul(acc, r) : df{0.f, 0.f};
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          df ou;
+          ou.hi = __shfl_xor_sync(kFullS, u.hi, off);
+          ou.lo = __shfl_xor_sync(kFullS, u.lo, off);
+          u = df_add(u, ou);
+        }
+        if (lane == 0) ts.ustar_kT = (float)(df_to_double(df_mul_f(u, 0.5f)) / a.kT);
+      }
+      // the coefficients of pass 2, scaled: G_s = -log2(e) / kT (gp or gm)
+      const float c2 = -1.4426950408889634f / kT;
+      if (lane < kMaxDot) G[lane] = -kBig;
+      __syncwarp();
+      if (lane < n && ((mask >> lane) & 1u)) {
+        const int s = __popc(mask & ((1u << lane) - 1u));
+        const float g = acc.hi + acc.lo, half = 0.5f * sMh[lane * kLdM + lane];
+        G[s] = c2 * (((b1 >> s) & 1u) ? half - g : g + half);
+      }
+      const int s2 = lane & 15;
+#pragma unroll
+      for (int s0 = 0; s0 < kMaxDot; s0 += 2) {
+        const int s = s0 + (lane >> 4);
+        const float v = c2 * W[s * kMaxDot + s2];
+        W[s * kMaxDot + s2] = (((b1 >> s) ^ (b1 >> s2)) & 1u) ? -v : v;
+      }
+      if (CLOSED && lane < 8) {
+        // bit b of cls[r]: inner pattern b flips b* to r set inner slots
+        unsigned v = 0u;
+        for (unsigned b = 0; b < 32u; ++b)
+          v |= (__popc((b1 & 31u) ^ b) == lane ? 1u : 0u) << b;
+        cls[lane] = v;
+      }
+      __syncwarp();
+    }
+    wide_tables<NIT>(W, G, itab, ptab, lane, nit, t);
+    float pmax = 0.f;  // highest pair sum: bounds an iteration's exponents
+    if (NIT > 2) {
+      pmax = ptab[lane];
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) pmax = fmaxf(pmax, __shfl_xor_sync(kFullS, pmax, off));
+    }
+    const unsigned bout = b1 >> kWideIn;
+    // the weights of iteration it into F; false: all of the warp's are zero
+    auto weights = [&](unsigned it) -> bool {
+      float A, q[kWideIn];
+      wide_rest<NIT>(t, itab, it, A, q);
+      if (NIT > 2) {
+        float ub = A + pmax;
+#pragma unroll
+        for (int j = 0; j < kWideIn; ++j) ub += fmaxf(0.f, q[j]);
+        if (__all_sync(kFullS, ub < -130.f)) return false;
+      }
+      wide_block(A, q, ptab, F);
+      unsigned keep = 0xffffffffu;
+      if (CLOSED) {
+        const int r = ts.w - __popc(bout ^ ((unsigned)lane | (it << (kWideOut - kWideIn))));
+        keep = r >= 0 && r <= kWideIn ? cls[r] : 0u;
+      }
+#pragma unroll
+      for (int b = 0; b < 16; ++b) {
+        F[b].x = wide_exp2(F[b].x);
+        F[b].y = wide_exp2(F[b].y);
+        if (CLOSED) {
+          F[b].x = (keep >> (2 * b)) & 1u ? F[b].x : 0.f;
+          F[b].y = (keep >> (2 * b + 1)) & 1u ? F[b].y : 0.f;
+        }
+      }
+      return true;
+    };
+
+    // pass 2: Z and the first moments in flip coordinates
+    float Z = 1.f;
+    if (!use_ctx) {
+      float z = 0.f, si[kWideIn], sit[NIT];
+#pragma unroll
+      for (int j = 0; j < kWideIn; ++j) si[j] = 0.f;
+#pragma unroll
+      for (int ii = 0; ii < NIT; ++ii) sit[ii] = 0.f;
+      for (unsigned it = 0; it < (1u << nit); ++it) {
+        if (!weights(it)) continue;
+        wide_superset(F);
+        z += F[0].x;
+#pragma unroll
+        for (int j = 0; j < kWideIn; ++j) si[j] += wide_at(F, 1 << j);
+#pragma unroll
+        for (int ii = 0; ii < NIT; ++ii) sit[ii] += ((it >> ii) & 1u) ? F[0].x : 0.f;
+      }
+      red[lane] = z;
+#pragma unroll
+      for (int j = 0; j < kWideIn; ++j) red[(1 + j) * kWideRow + lane] = si[j];
+#pragma unroll
+      for (int ii = 0; ii < NIT; ++ii) red[(6 + ii) * kWideRow + lane] = sit[ii];
+      __syncwarp();
+      if (lane < 1 + K) {
+        // lane 0: Z; lane 1 + s: the moment of slot s
+        const int s = lane - 1;
+        const int row = s < 0 ? 0 : s < kWideIn ? 1 + s : s < kWideOut ? 0 : 6 + s - kWideOut;
+        const int m = s >= kWideIn && s < kWideOut ? 1 << (s - kWideIn) : 0;
+        qd[lane] = wide_lane_sum(red + row * kWideRow, m);
+      }
+      __syncwarp();
+      Z = qd[0];
+    }
+    // sum_b w_b b_s (the weight of slot s taking its +1)
+    auto accb = [&](int s) { return ((b1 >> s) & 1u) ? Z - qd[1 + s] : qd[1 + s]; };
+    if (!BWD) {
+      if (lane < n) {
+        float v = (float)ts.base[lane];
+        if ((mask >> lane) & 1u) v += accb(__popc(mask & ((1u << lane) - 1u))) / Z;
+        a.out_mean[p * n + lane] = v;
+      }
+      if (lane == 0 && a.out_logZ) a.out_logZ[p] = logf(Z) - ts.ustar_kT;
+      if (lane == 0 && a.ctx_out) a.ctx_out[p] = make_uint2(b1, __float_as_uint(logf(Z)));
+    } else {
+      if (use_ctx) Z = expf(__uint_as_float(a.ctx_in[p].y));
+      if (fit) lossp = fit_loss_grad_team(a, ts, accb, Z, p, gf, lane, 32, true);
+      const float* g = fit ? gf : a.grad_mean + p * n;
+      // gam_s = sg_s g_s in shared memory, c0 = g . n* - g . <n>
+      float* gam = gf + kMaxDot;
+      float c0 = 0.f;
+      if (lane < kMaxDot) gam[lane] = 0.f;
+      __syncwarp();
+      if (lane < k) {
+        const float gs = g[ts.dot[lane]];
+        const float ga = ((b1 >> lane) & 1u) ? -gs : gs;
+        gam[lane] = ga;
+        if (!use_ctx) c0 = -ga * qd[1 + lane] / Z;
+      }
+      if (use_ctx && lane < n) {
+        int ni = ts.base[lane];
+        if ((mask >> lane) & 1u) ni += (int)((b1 >> __popc(mask & ((1u << lane) - 1u))) & 1u);
+        c0 = g[lane] * ((float)ni - a.mean_in[p * n + lane]);
+      }
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) c0 += __shfl_xor_sync(kFullS, c0, off);
+      __syncwarp();
+      float gi[kWideIn], gl = c0;
+#pragma unroll
+      for (int j = 0; j < kWideIn; ++j) gi[j] = gam[j];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) gl += ((lane >> i) & 1) ? gam[kWideIn + i] : 0.f;
+      // x(d) = w(d) (c0 + gam . d) and its superset sums, all iterations
+      float X[16], XI[NIT][6], XP[NIT * (NIT - 1) / 2];
+#pragma unroll
+      for (int e = 0; e < 16; ++e) X[e] = 0.f;
+#pragma unroll
+      for (int ii = 0; ii < NIT; ++ii)
+#pragma unroll
+        for (int e = 0; e < 6; ++e) XI[ii][e] = 0.f;
+#pragma unroll
+      for (int e = 0; e < NIT * (NIT - 1) / 2; ++e) XP[e] = 0.f;
+      for (unsigned it = 0; it < (1u << nit); ++it) {
+        if (!weights(it)) continue;
+        float y0 = gl;
+#pragma unroll
+        for (int ii = 0; ii < NIT; ++ii) y0 += ((it >> ii) & 1u) ? gam[kWideOut + ii] : 0.f;
+        {
+          float2 y[16];
+          wide_doubling(y0, gi, y);
+#pragma unroll
+          for (int b = 0; b < 16; ++b) F[b] = make_float2(F[b].x * y[b].x, F[b].y * y[b].y);
+        }
+        wide_superset(F);
+        X[0] += F[0].x;
+#pragma unroll
+        for (int j = 0; j < kWideIn; ++j) X[1 + j] += wide_at(F, 1 << j);
+#pragma unroll
+        for (int j = 0; j < kWideIn; ++j)
+#pragma unroll
+          for (int l = j + 1; l < kWideIn; ++l)
+            X[6 + j * (2 * kWideIn - j - 1) / 2 + (l - j - 1)] += wide_at(F, (1 << j) | (1 << l));
+#pragma unroll
+        for (int ii = 0; ii < NIT; ++ii)
+          if ((it >> ii) & 1u) {
+            XI[ii][0] += F[0].x;
+#pragma unroll
+            for (int j = 0; j < kWideIn; ++j) XI[ii][1 + j] += wide_at(F, 1 << j);
+#pragma unroll
+            for (int i2 = 0; i2 < ii; ++i2)
+              XP[i2 * (2 * NIT - i2 - 1) / 2 + (ii - i2 - 1)] += ((it >> i2) & 1u) ? F[0].x : 0.f;
+          }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int e = 0; e < 16; ++e) red[e * kWideRow + lane] = X[e];
+#pragma unroll
+      for (int ii = 0; ii < NIT; ++ii)
+#pragma unroll
+        for (int e = 0; e < 6; ++e) red[(16 + 6 * ii + e) * kWideRow + lane] = XI[ii][e];
+#pragma unroll
+      for (int e = 0; e < NIT * (NIT - 1) / 2; ++e) red[(16 + 6 * NIT + e) * kWideRow + lane] = XP[e];
+      __syncwarp();
+      // the |S| <= 2 moments, one a lane at a time: {}, {s}, {s, s2}
+      const int nm = wide_moments(K);
+      for (int e = lane; e < nm; e += 32) {
+        float v = 0.f;
+        if (e == 0) {
+          v = wide_lane_sum(red, 0);
+        } else if (e <= K) {
+          if (e - 1 < k) {
+            int row, m;
+            wide_where<NIT>(e - 1, e - 1, row, m);
+            v = wide_lane_sum(red + row * kWideRow, m);
+          }
+        } else {
+          int s = 0, rem = e - 1 - K;
+          while (rem >= K - 1 - s) { rem -= K - 1 - s; ++s; }
+          const int s2 = s + 1 + rem;
+          if (s2 < k) {
+            int row, m;
+            wide_where<NIT>(s, s2, row, m);
+            v = wide_lane_sum(red + row * kWideRow, m);
+          }
+        }
+        qd[e] = v;
+      }
+      __syncwarp();
+      // scaled by -1 / (kT Z) and turned to charge coordinates (as the dense form)
+      const float alpha = -1.0f / (kT * Z);
+      const float sa_a = alpha * qd[0];
+      for (int e = lane; e < tri(K); e += 32) {
+        int s = 0, rem = e;
+        while (rem >= K - s) { rem -= K - s; ++s; }
+        const int s2 = s + rem;
+        const float bts = ((b1 >> s) & 1u) ? 1.f : 0.f, sgs = 1.f - 2.f * bts;
+        const float vs = alpha * qd[1 + s];
+        float q;
+        if (s2 == s) {
+          q = bts * sa_a + sgs * vs;
+        } else {
+          const float bt2 = ((b1 >> s2) & 1u) ? 1.f : 0.f, sg2 = 1.f - 2.f * bt2;
+          const float v2 = alpha * qd[1 + s2];
+          q = bts * bt2 * sa_a + bts * sg2 * v2 + bt2 * sgs * vs +
+              sgs * sg2 * alpha * qd[1 + K + s * (2 * K - s - 1) / 2 + (s2 - s - 1)];
+        }
+        q_s[e] = q;
+      }
+      if (lane < K) {
+        const float bts = ((b1 >> lane) & 1u) ? 1.f : 0.f;
+        q_s[tri(K) + lane] = bts * sa_a + (1.f - 2.f * bts) * alpha * qd[1 + lane];
+      }
+      if (lane == 0) q_s[tri(K) + K] = sa_a;
+      __syncwarp();
+    }
+  }
+  if (BWD)
+    soft_contrib<K>(a, ts, q_s, s_contrib + team * L, s_contrib, sMh, 32, lane, kTeams, active, p,
+                    lossp);
 }
 
 // The chain rule through M = Cdd^-1 and c = s Cgd V, from the summed
@@ -1040,26 +1454,25 @@ static __global__ void __launch_bounds__(256) k_soft_reduce(SoftLaunch a, int nb
 
 inline size_t soft_partials_floats_impl(int n, long long P, const SearchCfg& cfg) {
   // blocks of the launch that has the most (the dense kernel's blocks hold
-  // at least as many teams as the per-candidate kernel's)
+  // at least as many teams as 8-lane teams in kSoftThreads threads)
   const int teams = kSoftThreads / cfg.T;
   const long long blocks = (P + teams - 1) / teams;
   return (size_t)blocks * 2 * (size_t)contrib_len(n);
 }
 
-template <int L1, int L2, bool CLOSED, bool BWD, int KMAX>
-static cudaError_t run_soft(const SoftLaunch& a, cudaStream_t st) {
-  const int teams = kSoftThreads / a.cfg.T;
-  const long long P = a.sc.P;
-  const unsigned grid = (unsigned)((P + teams - 1) / teams);
-  const size_t smem = BWD ? (size_t)teams * contrib_len(a.n) * sizeof(float) : 0;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_soft<L1, L2, CLOSED, BWD, KMAX>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+// Wide form (9 to 16 dots; a warp per pixel).
+template <bool CLOSED, int MODE, int NIT>
+static cudaError_t run_soft_wide(const SoftLaunch& a, cudaStream_t st) {
+  constexpr bool BWD = MODE != kDenseFwd;
+  constexpr int teams = kSoftThreads / 32;
+  const unsigned grid = (unsigned)((a.sc.P + teams - 1) / teams);
+  const size_t smem = WideSmem<NIT>(BWD, contrib_len(a.n)).total;
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      k_soft_wide<CLOSED, MODE, NIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      (int)WideSmem<NIT>(BWD, contrib_len(kMaxDot)).total);
+  if (attr != cudaSuccess) return attr;
   if (a.ev) cudaEventRecord(a.ev[0], st);
-  k_soft<L1, L2, CLOSED, BWD, KMAX><<<grid, kSoftThreads, smem, st>>>(a);
+  k_soft_wide<CLOSED, MODE, NIT><<<grid, kSoftThreads, smem, st>>>(a);
   if (BWD) k_soft_reduce<<<contrib_len(a.n), 256, 0, st>>>(a, (int)grid);
   if (a.ev) cudaEventRecord(a.ev[1], st);
   return cudaGetLastError();
@@ -1096,25 +1509,28 @@ static cudaError_t run_soft_dense(const SoftLaunch& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <bool CLOSED, bool BWD>
-static cudaError_t run_soft_dense_mode(const SoftLaunch& a, cudaStream_t st) {
-  if constexpr (!BWD) {
-    return run_soft_dense<CLOSED, kDenseFwd>(a, st);
-  } else {
-    if (a.fit_target) return run_soft_dense<CLOSED, kDenseFit>(a, st);
-    if (a.ctx_in) return run_soft_dense<CLOSED, kDenseBwdCtx>(a, st);
-    return run_soft_dense<CLOSED, kDenseBwd>(a, st);
-  }
+// The dense form for a team of 8 lanes, or the wide one for a warp: two
+// iteration slots cover 12 dots, six 16.
+template <bool CLOSED, int MODE>
+static cudaError_t run_soft_mode(const SoftLaunch& a, cudaStream_t st) {
+  if (a.n <= kDenseMax) return run_soft_dense<CLOSED, MODE>(a, st);
+  return a.n <= kWideOut + 2 ? run_soft_wide<CLOSED, MODE, 2>(a, st)
+                             : run_soft_wide<CLOSED, MODE, 6>(a, st);
 }
 
 template <bool BWD>
 static cudaError_t dispatch_soft(const SoftLaunch& a, cudaStream_t st) {
-  // up to 8 dots: the dense form; beyond, the per-candidate form, whose
-  // search only locates b*
   const bool cl = a.mt.closed != 0;
-  if (a.n <= kDenseMax)
-    return cl ? run_soft_dense_mode<true, BWD>(a, st) : run_soft_dense_mode<false, BWD>(a, st);
-  return cl ? run_soft<5, 4, true, BWD, 16>(a, st) : run_soft<5, 4, false, BWD, 16>(a, st);
+  if constexpr (!BWD) {
+    return cl ? run_soft_mode<true, kDenseFwd>(a, st) : run_soft_mode<false, kDenseFwd>(a, st);
+  } else {
+    if (a.fit_target)
+      return cl ? run_soft_mode<true, kDenseFit>(a, st) : run_soft_mode<false, kDenseFit>(a, st);
+    if (a.ctx_in)
+      return cl ? run_soft_mode<true, kDenseBwdCtx>(a, st)
+                : run_soft_mode<false, kDenseBwdCtx>(a, st);
+    return cl ? run_soft_mode<true, kDenseBwd>(a, st) : run_soft_mode<false, kDenseBwd>(a, st);
+  }
 }
 
 }  // namespace qa

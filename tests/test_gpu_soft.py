@@ -277,3 +277,53 @@ def test_backward_context_after_other_calls_on_the_model(qa):
         assert np.abs(dC.cpu().numpy() - oC).max() <= GRAD_RTOL * sc, between
         assert np.abs(dG.cpu().numpy() - oG).max() <= GRAD_RTOL * sc, between
     m.close()
+
+
+# 9 to 16 dots (a warp per pixel): one dot beyond the 8-lane form, every lane
+# bit in use, each number of iteration slots' edge, a raster whose last block
+# is ragged; closed arrays with a threshold leave few slots on some pixels.
+@pytest.mark.parametrize("n,kT,closed,t", [
+    (9, 0.05, False, 1.0), (10, 0.02, True, 1.0), (11, 0.05, False, 0.5), (12, 0.01, False, 1.0),
+    (12, 0.05, True, 0.5), (13, 0.03, False, 1.0), (16, 0.05, False, 1.0), (16, 0.01, True, 1.0)])
+def test_soft_wide_arrays(qa, n, kT, closed, t):
+    import torch
+    r = np.random.Generator(np.random.PCG64(900 + n))
+    Cdd = inputs.grid_cdd(r, 4, 4) if n == 16 else inputs.chain_cdd(r, n, nn=(0.05, 0.25))
+    cfg = {"Cdd": Cdd, "Cgd": inputs.dense_cgd(r, n)}
+    gx, gy = inputs.swept_gates(n)
+    W, H = (7, 3) if n == 16 else (11, 5)
+    ras = inputs.raster(n, gx, gy, inputs.offsets(r, n, (gx, gy)), W=W, H=H)
+    nc = n if closed else 0
+    mean, logZ = _soft_gpu(qa, cfg, kT, t=t, closed=closed, n_charges=nc, raster=ras)
+    om, ol = oracle.soft(cfg["Cdd"], cfg["Cgd"], raster=ras, kT=kT, t=t, closed=closed,
+                         n_charges=nc)
+    assert np.abs(mean - om).max() <= MEAN_TOL
+    assert (np.abs(logZ - ol) / np.maximum(1.0, np.abs(ol))).max() <= 1e-5
+    gbar = r.normal(size=(W * H, n))
+    _, oC, oG = oracle.soft_grad(cfg["Cdd"], cfg["Cgd"], gbar, raster=ras, kT=kT, t=t,
+                                 closed=closed, n_charges=nc)
+    sc = max(np.abs(oC).max(), np.abs(oG).max())
+    dC, dG = _grad_gpu(qa, cfg, kT, gbar, raster=ras, t=t, closed=closed, n_charges=nc)
+    m = qa.Model(cfg["Cdd"], cfg["Cgd"])
+    mean2 = torch.empty((W * H, n), dtype=torch.float32, device="cuda")
+    pctx = torch.empty(W * H, dtype=torch.int64, device="cuda")
+    qa.qa_soft_occupation_ctx(m.handle, ras, kT, t, closed, nc, mean2, None, pctx)
+    g = torch.tensor(gbar, dtype=torch.float32, device="cuda").contiguous()
+    eC = torch.empty((n, n), dtype=torch.float64, device="cuda")
+    eG = torch.empty((n, n), dtype=torch.float64, device="cuda")
+    qa.qa_soft_occupation_backward_ctx(m.handle, ras, kT, t, closed, nc, g, mean2, pctx, eC, eG)
+    # the fused step's gradient, per-dot target <n> - gbar: g = 2 gbar / (P n)
+    target = (mean2 - g).contiguous()
+    Cdd_d, Cgd_d = torch.tensor(cfg["Cdd"], device="cuda"), torch.tensor(cfg["Cgd"], device="cuda")
+    state = torch.zeros(qa.fit_state_len(n, n), dtype=torch.float64, device="cuda")
+    fC, fG = torch.empty_like(eC), torch.empty_like(eG)
+    qa.qa_fit_step(m.handle, ras, kT, t, closed, nc, target, True, Cdd_d, Cgd_d, state, 1e-3,
+                   dL_dCdd=fC, dL_dCgd=fG)
+    torch.cuda.synchronize()
+    m.close()
+    np.testing.assert_array_equal(mean2.cpu().numpy(), mean.astype(np.float32))
+    f = W * H * n / 2.0
+    for c, d in ((dC, dG), (eC.cpu().numpy(), eG.cpu().numpy()),
+                 (fC.cpu().numpy() * f, fG.cpu().numpy() * f)):
+        assert np.abs(c - oC).max() <= GRAD_RTOL * sc
+        assert np.abs(d - oG).max() <= GRAD_RTOL * sc
