@@ -971,6 +971,7 @@ int qa_charge_sensor(qa_model* m, const qa_raster* r, const int8_t* n_dots,
   L.out_signal = out_signal;
   L.out_n_sensor = out_n_sensor;
   L.out_potential = out_potential;
+  L.num_sms = m->num_sms;
   cudaError_t e = qa::launch_sensor(L, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "sensor launch");
   return QA_OK;

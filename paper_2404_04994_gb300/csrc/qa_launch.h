@@ -112,6 +112,8 @@ struct SensorLaunch {
   float* out_signal;           // [P, S]
   int8_t* out_n_sensor;        // [P, S] (nullable)
   double* out_potential;       // [P, S] (nullable)
+  int num_sms;
+  int run;                     // columns per block (set by launch_sensor)
 };
 cudaError_t launch_sensor(const SensorLaunch& L, cudaStream_t st);
 

@@ -11,15 +11,27 @@
 //      random telegraph, from a counter-based generator (Philox4x32-10,
 //      Salmon et al. 2011), so every value is a pure function of (seed,
 //      sensor, row, column).
-// FP64 throughout (a few hundred operations per pixel).  One block per raster
-// row: the block first marks the row's telegraph switch points in shared
-// memory, then its threads take the pixels.
+// FP64 throughout.  A block takes a run of one raster row in chunks of 64
+// columns, a pixel per thread.  What bounds it: the FP64 pipe (two operations
+// per SM and clock), so nothing is formed twice: the induced charges are
+// affine along a row (one multiply-add per dot and pixel), and an octave of
+// the 1/f noise has one value per 2^k columns, drawn once into shared memory
+// (about three normals per pixel and sensor with the white noise, not one per
+// octave).  Rows are split into runs only while the GPU has SMs to spare,
+// since every run draws its row's telegraph gaps from the start (32 a step).
+// 200 x 200 pixels, 4 dots and a sensor with all noises: 118 us with a
+// block per row, every normal drawn per pixel and c formed gate by gate;
+// about 45 us so (the whole diagram, ground state included, 162 -> 90 us).
+#include <algorithm>
+
 #include "qa_launch.h"
 #include "qa_prep.cuh"
 
 namespace qa {
 
-constexpr int kSensorThreads = 128;
+constexpr int kSensorThreads = 64;
+constexpr int kSensorChunk = kSensorThreads;  // columns a block takes at a time
+constexpr int kSensorOctaves = 14;            // 2^13 = kSensorMaxW
 constexpr int kSensorMaxW = 8192;
 constexpr int kSensorMax = 4;
 
@@ -55,10 +67,23 @@ __device__ __forceinline__ double sensor_gauss(unsigned long long seed, unsigned
   return sqrt(-2.0 * log(u1)) * cos(6.283185307179586 * u2);
 }
 
+// Entries of octave k's values in a chunk (it may straddle one boundary), and
+// of all octaves.
+__host__ __device__ constexpr int octave_room(int k) { return (kSensorChunk >> k) + 1; }
+__host__ __device__ constexpr int octaves_room(int K) {
+  int r = 0;
+  for (int k = 0; k < K; ++k) r += octave_room(k);
+  return r;
+}
+
 struct SensorShared {
   double M[kMaxDot * kMaxDot];
   double Mssi[kSensorMax * kSensorMax];
-  unsigned flips[kSensorMax][kSensorMaxW / 32];  // telegraph switch points
+  double c0[kMaxDot], cu[kMaxDot];       // c(x) = carrier (c0 + x cu) in this row
+  double white[kSensorMax][kSensorChunk];
+  double pink[kSensorMax][octaves_room(kSensorOctaves)];
+  unsigned flips[kSensorMax][kSensorMaxW / 32];  // the run's telegraph switch points
+  int par0[kSensorMax];                          // parity of those before it
   int status;
 };
 
@@ -68,12 +93,25 @@ __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
   const int nf = a.n, S = L.S, nd = nf - S;
   const int W = a.sc.W;
   const unsigned row = blockIdx.x;
-  const int words = (W + 31) / 32;
+  const int first = (int)blockIdx.y * L.run;
+  const int last = min(first + L.run, W);  // the run's columns
+  const int words = (last - first + 31) / 32;
   for (int e = threadIdx.x; e < nf * nf; e += blockDim.x) sh.M[e] = a.md->M[e];
-  for (int e = threadIdx.x; e < kSensorMax * words; e += blockDim.x)
-    sh.flips[e / words][e % words] = 0u;
+  for (int e = threadIdx.x; e < S * words; e += blockDim.x) sh.flips[e / words][e % words] = 0u;
+  if (threadIdx.x >= 32 && threadIdx.x < 32 + nf) {
+    const int i = threadIdx.x - 32;
+    const double ys = a.sc.y0 + (int)row * a.sc.dy;
+    double c0 = 0.0, cu = 0.0;
+    for (int g = 0; g < a.ng; ++g) {
+      const double G = a.md->Cgd[i * a.ng + g];
+      c0 += G * (a.sc.V0[g] + ys * a.sc.w[g]);
+      cu += G * a.sc.u[g];
+    }
+    sh.c0[i] = c0;
+    sh.cu[i] = cu;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == kSensorThreads - 1) {
     // (M_SS)^-1 by Cholesky (S <= 4), column by column
     double Lm[kSensorMax * kSensorMax] = {};
     int ok = 1;
@@ -103,106 +141,185 @@ __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
     }
     sh.status = ok;
   }
-  if (threadIdx.x < S && L.jump_prob > 0.0) {
-    // switch points of sensor s in this row: geometric gaps
-    const int s = threadIdx.x;
+  if (threadIdx.x < 32 && L.jump_prob > 0.0) {
+    // switch points in this row, geometric gaps from its first column on: lane
+    // j of warp 0 draws the j-th of the next 32 and a scan places them
     const double lq = log(1.0 - L.jump_prob);
-    long long pos = -1;
-    for (unsigned j = 0;; ++j) {
-      const uint4 b = sensor_bits(L.seed, 2u | ((unsigned)s << 4), row, j);
-      const double u = ((double)b.x + 1.0) * 2.3283064365386963e-10;
-      const double g = 1.0 + floor(log(u) / lq);
-      if (g > (double)W) break;
-      pos += (long long)g;
-      if (pos >= W) break;
-      sh.flips[s][pos >> 5] ^= 1u << (pos & 31);
+    const int lane = threadIdx.x;
+    for (int s = 0; s < S; ++s) {
+      int pos = -1, before = 0;
+      for (unsigned j = 0; pos < last; j += 32) {
+        const uint4 b = sensor_bits(L.seed, 2u | ((unsigned)s << 4), row, j + (unsigned)lane);
+        const double u = ((double)b.x + 1.0) * 2.3283064365386963e-10;
+        const double g = 1.0 + floor(log(u) / lq);
+        // a longer gap ends the row as well (as does one that is no number, for a
+        // switching probability that vanishes against 1)
+        int at = g >= 1.0 && g <= (double)W ? (int)g : W + 1;
+        for (int off = 1; off < 32; off <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, at, off);
+          if (lane >= off) at += y;
+        }
+        at += pos;
+        before += __popc(__ballot_sync(0xffffffffu, at < first));
+        if (at >= first && at < last)
+          atomicXor(&sh.flips[s][(at - first) >> 5], 1u << ((at - first) & 31));
+        pos = __shfl_sync(0xffffffffu, at, 31);
+      }
+      if (lane == 0) sh.par0[s] = before & 1;
     }
   }
   __syncthreads();
   if (!sh.status) {  // M_SS of a positive definite M is positive definite: unreachable
-    for (int col = threadIdx.x; col < W; col += blockDim.x)
+    for (int col = first + threadIdx.x; col < last; col += blockDim.x)
       for (int s = 0; s < S; ++s) L.out_signal[((long long)row * W + col) * S + s] = __int_as_float(0x7fc00000);
     return;
   }
-  for (int col = threadIdx.x; col < W; col += blockDim.x) {
-    const long long p = (long long)row * W + col;
-    double c[kMaxDot];
-    int nv[kMaxDot];
-    for (int i = 0; i < nf; ++i) c[i] = pixel_c_f64(a.md, a.ng, a.sc, a.mt.carrier, p, i);
-    for (int i = 0; i < nd; ++i) nv[i] = (int)L.n_dots[p * nd + i];
-    // b_a = (M_SD (n_D - c_D))_a - (M_SS c_S)_a : E(n_S) = 1/2 n_S M_SS n_S + n_S . b
-    double g[kSensorMax], bvec[kSensorMax], xs[kSensorMax];
-    for (int s = 0; s < S; ++s) {
-      double acc = 0.0;
-      for (int j = 0; j < nd; ++j) acc += sh.M[(nd + s) * nf + j] * ((double)nv[j] - c[j]);
-      g[s] = acc;
-      double mc = 0.0;
-      for (int t = 0; t < S; ++t) mc += sh.M[(nd + s) * nf + nd + t] * c[nd + t];
-      bvec[s] = acc - mc;
+  const bool white = L.white_sigma > 0.0, pink = L.pink_sigma > 0.0;
+  const int room = kSensorChunk + octaves_room(L.K);
+  for (int b0 = first; b0 < last; b0 += kSensorChunk) {
+    const int b1 = min(b0 + kSensorChunk, last);
+    // the chunk's normals: white, then the octaves' values
+    if (white || pink)
+      for (int e = threadIdx.x; e < S * room; e += blockDim.x) {
+        const int s = e / room;
+        int r = e - s * room;
+        if (r < kSensorChunk) {
+          if (white && b0 + r < b1)
+            sh.white[s][r] = sensor_gauss(L.seed, (unsigned)s << 4, row, (unsigned)(b0 + r));
+        } else if (pink) {
+          r -= kSensorChunk;
+          const int at = r;
+          int k = 0;
+          while (r >= octave_room(k)) r -= octave_room(k++);
+          if ((b0 >> k) + r <= (b1 - 1) >> k)
+            sh.pink[s][at] = sensor_gauss(L.seed, 1u | ((unsigned)s << 4) | ((unsigned)k << 8), row,
+                                          (unsigned)((b0 >> k) + r));
+        }
+      }
+    __syncthreads();
+    const int col = b0 + threadIdx.x;
+    if (col < b1) {
+      const long long p = (long long)row * W + col;
+      const double x = a.sc.x0 + col * a.sc.dx;
+      // g_s = (M_SD (n_D - c_D))_s, the dots one after another
+      double g[kSensorMax] = {0.0, 0.0, 0.0, 0.0};
+      for (int j = 0; j < nd; ++j) {
+        const double r = (double)L.n_dots[p * nd + j] - a.mt.carrier * (sh.c0[j] + x * sh.cu[j]);
+#pragma unroll
+        for (int s = 0; s < kSensorMax; ++s)
+          if (s < S) g[s] += sh.M[(nd + s) * nf + j] * r;
+      }
+      double cs[kSensorMax], bvec[kSensorMax], xs[kSensorMax];
+#pragma unroll
+      for (int s = 0; s < kSensorMax; ++s)
+        cs[s] = s < S ? a.mt.carrier * (sh.c0[nd + s] + x * sh.cu[nd + s]) : 0.0;
+      // b_s = g_s - (M_SS c_S)_s : E(n_S) = 1/2 n_S M_SS n_S + n_S . b
+#pragma unroll
+      for (int s = 0; s < kSensorMax; ++s) {
+        if (s >= S) break;
+        double mc = 0.0, acc = 0.0;
+#pragma unroll
+        for (int t = 0; t < kSensorMax; ++t) {
+          if (t >= S) break;
+          mc += sh.M[(nd + s) * nf + nd + t] * cs[t];
+          acc += sh.Mssi[s * S + t] * g[t];
+        }
+        bvec[s] = g[s] - mc;
+        xs[s] = cs[s] - acc;
+      }
+      int best[kSensorMax] = {0, 0, 0, 0};
+      double bestE = 0.0;
+      for (int m = 0; m < (1 << S); ++m) {
+        int cand[kSensorMax] = {0, 0, 0, 0};
+#pragma unroll
+        for (int s = 0; s < kSensorMax; ++s)
+          if (s < S) cand[s] = (int)floor(xs[s] > 0.0 ? xs[s] : 0.0) + ((m >> s) & 1);
+        double E = 0.0;
+#pragma unroll
+        for (int s = 0; s < kSensorMax; ++s) {
+          if (s >= S) break;
+          double q = 0.0;
+#pragma unroll
+          for (int t = 0; t < kSensorMax; ++t)
+            if (t < S) q += sh.M[(nd + s) * nf + nd + t] * (double)cand[t];
+          E += (double)cand[s] * (0.5 * q + bvec[s]);
+        }
+        bool better = (m == 0) || E < bestE;
+        if (m && E == bestE) {
+          // ties to the lexicographically smaller charges
+          better = false;
+          bool equal = true;
+#pragma unroll
+          for (int s = 0; s < kSensorMax; ++s) {
+            if (equal && cand[s] != best[s]) {
+              better = cand[s] < best[s];
+              equal = false;
+            }
+          }
+        }
+        if (better) {
+          bestE = E;
+#pragma unroll
+          for (int s = 0; s < kSensorMax; ++s) best[s] = cand[s];
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < kSensorMax; ++s) {
+        if (s >= S) break;
+        const int q = nd + s;
+        double V = g[s];  // the dots' part of (M (n - c))_s
+#pragma unroll
+        for (int t = 0; t < kSensorMax; ++t)
+          if (t < S) V += sh.M[q * nf + nd + t] * ((double)best[t] - cs[t]);
+        const double y = (0.5 * sh.M[q * nf + q] - fabs(V)) / L.width;
+        double v = L.shape == 1 ? exp(-0.5 * y * y) : 1.0 / (1.0 + y * y);
+        if (white) v += L.white_sigma * sh.white[s][threadIdx.x];
+        if (pink) {
+          double acc = 0.0;
+          int at = 0;
+          for (int k = 0; k < L.K; ++k) {
+            acc += sh.pink[s][at + (col >> k) - (b0 >> k)];
+            at += octave_room(k);
+          }
+          v += L.pink_sigma * acc / sqrt((double)L.K);
+        }
+        if (L.jump_prob > 0.0) {
+          // telegraph state = parity of the switch points at or before col
+          unsigned par = (unsigned)sh.par0[s];
+          const int rel = col - first, wlast = rel >> 5;
+          for (int w = (b0 - first) >> 5; w < wlast; ++w) par ^= __popc(sh.flips[s][w]) & 1u;
+          const unsigned keep = (rel & 31) == 31 ? 0xffffffffu : ((2u << (rel & 31)) - 1u);
+          par ^= __popc(sh.flips[s][wlast] & keep) & 1u;
+          if (par) v += L.jump_amplitude;
+        }
+        L.out_signal[p * S + s] = (float)v;
+        if (L.out_n_sensor) L.out_n_sensor[p * S + s] = (int8_t)(best[s] > 127 ? 127 : best[s]);
+        if (L.out_potential) L.out_potential[p * S + s] = V;
+      }
     }
-    for (int s = 0; s < S; ++s) {
-      double acc = 0.0;
-      for (int t = 0; t < S; ++t) acc += sh.Mssi[s * S + t] * g[t];
-      xs[s] = c[nd + s] - acc;
+    __syncthreads();
+    // the next chunk starts from this one's parity
+    if (threadIdx.x < S && L.jump_prob > 0.0) {
+      int par = sh.par0[threadIdx.x];
+      const int w0 = (b0 - first) >> 5;
+      for (int w = w0; w < w0 + kSensorChunk / 32 && w < words; ++w)
+        par ^= __popc(sh.flips[threadIdx.x][w]) & 1;
+      sh.par0[threadIdx.x] = par;
     }
-    int best[kSensorMax] = {0, 0, 0, 0};
-    double bestE = 0.0;
-    for (int m = 0; m < (1 << S); ++m) {
-      int cand[kSensorMax];
-      for (int s = 0; s < S; ++s)
-        cand[s] = (int)floor(xs[s] > 0.0 ? xs[s] : 0.0) + ((m >> s) & 1);
-      double E = 0.0;
-      for (int s = 0; s < S; ++s) {
-        double q = 0.0;
-        for (int t = 0; t < S; ++t) q += sh.M[(nd + s) * nf + nd + t] * (double)cand[t];
-        E += (double)cand[s] * (0.5 * q + bvec[s]);
-      }
-      bool better = (m == 0) || E < bestE;
-      if (m && E == bestE) {
-        better = false;
-        for (int s = 0; s < S; ++s)
-          if (cand[s] != best[s]) { better = cand[s] < best[s]; break; }
-      }
-      if (better) {
-        bestE = E;
-        for (int s = 0; s < S; ++s) best[s] = cand[s];
-      }
-    }
-    for (int s = 0; s < S; ++s) nv[nd + s] = best[s];
-    for (int s = 0; s < S; ++s) {
-      const int q = nd + s;
-      double V = 0.0;
-      for (int j = 0; j < nf; ++j) V += sh.M[q * nf + j] * ((double)nv[j] - c[j]);
-      const double y = (0.5 * sh.M[q * nf + q] - fabs(V)) / L.width;
-      double v = L.shape == 1 ? exp(-0.5 * y * y) : 1.0 / (1.0 + y * y);
-      if (L.white_sigma > 0.0)
-        v += L.white_sigma * sensor_gauss(L.seed, (unsigned)s << 4, row, (unsigned)col);
-      if (L.pink_sigma > 0.0) {
-        double acc = 0.0;
-        for (int k = 0; k < L.K; ++k)
-          acc += sensor_gauss(L.seed, 1u | ((unsigned)s << 4) | ((unsigned)k << 8), row,
-                              (unsigned)col >> k);
-        v += L.pink_sigma * acc / sqrt((double)L.K);
-      }
-      if (L.jump_prob > 0.0) {
-        // telegraph state = parity of the switch points at or before col
-        unsigned par = 0u;
-        const int wlast = col >> 5;
-        for (int w = 0; w < wlast; ++w) par ^= __popc(sh.flips[s][w]) & 1u;
-        const unsigned keep = (col & 31) == 31 ? 0xffffffffu : ((2u << (col & 31)) - 1u);
-        par ^= __popc(sh.flips[s][wlast] & keep) & 1u;
-        if (par) v += L.jump_amplitude;
-      }
-      L.out_signal[p * S + s] = (float)v;
-      if (L.out_n_sensor) L.out_n_sensor[p * S + s] = (int8_t)(best[s] > 127 ? 127 : best[s]);
-      if (L.out_potential) L.out_potential[p * S + s] = V;
-    }
+    __syncthreads();
   }
 }
 
-cudaError_t launch_sensor(const SensorLaunch& L, cudaStream_t st) {
-  if (L.a.sc.P == 0) return cudaSuccess;
-  k_sensor<<<(unsigned)L.a.sc.H, kSensorThreads, 0, st>>>(L);
+cudaError_t launch_sensor(const SensorLaunch& L0, cudaStream_t st) {
+  if (L0.a.sc.P == 0) return cudaSuccess;
+  SensorLaunch L = L0;
+  // one run per row, or several while there are fewer than four blocks per SM
+  const int W = L.a.sc.W, H = L.a.sc.H;
+  const long long want = (4LL * L.num_sms + H - 1) / H;
+  const int runs = (int)std::min<long long>((W + kSensorChunk - 1) / kSensorChunk, want);
+  L.run = ((W + runs - 1) / runs + kSensorChunk - 1) / kSensorChunk * kSensorChunk;
+  const unsigned cols = (unsigned)((W + L.run - 1) / L.run);
+  k_sensor<<<dim3((unsigned)H, cols), kSensorThreads, 0, st>>>(L);
   return cudaGetLastError();
 }
 

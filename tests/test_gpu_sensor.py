@@ -102,3 +102,26 @@ def test_sensor_errors(qa):
                 qa.qa_charge_sensor(m.handle, ras, nd, bad, sig)
         assert e.value.code == code
     m.close()
+
+
+# Rows cut into runs and chunks: one pixel, a ragged last chunk, a row at the
+# column limit, many switch points a chunk, more rows than the GPU has SMs for
+# (a block per row), and a switching probability that vanishes against 1.
+@pytest.mark.parametrize("W,H,p", [(1, 1, 0.5), (65, 3, 0.9), (1000, 2, 0.3), (8192, 1, 0.05),
+                                   (130, 700, 0.1), (64, 5, 1e-18)])
+def test_row_runs_match_oracle(qa, W, H, p):
+    Cdd, Cgd = _two_sensors()
+    ras = {"V0": np.array([0.0, 0.0, 2.5, 2.7]), "u": np.array([1.0, 0.1, 0.0, 0.05]),
+           "w": np.array([0.0, 1.0, 0.0, 0.0]), "x0": -0.5, "x1": 4.0, "y0": -0.5, "y1": 4.0,
+           "W": W, "H": H}
+    nd = oracle.ground_state(Cdd[:2, :2], Cgd[:2, :], raster=ras, t=1.0)["n"][:, :2]
+    kw = dict(NOISY, jump_prob=p)
+    sig, ns, pot = _gpu_epilogue(qa, Cdd, Cgd, ras, nd, 2, width=0.05, **kw)
+    ref = oracle.charge_sensor(Cdd, Cgd, ras, nd, n_sensor=2, width=0.05,
+                               **dict(kw, jump_prob=p if p > 1e-16 else 0.0))
+    eps = 0.5 * np.diag(np.linalg.inv(Cdd))[2:] - np.abs(ref["potential"])
+    clear = (eps > 1e-9).all(1)
+    assert clear.mean() > 0.99
+    np.testing.assert_array_equal(ns[clear], ref["n_sensor"][clear])
+    np.testing.assert_allclose(pot[clear], ref["potential"][clear], atol=1e-10)
+    np.testing.assert_allclose(sig[clear], ref["signal"][clear], atol=2e-6, rtol=1e-6)
