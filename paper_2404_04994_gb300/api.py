@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -183,12 +184,20 @@ def _host(a, shape=None):
 
 
 def _stream(stream):
+    """The stream to launch on; None: torch's current one, read through the
+    raw-stream getter (torch.cuda.current_stream() builds a Stream object,
+    5 us of a small call's 50)."""
     if stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        if torch.cuda.is_initialized():
+            try:
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:  # a build of torch without them
+                pass
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _dev(t, dtype, numel=None, name="buffer"):
@@ -204,7 +213,7 @@ def _dev(t, dtype, numel=None, name="buffer"):
         raise ValueError(f"{name} must be contiguous")
     if numel is not None and t.numel() != numel:
         raise ValueError(f"{name} must have {numel} elements, got {t.numel()}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def make_raster(r, n_gate):
@@ -213,13 +222,24 @@ def make_raster(r, n_gate):
     a caller making many calls on one raster can build it once."""
     if isinstance(r, qa_raster):
         return r
-    V0, pV0 = _host(r["V0"], (n_gate,))
-    u, pu = _host(r["u"], (n_gate,))
-    w, pw = _host(r["w"], (n_gate,))
-    s = qa_raster(pV0, pu, pw, float(r["x0"]), float(r["x1"]), float(r["y0"]),
-                  float(r["y1"]), int(r["W"]), int(r["H"]))
+    V0, u, w = (np.ascontiguousarray(r[k], dtype=np.float64) for k in ("V0", "u", "w"))
+    for a in (V0, u, w):
+        if a.shape != (n_gate,):
+            raise ValueError(f"expected shape {(n_gate,)}, got {a.shape}")
+    # the struct's bytes in one go: ctypes pointer objects cost 1 us apiece
+    s = qa_raster.from_buffer_copy(_RASTER.pack(
+        _address(V0), _address(u), _address(w), float(r["x0"]), float(r["x1"]),
+        float(r["y0"]), float(r["y1"]), int(r["W"]) & 0xffffffff, int(r["H"]) & 0xffffffff))
     s._keep = (V0, u, w)
     return s
+
+
+_RASTER = struct.Struct("@PPPddddII")  # qa_raster's layout (W, H by their 32 bits)
+assert _RASTER.size == ctypes.sizeof(qa_raster)
+
+
+def _address(a):
+    return a.__array_interface__["data"][0]
 
 
 # --------------------------------------------------------------------------
