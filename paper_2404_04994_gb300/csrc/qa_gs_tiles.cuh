@@ -94,7 +94,7 @@ struct PrepShared {
   df sV[kMaxGate], sU[kMaxGate], sW[kMaxGate];
   df sc0[kMaxDot], sdu[kMaxDot], sdw[kMaxDot];
   df sG[kMaxDot][kPointGates];     // point lists of <= kPointGates gates: s Cgd
-  float qK[kPrepThreads][kQPRow];  // team QP: KKT rows, active lists, unknowns, c
+  __align__(16) float qK[kPrepThreads][kQPRow];  // team QP: factor rows, active lists, unknowns, c
   int qa[kPrepThreads];
   float qz[kPrepThreads];
   float qzl[kPrepThreads];
@@ -1136,7 +1136,7 @@ __device__ inline void resolve_entry(const GsLaunch& L, const ArrayDesc& a, Reso
 //      lexicographically smallest charge vector.
 // ---------------------------------------------------------------------------
 struct RecheckShared {
-  double qK[32][kQPRow];  // FP64 team QP of warp 0
+  __align__(16) double qK[32][kQPRow];  // FP64 team QP of warp 0
   int qa[32];
   double qz[32], qc[32], v64[kMaxDot], sx64[kMaxDot];
   int sqp;
