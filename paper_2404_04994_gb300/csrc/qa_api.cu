@@ -130,6 +130,54 @@ qa::df split(double v) {
   return {hi, (float)(v - (double)hi)};
 }
 
+// The sphere search's factor of M (SphereConsts): Cdd = L L^T with the dots
+// ordered so that the levels' weights 1 / L_kk fall -- the first levels, which
+// every pattern passes, then separate the patterns most -- and W = L^-1.
+void fill_sphere(int n, qa::ModelData* md) {
+  qa::SphereConsts& s = md->s;
+  std::memset(&s, 0, sizeof(s));
+  for (int i = 0; i < qa::kMaxDot; ++i) s.ord[i] = s.pos[i] = (unsigned char)i;
+  if (n < qa::kSphereMinDot) return;
+  double A[qa::kMaxDot][qa::kMaxDot], L[qa::kMaxDot][qa::kMaxDot] = {}, W[qa::kMaxDot][qa::kMaxDot] = {};
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < n; ++j) A[i][j] = md->Cdd[i * n + j];
+  for (int k = 0; k < n; ++k) {
+    int at = k;
+    for (int i = k + 1; i < n; ++i)
+      if (A[i][i] < A[at][at]) at = i;
+    if (at != k) {
+      for (int j = 0; j < n; ++j) std::swap(A[k][j], A[at][j]);
+      for (int j = 0; j < n; ++j) std::swap(A[j][k], A[j][at]);
+      for (int j = 0; j < k; ++j) std::swap(L[k][j], L[at][j]);
+      std::swap(s.ord[k], s.ord[at]);
+    }
+    if (!(A[k][k] > 0.0)) return;
+    L[k][k] = std::sqrt(A[k][k]);
+    for (int i = k + 1; i < n; ++i) L[i][k] = A[i][k] / L[k][k];
+    for (int i = k + 1; i < n; ++i)
+      for (int j = k + 1; j <= i; ++j) A[i][j] = A[j][i] = A[i][j] - L[i][k] * L[j][k];
+  }
+  double ysq = 0.0, msum = 0.0;
+  for (int k = 0; k < n; ++k) {
+    W[k][k] = std::sqrt(0.5) / L[k][k];
+    for (int j = k - 1; j >= 0; --j) {
+      double r = 0.0;
+      for (int q = j; q < k; ++q) r += L[k][q] * W[q][j];
+      W[k][j] = -r / L[k][k];
+    }
+    double y = 0.0;
+    for (int j = 0; j <= k; ++j) y += std::fabs(W[k][j]);
+    ysq += y * y;
+    for (int j = 0; j < k; ++j) s.W[k][j] = (float)W[k][j];
+    s.wd[k] = (float)W[k][k];
+    for (int j = 0; j < n; ++j) msum += std::fabs(md->M[k * n + j]);
+  }
+  for (int k = 0; k < n; ++k) s.pos[s.ord[k]] = (unsigned char)k;
+  s.ysq = (float)(ysq * (1.0 + 1e-6));
+  s.msum = (float)(msum * (1.0 + 1e-6));
+  s.valid = std::isfinite(s.ysq) && std::isfinite(s.msum);
+}
+
 // FP32 / double-float forms of the model used by every kernel.
 void fill_consts(int n, qa::ModelData* md) {
   qa::ModelConsts& k = md->k;
@@ -168,6 +216,7 @@ void fill_consts(int n, qa::ModelData* md) {
     for (int j = 0; j < i; ++j) qn += std::fmin(0.f, k.Mhi[i * qa::kLdM + j]);
   k.qneg = qn;
   k.model_bad = md->status != 0;
+  fill_sphere(n, md);
 }
 
 // Validate + convert host matrices into a ModelData (Maxwell form).
@@ -389,6 +438,33 @@ qa::RasterK raster_constants(const qa_model* m, const qa::Scan& sc) {
   return rk;
 }
 
+// Whether an array takes the sphere search (cfg: the FP32 search it would
+// take).  Its cost per pixel hardly depends on the candidates' number, 2^kexp
+// expected, the exhaustive walk's doubles with every dot: the line lies where
+// they cross, kexp just above 11 (300 x 200 rasters, exhaustive / sphere, us:
+// 11 dots t = 1 81 / 98, 13 dots t = 0.8 136 / 112, 12 dots t = 1 126 / 107;
+// closed 11 dots 154 / 167, 13 dots t = 0.8 291 / 189, 12 dots 252 / 174).  An
+// open raster too small to fill the GPU walks its candidates in wider teams
+// while the sphere search's few close pixels take a longer list kernel, so
+// there the line is 13 dots (100 x 100: 12 dots 33 / 45, 13 dots 41 / 41, 14
+// dots 53 / 49, 16 dots 58 / 43; closed 12 dots 60 / 53).
+bool use_sphere(int n, double t, long long P, bool closed, const qa::SearchCfg& cfg) {
+  const double kexp = t >= 1.0 ? (double)n : (double)n * std::log2(1.0 + t);
+  return n >= qa::kSphereMinDot && cfg.T >= qa::kTeamFinishMin && cfg.L1 == 5 &&
+         kexp >= (closed || P >= 30000 ? 11.01 : 12.6);
+}
+
+// The sphere search of a single-array call whose other fields are set: its
+// close list takes the block counts' room beyond the grid's entries (at most
+// ceil(P / 8) of P + 1).
+void set_sphere(const qa_model* m, qa::GsLaunch* a) {
+  static_assert(7 * sizeof(qa::BlockCounts) >= 8 * sizeof(qa::CloseEntry),
+                "eight pixels' entries in seven unused counts");
+  a->one.sphere = !m->host_stale && m->host.s.valid &&
+                  use_sphere(m->n, a->one.mt.t, a->one.sc.P, a->one.mt.closed != 0, a->one.cfg);
+  a->close_list = reinterpret_cast<qa::CloseEntry*>(a->bc_prep + qa::sphere_blocks(*a));
+}
+
 int prep_team(int n) {
   int t = 1;
   while (t < n) t <<= 1;
@@ -542,17 +618,22 @@ int run_ground_state(qa_model* m, const ScanIn& in, double t, int closed,
   a.bc_prep = m->d_bc_prep;
   a.bc_search = m->d_bc_search;
   a.cnt = m->d_cnt;
+  a.num_sms = m->num_sms;
+  set_sphere(m, &a);
   a.one.out_n = out_n;
   a.one.out_n16 = out_n16;
   a.one.out_U = out_U;
   a.one.out_flags = out_flags;
-  a.num_sms = m->num_sms;
   m->last_cfg = a.one.cfg;
   m->last_P = P;
   a.ev = m->timing ? m->ev : nullptr;
   m->last_kind = 1;
-  m->n_bc_prep = qa::fused_tiles(a) ? qa::search_blocks(a) : qa::prep_blocks(a);
-  m->n_bc_search = qa::search_blocks(a);
+  if (a.one.sphere) {
+    m->n_bc_prep = m->n_bc_search = qa::sphere_blocks(a);
+  } else {
+    m->n_bc_prep = qa::fused_tiles(a) ? qa::search_blocks(a) : qa::prep_blocks(a);
+    m->n_bc_search = qa::search_blocks(a);
+  }
   e = qa::launch_ground_state(a, st);
   if (e != cudaSuccess) return cuda_fail(e, "ground-state launch");
   return QA_OK;
@@ -1218,6 +1299,8 @@ extern "C" int qa_ground_state_open_static(qa_model* m, const qa_raster* r,
   a.bc_prep = (qa::BlockCounts*)(ws + kStOffBcp);
   a.bc_search = (qa::BlockCounts*)(ws + kStOffBcs);
   a.cnt = cnt;
+  a.num_sms = m->num_sms;
+  set_sphere(m, &a);
   a.one.out_n = out_n;
   a.one.out_U = out_U;
   a.one.out_flags = out_flags;

@@ -113,6 +113,24 @@ struct __align__(16) ModelConsts {
   int pad2[2];
 };
 
+// Arrays of at least this many dots may take the sphere search (qa_sphere.cuh).
+constexpr int kSphereMinDot = 9;
+
+// Factor of M for the sphere search, formed on the host with the model: with
+// Cdd = L L^T in the order `ord` (at each step the dot of the smallest
+// remaining pivot), W = L^-1 / sqrt 2, so that (b - f)^T M (b - f) / 2 =
+// sum_k (sum_{l <= k} W_kl (b_l - f_l))^2.
+struct __align__(16) SphereConsts {
+  float W[kMaxDot][kMaxDot];            // strictly lower triangle, zero elsewhere
+  float wd[kMaxDot];                    // diagonal
+  unsigned char ord[kMaxDot];           // dot of each level
+  unsigned char pos[kMaxDot];           // level of each dot
+  float ysq;                            // sum_k (sum_l |W_kl|)^2
+  float msum;                           // sum_ij |M_ij|
+  int valid;                            // 0: no factor (few dots, or updated on the device)
+  int pad;
+};
+
 // Device copy of a model (written by the host or by the device update).
 struct __align__(16) ModelData {
   double Cdd[kMaxDot * kMaxDot];
@@ -123,6 +141,7 @@ struct __align__(16) ModelData {
   int status;                         // 0 ok; nonzero: Cdd not PD on update
   int pad;
   ModelConsts k;                      // FP32 forms of the above
+  SphereConsts s;
 };
 
 // Where the voltages come from: a raster (by value) or a device list.
@@ -155,6 +174,8 @@ struct Counters {
       unresolved, overflow, doubled, shortlist_max, resolved;
   unsigned int n_flag;  // length of the FP64 recheck list
   unsigned int n_tie;   // length of the near-tie list
+  unsigned int n_close; // length of the close list
+  unsigned int next;    // single array: the sphere search's work queue
   unsigned int q_prep;  // batched launch: work-queue heads
   unsigned int q_search;
   unsigned int q_var[20];  // batched launch: the search queue of each kernel variant
@@ -162,7 +183,7 @@ struct Counters {
   unsigned int soft_done;  // blocks of the soft gradient reduction that have finished
 };
 
-// A single-array call's first kernel clears every counter but the two list
+// A single-array call's first kernel clears every counter but the list
 // heads, which its own blocks append to while others are still starting; the
 // last block of the call's list kernel clears those (and lists_done)
 // instead, so the heads are zero whenever a call starts.
@@ -171,8 +192,10 @@ __device__ __forceinline__ void zero_accumulators(Counters* c) {
   constexpr int k0 = (int)(offsetof(Counters, n_flag) / sizeof(unsigned));
   constexpr int k1 = (int)(offsetof(Counters, n_tie) / sizeof(unsigned));
   constexpr int k2 = (int)(offsetof(Counters, lists_done) / sizeof(unsigned));
+  constexpr int k3 = (int)(offsetof(Counters, n_close) / sizeof(unsigned));
+  constexpr int k4 = (int)(offsetof(Counters, next) / sizeof(unsigned));
   for (int e = threadIdx.x; e < nw; e += blockDim.x)
-    if (e != k0 && e != k1 && e != k2) reinterpret_cast<unsigned*>(c)[e] = 0u;
+    if (e != k0 && e != k1 && e != k2 && e != k3 && e != k4) reinterpret_cast<unsigned*>(c)[e] = 0u;
 }
 
 // A pixel queued for the near-tie resolve or the FP64 recheck: its array (0
@@ -182,6 +205,15 @@ struct ListEntry {
   int p;
   float m1;
   int tie;  // 1 when the order of the best two candidates is in doubt
+};
+
+// A pixel the sphere search could not settle: the candidates within its
+// margin (nl of them, two to four; patterns over the dots), or none (nl = 0).
+struct CloseEntry {
+  int array;
+  int p;
+  unsigned pat01, pat23;
+  int nl;
 };
 
 // Copy the model's FP32 constants into shared memory (16-byte vectors).

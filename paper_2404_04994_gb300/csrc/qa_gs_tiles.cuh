@@ -8,6 +8,7 @@
 #include "qa_launch.h"
 #include "qa_prep.cuh"
 #include "qa_search.cuh"
+#include "qa_sphere.cuh"
 
 namespace qa {
 
@@ -31,12 +32,30 @@ __device__ __forceinline__ void store_charge(const ArrayDesc& a, long long idx, 
   }
 }
 
-// number of k-subsets of size w (k <= 16)
+// number of k-subsets of size w (k <= 16), 0 outside 0 <= w <= k: 16-bit
+// entries (C(16, 8) = 12870), by rows (a loop of 64-bit divisions, run by one
+// lane of a team while the others wait, took a fifth of a closed pixel's
+// prep)
+__constant__ unsigned short kBinom[17][17] = {
+    {1},
+    {1, 1},
+    {1, 2, 1},
+    {1, 3, 3, 1},
+    {1, 4, 6, 4, 1},
+    {1, 5, 10, 10, 5, 1},
+    {1, 6, 15, 20, 15, 6, 1},
+    {1, 7, 21, 35, 35, 21, 7, 1},
+    {1, 8, 28, 56, 70, 56, 28, 8, 1},
+    {1, 9, 36, 84, 126, 126, 84, 36, 9, 1},
+    {1, 10, 45, 120, 210, 252, 210, 120, 45, 10, 1},
+    {1, 11, 55, 165, 330, 462, 462, 330, 165, 55, 11, 1},
+    {1, 12, 66, 220, 495, 792, 924, 792, 495, 220, 66, 12, 1},
+    {1, 13, 78, 286, 715, 1287, 1716, 1716, 1287, 715, 286, 78, 13, 1},
+    {1, 14, 91, 364, 1001, 2002, 3003, 3432, 3003, 2002, 1001, 364, 91, 14, 1},
+    {1, 15, 105, 455, 1365, 3003, 5005, 6435, 6435, 5005, 3003, 1365, 455, 105, 15, 1},
+    {1, 16, 120, 560, 1820, 4368, 8008, 11440, 12870, 11440, 8008, 4368, 1820, 560, 120, 16, 1}};
 __device__ __forceinline__ unsigned long long binom(int k, int w) {
-  if (w < 0 || w > k) return 0ull;
-  unsigned long long r = 1ull;
-  for (int i = 1; i <= w; ++i) r = r * (unsigned long long)(k - w + i) / (unsigned long long)i;
-  return r;
+  return (w < 0 || w > k) ? 0ull : (unsigned long long)kBinom[k][w];
 }
 
 // The descriptor of a list entry's array.
@@ -91,7 +110,6 @@ __device__ __forceinline__ U block_sum(U v, U* red) {
 constexpr int kPointGates = 16;
 struct PrepShared {
   ModelConsts cs;
-  df sV[kMaxGate], sU[kMaxGate], sW[kMaxGate];
   df sc0[kMaxDot], sdu[kMaxDot], sdw[kMaxDot];
   df sG[kMaxDot][kPointGates];     // point lists of <= kPointGates gates: s Cgd
   __align__(16) float qK[kPrepThreads][kQPRow];  // team QP: factor rows, active lists, unknowns, c
@@ -128,8 +146,11 @@ __device__ inline void prep_stage_array(const ArrayDesc& a, PrepShared& sh) {
         sh.sdw[threadIdx.x] = a.rk.dw[threadIdx.x];
       }
     } else {
-      raster_consts(a.md, a.n, a.ng, a.sc, a.mt.carrier, sh.sV, sh.sU, sh.sW, sh.sc0,
-                    sh.sdu, sh.sdw);
+      // (its voltage vectors in the QP rows, which no pixel uses yet)
+      static_assert(sizeof(sh.qK) >= 3 * kMaxGate * sizeof(df), "room for V0, u, w");
+      df* v = reinterpret_cast<df*>(&sh.qK[0][0]);
+      raster_consts(a.md, a.n, a.ng, a.sc, a.mt.carrier, v, v + kMaxGate, v + 2 * kMaxGate,
+                    sh.sc0, sh.sdu, sh.sdw);
     }
   }
   __syncthreads();
@@ -164,19 +185,28 @@ struct PrepAcc {
 };
 
 // ---------------------------------------------------------------------------
-// (a1)-(a4) for one tile: induced charge, continuous minimum, candidate set,
-// h = M (base - c).  A team of TP lanes (a power of two >= N, at most 16)
+// (a1)-(a4) for one pixel: induced charge, continuous minimum and candidate
+// set (prep_set), h = M (base - c) and S (prep_h).  A team of TP lanes (a power of two >= N, at most 16)
 // prepares one pixel, lane i owning dot i; team-wide sums, ballots and gathers
 // use shuffles restricted to the team's lanes, so teams of one warp may
-// diverge.  Pixels team_base + threadIdx.x / TP below p_end are processed.
-// All threads of the block must call (block reductions at the end).
+// diverge.  Every lane of the team must call; a team without a pixel passes
+// active = false.  Per lane: c, x and base of its dot (and whether the dot is
+// live); per team: the rest.
 // ---------------------------------------------------------------------------
+struct PrepPixel {
+  df c, x;
+  int base;
+  bool live;
+  unsigned mask;   // ambiguous dots
+  int w;           // closed: candidate weight; open: -1
+  unsigned flags;
+  unsigned qp_set; // QP pixels: the active set the QP settled on
+};
+
 template <bool CLOSED>
-__device__ inline void prep_tile(const ArrayDesc& a, PrepShared& sh, long long team_base,
-                                 long long p_end, PrepAcc& tot) {
+__device__ __forceinline__ PrepPixel prep_set(const ArrayDesc& a, PrepShared& sh, long long p,
+                                              bool active) {
   const int n = a.n;
-  const float* sMhi = sh.cs.Mhi;
-  const float* sMlo = sh.cs.Mlo;
   const float bx_qp_scale = a.bx_qp_scale > 0.f ? a.bx_qp_scale : sh.cs.bx_qp_scale;
   const bool model_bad = sh.cs.model_bad != 0;
 
@@ -185,16 +215,10 @@ __device__ inline void prep_tile(const ArrayDesc& a, PrepShared& sh, long long t
   const int lane = threadIdx.x & 31;
   const int tbase = lane & ~(TP - 1);                   // team's first lane
   const unsigned tmask = (TP == 32 ? 0xffffffffu : ((1u << TP) - 1u)) << tbase;
-  const long long p = team_base + threadIdx.x / TP;
-  const bool active = p < p_end;
   const bool live = active && lt < n;
   const int nhat = a.mt.n_charges;
 
   // team reductions over lanes (dead lanes contribute zero)
-  auto tsum_f = [&](float v) {
-    for (int off = 1; off < TP; off <<= 1) v += __shfl_xor_sync(tmask, v, off, TP);
-    return v;
-  };
   auto tmax_f = [&](float v) {
     for (int off = 1; off < TP; off <<= 1) v = fmaxf(v, __shfl_xor_sync(tmask, v, off, TP));
     return v;
@@ -413,14 +437,29 @@ __device__ inline void prep_tile(const ArrayDesc& a, PrepShared& sh, long long t
     flags |= kFlagDoubled;
   }
   if (model_bad) flags |= kFlagUnresolved;
+  return {c, x, base, live, mask, w, flags, qp_set};
+}
 
+// The second half: h of the lane's dot (returned) and S, the sum of the
+// magnitudes entering a candidate's energy (per team).
+__device__ __forceinline__ float prep_h(const ArrayDesc& a, PrepShared& sh, const PrepPixel& q,
+                                        float& S) {
+  const int n = a.n;
+  const float* sMhi = sh.cs.Mhi;
+  const float* sMlo = sh.cs.Mlo;
+  const int TP = a.prep_team;
+  const int lt = threadIdx.x & (TP - 1);
+  const int tbase = threadIdx.x & 31 & ~(TP - 1);
+  const unsigned tmask = (TP == 32 ? 0xffffffffu : ((1u << TP) - 1u)) << tbase;
+  const bool live = q.live, amb = q.live && ((q.mask >> lt) & 1u);
+  const unsigned mask = q.mask;
   // h_i = (M (base - c))_i, r = base - c in double-float staged in the
   // team's rows of qx / qz (free after the QP); the products' high parts are
   // summed error-free and their low parts and rounding errors in plain FP32
   // (error O(u^2) of sum |M_ij r_j|, far below the final rounding of h to
   // FP32).  Four columns per step with their loads issued together and two
   // independent sums (even and odd columns), joined error-free at the end.
-  const df r = df_sub({(float)base, 0.f}, c);
+  const df r = df_sub({(float)q.base, 0.f}, q.c);
   const int tb0 = threadIdx.x - lt;
   __syncwarp(tmask);
   sh.qx[threadIdx.x] = r.hi;
@@ -467,33 +506,62 @@ __device__ inline void prep_tile(const ArrayDesc& a, PrepShared& sh, long long t
     }
     Si = sp[0] + sp[1];
   }
-  const float S = tsum_f(Si);
-  const int k = __popc(mask);
+  for (int off = 1; off < TP; off <<= 1) Si += __shfl_xor_sync(tmask, Si, off, TP);
+  S = Si;
+  return h;
+}
 
-  PixRec* rec = a.recs + (active ? p : 0);
-  if (live) {
+// The FP32 gap below which a pixel's best two candidates are a near tie.
+__device__ __forceinline__ float pixel_bound(const ArrayDesc& a, float S, int k) {
+  // the pruned search walks a shallower middle level than the resolve's
+  // re-walk (kCheckL2), which shortlists by this bound, and forms each
+  // rest state from up to kBnbItBits + 2 more table sums
+  return bnb_search(a.cfg.L1, a.cfg.L2)
+             ? near_tie_bound(S, k, max(a.cfg.L2, kCheckL2), kBnbItBits + 2)
+             : near_tie_bound(S, k, a.cfg.L2);
+}
+
+// The pixel's record, for the search and the list kernels (lane lt its dot).
+template <bool CLOSED>
+__device__ __forceinline__ void store_record(PixRec* rec, const PrepPixel& q, int lt, float h,
+                                             float bound) {
+  if (q.live) {
     rec->h[lt] = h;
-    rec->chi[lt] = c.hi;
-    rec->clo[lt] = c.lo;
-    rec->base[lt] = (short)base;
+    rec->chi[lt] = q.c.hi;
+    rec->clo[lt] = q.c.lo;
+    rec->base[lt] = (short)q.base;
   }
+  if (lt == 0) {
+    rec->mask = (unsigned short)q.mask;
+    rec->k = (unsigned char)__popc(q.mask);
+    rec->w = (signed char)(CLOSED ? q.w : -1);
+    rec->flags = (unsigned char)q.flags;
+    rec->qpA = (unsigned short)q.qp_set;
+    rec->bound = bound;
+  }
+}
+
+// prep_set and prep_h for one block's pixels team_base + threadIdx.x / TP below p_end,
+// their records and counts.  All threads of the block must call (block
+// reductions at the end).
+template <bool CLOSED>
+__device__ inline void prep_tile(const ArrayDesc& a, PrepShared& sh, long long team_base,
+                                 long long p_end, PrepAcc& tot) {
+  const int TP = a.prep_team;
+  const int lt = threadIdx.x & (TP - 1);
+  const long long p = team_base + threadIdx.x / TP;
+  const bool active = p < p_end;
+  const PrepPixel q = prep_set<CLOSED>(a, sh, p, active);
+  float S;
+  const float h = prep_h(a, sh, q, S);
+  const int k = __popc(q.mask);
+  if (active) store_record<CLOSED>(a.recs + p, q, lt, h, pixel_bound(a, S, k));
   unsigned long long my_cand = 0;
   unsigned my_qp = 0, my_doubled = 0;
   if (active && lt == 0) {
-    rec->mask = (unsigned short)mask;
-    rec->k = (unsigned char)k;
-    rec->w = (signed char)(CLOSED ? w : -1);
-    rec->flags = (unsigned char)flags;
-    rec->qpA = (unsigned short)qp_set;
-    // the pruned search walks a shallower middle level than the resolve's
-    // re-walk (kCheckL2), which shortlists by this bound, and forms each
-    // rest state from up to kBnbItBits + 2 more table sums
-    rec->bound = bnb_search(a.cfg.L1, a.cfg.L2)
-                     ? near_tie_bound(S, k, max(a.cfg.L2, kCheckL2), kBnbItBits + 2)
-                     : near_tie_bound(S, k, a.cfg.L2);
-    my_cand = CLOSED ? binom(k, w) : (1ull << k);
-    my_qp = (flags & kFlagQP) ? 1u : 0u;
-    my_doubled = (flags & kFlagDoubled) ? 1u : 0u;
+    my_cand = CLOSED ? binom(k, q.w) : (1ull << k);
+    my_qp = (q.flags & kFlagQP) ? 1u : 0u;
+    my_doubled = (q.flags & kFlagDoubled) ? 1u : 0u;
   }
   __syncwarp();
   // one block sum of the three counts packed in 64 bits: candidates in the
@@ -861,6 +929,548 @@ __device__ inline void search_tile(const GsLaunch& L, const ArrayDesc& a, Search
     acc.boundary += (unsigned)((packed >> 42) & 0x3ffu);
     acc.overflow += (unsigned)(packed >> 52);
   }
+}
+
+// U = r^T M r of the lane's charges ni: a row per lane, as in search_tile's
+// wide teams, summed over the team (every lane of tmask calls; rhi, rlo: the
+// team's scratch rows).
+__device__ __forceinline__ df team_energy(const ModelConsts& cs, int n, int lt, unsigned tmask,
+                                          bool live, int ni, df c, float* rhi, float* rlo) {
+  const df r = live ? df_sub({(float)ni, 0.f}, c) : df{0.f, 0.f};
+  __syncwarp(tmask);
+  rhi[lt] = r.hi;
+  rlo[lt] = r.lo;
+  __syncwarp(tmask);
+  df u = {0.f, 0.f};
+  if (live) {
+    const float* Mh = cs.Mhi + lt * kLdM;
+    const float* Ml = cs.Mlo + lt * kLdM;
+    float shi = 0.f, slo = 0.f;
+    for (int j = 0; j < n; ++j) {
+      const float mh = Mh[j], ml = Ml[j];
+      const float xh = rhi[j], xl = rlo[j];
+      const df pr = two_prod(mh, xh);
+      const float small = __fmaf_rn(mh, xl, __fmaf_rn(ml, xh, pr.lo));
+      const df sm = two_sum(shi, pr.hi);
+      shi = sm.hi;
+      slo = __fadd_rn(slo, __fadd_rn(sm.lo, small));
+    }
+    u = df_mul(fast_two_sum(shi, slo), r);
+  }
+#pragma unroll
+  for (int off = 1; off < kSphT; off <<= 1) {
+    df o;
+    o.hi = __shfl_xor_sync(tmask, u.hi, off, kSphT);
+    o.lo = __shfl_xor_sync(tmask, u.lo, off, kSphT);
+    u = df_add(u, o);
+  }
+  return u;
+}
+
+// ---------------------------------------------------------------------------
+// (a1)-(a6), (a8) in one pass for arrays of 9 to 16 dots: a team of 16 lanes,
+// lane i owning dot i, prepares a pixel, searches its candidate set with the
+// sphere search and writes its outputs; c, the candidate set and h stay in
+// the lanes.  A pixel with candidates too close to call, or whose search does
+// not end (no factor, or too many nodes), gets its record and goes on the
+// close list (settle_entry); one whose candidate set is in doubt gets its
+// record and goes on the FP64 list.
+// What bounds it: instruction issue (1,430 warp instructions per 16-dot pixel,
+// 2.4 - 3 a cycle; the tile kernels' 3,061, three quarters of them in the
+// FP32 search).  Sixteen lanes a pixel as in the prep, so that a pixel's whole
+// way keeps its lanes.  Whole calls, before / after: 16 dots 100 x 100 57 / 42
+// us (closed 93 / 60), 16-dot list of 10^4 vectors 71 / 54 us, 12 dots
+// 400 x 301 241 / 172 us.
+// ---------------------------------------------------------------------------
+constexpr int kSphereTeams = kPrepThreads / kSphT;
+struct SphereShared {
+  PrepShared p;
+  SphereModel m;
+  float4 lev[kSphereTeams][kMaxDot / 2];
+  unsigned long long cand[kSphereTeams], ev[kSphereTeams];
+  unsigned qp[kSphereTeams], doubled[kSphereTeams], boundary[kSphereTeams],
+      overflow[kSphereTeams];
+  int valid;
+};
+static_assert(kSphT * sizeof(float) * kQPRow >= kSphStack * sizeof(uint2),
+              "the team's QP rows hold its waiting nodes");
+
+// Block set-up (all threads), once per array.
+__device__ inline void sphere_stage_array(const ArrayDesc& a, SphereShared& sh) {
+  sphere_stage(a.md->s, sh.m);
+  if (threadIdx.x == 0) sh.valid = a.md->s.valid;
+  prep_stage_array(a, sh.p);  // ends with a barrier
+}
+__device__ inline void sphere_zero_counts(SphereShared& sh) {
+  if (threadIdx.x < kSphereTeams) {
+    sh.cand[threadIdx.x] = sh.ev[threadIdx.x] = 0ull;
+    sh.qp[threadIdx.x] = sh.doubled[threadIdx.x] = 0u;
+    sh.boundary[threadIdx.x] = sh.overflow[threadIdx.x] = 0u;
+  }
+}
+// The block's counts (thread 0 after a barrier).
+__device__ inline void sphere_counts(const SphereShared& sh, BlockCounts& prep,
+                                     BlockCounts& search) {
+  PrepAcc p;
+  SearchAcc s;
+  for (int t = 0; t < kSphereTeams; ++t) {
+    p.candidates += sh.cand[t];
+    p.qp += sh.qp[t];
+    p.doubled += sh.doubled[t];
+    s.evaluated += sh.ev[t];
+    s.boundary += sh.boundary[t];
+    s.overflow += sh.overflow[t];
+  }
+  prep.candidates = p.candidates;
+  prep.qp = p.qp;
+  prep.doubled = p.doubled;
+  search.evaluated = s.evaluated;
+  search.near_tie = 0u;
+  search.boundary = s.boundary;
+  search.overflow = s.overflow;
+}
+
+// One warp's two pixels, p its team's (active: below the end).
+template <bool CLOSED>
+__device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, SphereShared& sh,
+                                    int array, long long p, bool active) {
+  const int n = a.n;
+  const int lt = threadIdx.x & (kSphT - 1);
+  const int tq = threadIdx.x & ~(kSphT - 1);
+  const int team = threadIdx.x / kSphT;
+  const unsigned hw = threadIdx.x & 16u;
+  const PrepPixel q = prep_set<CLOSED>(a, sh.p, p, active);
+  const bool amb = q.live && ((q.mask >> lt) & 1u);
+  const int k = __popc(q.mask);
+  const bool qp = (q.flags & kFlagQP) != 0u;
+  constexpr float u24 = 5.9604645e-8f;
+  // the centre f = x - base
+  const float f = q.live ? __fadd_rn(__fsub_rn(q.x.hi, (float)q.base), q.x.lo) : 0.f;
+  // A bound of the near-tie bound: S as in prep_h but with a plain FP32 h,
+  // whose error (17 roundings of 16 products) is added.  The record's h, in
+  // double-float, is formed for the few pixels that need their record; h was
+  // an eighth of this kernel's instructions.
+  const float r0 = q.live ? __fadd_rn(__fsub_rn((float)q.base, q.c.hi), -q.c.lo) : 0.f;
+  const float* Mrow = sh.p.cs.Mhi + lt * kLdM;
+  __syncwarp();
+  sh.p.qx[threadIdx.x] = r0;
+  sh.p.qz[threadIdx.x] = q.live ? __fadd_rn(__fsub_rn(q.x.hi, q.c.hi), q.x.lo - q.c.lo) : 0.f;
+  __syncwarp();
+  float S = 0.f;
+  {
+    float h0 = 0.f, h1 = 0.f;
+#pragma unroll
+    for (int j = 0; j < kMaxDot; j += 4) {
+      const float4 r4 = *reinterpret_cast<const float4*>(&sh.p.qx[tq + j]);
+      h0 = fmaf(Mrow[j], r4.x, h0);
+      h1 = fmaf(Mrow[j + 1], r4.y, h1);
+      h0 = fmaf(Mrow[j + 2], r4.z, h0);
+      h1 = fmaf(Mrow[j + 3], r4.w, h1);
+    }
+    const unsigned below = q.mask & ((1u << lt) - 1u);
+    if (amb) {
+      S = fabsf(h0 + h1);
+      if (below == (1u << lt) - 1u) {
+        S += sh.p.cs.absl[lt];
+      } else {
+        S += 0.5f * Mrow[lt];
+#pragma unroll
+        for (int j = 0; j < kMaxDot; ++j) S += ((below >> j) & 1u) ? fabsf(Mrow[j]) : 0.f;
+      }
+    }
+  }
+#pragma unroll
+  for (int off = 8; off > 0; off >>= 1) S += __shfl_xor_sync(kFull, S, off);
+  // the gradient M (x - c) where a constraint is active (else zero, closed: a
+  // multiple of 1)
+  float a1 = 0.f, neg = 0.f, rmax = 1.f;
+  if (__any_sync(kFull, qp)) {
+    float z = 0.f;
+#pragma unroll
+    for (int j = 0; j < kMaxDot; ++j) z = fmaf(Mrow[j], sh.p.qz[tq + j], z);
+    rmax = fmaxf(fabsf(r0), fabsf(sh.p.qz[threadIdx.x]));
+    if (CLOSED) {  // the multiple of 1: the least entry, a free dot's
+      float zm = q.live ? z : kInf;
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) zm = fminf(zm, __shfl_xor_sync(kFull, zm, off));
+      z -= zm;
+    }
+    a1 = (qp && amb) ? fmaxf(z, 0.f) : 0.f;
+    neg = (qp && amb) ? fmaxf(-z, 0.f) : 0.f;
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) {
+      neg += __shfl_xor_sync(kFull, neg, off);
+      rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
+    }
+  }
+  const float ez = u24 * a.md->s.msum * fmaxf(rmax, 1.f);  // u sum |M| |r|
+  const float bound = pixel_bound(a, S * 1.00001f + 20.f * ez, k);
+  neg += (qp ? 24.f : 2.f) * ez;
+  // no factor, or a centre outside [-1, 1] (an unsettled QP): left to the
+  // FP32 search
+  const bool far = ((__ballot_sync(kFull, !(fabsf(f) <= 1.f)) >> hw) & 0xffffu) != 0u;
+  int close = 0;
+  unsigned ev = 0;
+  const unsigned bits = sphere_search<CLOSED>(
+      a.md->s, sh.m, n, lt, active && sh.valid && !far, f, a1, q.mask, q.w, bound, neg,
+      &sh.p.qx[tq], &sh.p.qz[tq], sh.lev[team], reinterpret_cast<uint2*>(&sh.p.qK[tq][0]), close,
+      ev);
+  const bool done = active && close == 1;
+  // candidates too close to tell apart (up to four): left, with their patterns
+  // over the dots, to the list kernel; so is a search that did not end
+  if (__any_sync(kFull, active && close != 1)) {
+    const unsigned* lst = reinterpret_cast<const unsigned*>(&sh.p.qz[tq]);
+    unsigned pat[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      pat[e] = (__ballot_sync(kFull, lt < n && e < close && ((lst[e] >> sh.m.pos[lt]) & 1u)) >> hw) &
+               0xffffu;
+    if (active && close != 1 && lt == 0) {
+      const unsigned at = atomicAdd(&L.cnt->n_close, 1u);
+      L.close_list[at] = CloseEntry{array, (int)p, pat[0] | (pat[1] << 16), pat[2] | (pat[3] << 16),
+                                    close <= 4 ? close : 0};
+    }
+    __syncwarp();
+  }
+
+  // n* = base + bits and U(n*) = 1/2 r^T M r
+  int ni = q.base + (int)((bits >> lt) & 1u);
+  const df u = team_energy(sh.p.cs, n, lt, kFull, q.live, ni, q.c, &sh.p.qx[tq], &sh.p.qz[tq]);
+  unsigned flags = q.flags, ov = 0u;
+  // int8 maps of 16 dots: the team's charges as one 16-byte store
+  const bool vec = !a.out_n16 && n == 16 && (reinterpret_cast<uintptr_t>(a.out_n) & 15u) == 0;
+  if (vec) {
+    if (ni > 127) {
+      ni = 127;
+      ov = kFlagOverflow;
+    }
+    unsigned word = ((unsigned)ni & 0xffu) << (8 * (lt & 3));
+    word |= __shfl_xor_sync(kFull, word, 1);
+    word |= __shfl_xor_sync(kFull, word, 2);
+    const unsigned w1 = __shfl_sync(kFull, word, hw + 4), w2 = __shfl_sync(kFull, word, hw + 8);
+    const unsigned w3 = __shfl_sync(kFull, word, hw + 12);
+    const unsigned w0 = word;
+    if (done && lt == 0)
+      *reinterpret_cast<int4*>(a.out_n + p * n) =
+          make_int4((int)w0, (int)w1, (int)w2, (int)w3);
+  } else if (done && q.live) {
+    store_charge(a, p * n + lt, ni, ov);
+  }
+  if ((__ballot_sync(kFull, ov != 0u) >> hw) & 0xffffu) flags |= kFlagOverflow;
+  const unsigned evw = __reduce_add_sync(kFull, ev);
+  if (active && lt == 0) {
+    sh.cand[team] += CLOSED ? binom(k, q.w) : (1ull << k);
+    sh.qp[team] += qp ? 1u : 0u;
+    sh.doubled[team] += (q.flags & kFlagDoubled) ? 1u : 0u;
+    if (hw == 0u) sh.ev[team] += evw;
+  }
+  const bool listed = done && (flags & (kFlagBoundary | kFlagQPCap | kFlagUnresolved)) != 0u;
+  if (active && (close != 1 || listed)) {
+    float Sx;
+    const float h = prep_h(a, sh.p, q, Sx);
+    store_record<CLOSED>(a.recs + p, q, lt, h, pixel_bound(a, Sx, k));
+  }
+  if (done && lt == 0) {
+    if (a.out_U) a.out_U[p] = 0.5 * df_to_double(u);
+    if (a.out_flags) a.out_flags[p] = (uint8_t)flags;
+    if (listed) {
+      L.flag_list[atomicAdd(&L.cnt->n_flag, 1u)] = ListEntry{array, (int)p, 0.f, 0};
+      ++sh.boundary[team];
+    }
+    if (flags & kFlagOverflow) ++sh.overflow[team];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Pixels that the sphere search left (the close list): the FP32 search's
+// near-tie flag and, where it is set, the argmin by exact energies.
+// ---------------------------------------------------------------------------
+// The pruned FP32 search's minimum of one block (an outer pattern with its
+// middle pattern): the tables' entries, sums and middle walk of search_bnb,
+// formed for that block alone.  pm, vv: its slot pairs and single-flip
+// energies; ptab: its inner pair table; nlb: the lane bits of its team.
+template <bool CLOSED>
+__device__ __forceinline__ float bnb_block_min(const float* pm, const float* vv, const float* ptab,
+                                               int k, int w, int nlb, unsigned blk) {
+  constexpr int L1 = kBnbL1, L2 = kBnbL2, kLB = 5;
+  static_assert(L2 == 2, "two middle slots");
+  const int nmid = min(max(k - L1, 0), L2), nout = max(k - kBnbIn, 0), nit = nout - nlb;
+  const unsigned o = blk >> L2, li = o & ((1u << nlb) - 1u), it = o >> nlb;
+  const int s0 = kBnbIn + nlb;
+  float wO[kLB], wI[kBnbItBits], L[kBnbIn], At = 0.f, Ai = 0.f, x = 0.f;
+#pragma unroll
+  for (int i = 0; i < kLB; ++i) wO[i] = (i < nlb && ((li >> i) & 1u)) ? 1.f : 0.f;
+#pragma unroll
+  for (int i = 0; i < kBnbItBits; ++i) wI[i] = (i < nit && ((it >> i) & 1u)) ? 1.f : 0.f;
+#pragma unroll
+  for (int i = 0; i < kLB; ++i) {
+    const float* prow = pm + min(kBnbIn + i, kMaxDot - 1) * kLdM;
+    float add = vv[min(kBnbIn + i, kMaxDot - 1)];
+#pragma unroll
+    for (int i2 = 0; i2 < i; ++i2) add = fmaf(wO[i2], prow[kBnbIn + i2], add);
+    At = fmaf(wO[i], add, At);
+  }
+#pragma unroll
+  for (int j = 0; j < kBnbIn; ++j) {
+    float a = vv[j], b = 0.f;
+#pragma unroll
+    for (int i = 0; i < kLB; ++i) a = fmaf(wO[i], pm[min(kBnbIn + i, kMaxDot - 1) * kLdM + j], a);
+#pragma unroll
+    for (int i = 0; i < kBnbItBits; ++i) b = fmaf(wI[i], pm[j * kLdM + min(s0 + i, kMaxDot - 1)], b);
+    L[j] = a + b;
+  }
+#pragma unroll
+  for (int ii = 0; ii < kBnbItBits; ++ii) {
+    const int si = min(s0 + ii, kMaxDot - 1);
+    float add = vv[si], cr = 0.f;
+#pragma unroll
+    for (int i2 = 0; i2 < ii; ++i2)
+      add = fmaf(wI[i2], pm[si * kLdM + min(s0 + i2, kMaxDot - 1)], add);
+    Ai = fmaf(wI[ii], add, Ai);
+#pragma unroll
+    for (int i = 0; i < kLB; ++i) cr = fmaf(wO[i], pm[min(kBnbIn + i, kMaxDot - 1) * kLdM + si], cr);
+    x = fmaf(wI[ii], cr, x);
+  }
+  float A = (At + x) + Ai, g0 = L[L1], g1 = L[L1 + 1];
+  const unsigned mid = blk & 3u;
+  const float mm = nmid > 1 ? pm[(L1 + 1) * kLdM + L1] : 0.f;
+  auto flip = [&](int m, float g, bool up) {
+    A = up ? A + g : A - g;
+#pragma unroll
+    for (int j = 0; j < L1; ++j) {
+      const float d = m < nmid ? pm[j * kLdM + L1 + m] : 0.f;
+      L[j] = up ? L[j] + d : L[j] - d;
+    }
+  };
+  if (mid) {  // the walk's middle patterns: 0, 1, 3, 2
+    flip(0, g0, true);
+    g1 += mm;
+    if (mid & 2u) {
+      flip(1, g1, true);
+      g0 += mm;
+      if (mid == 2u) flip(0, g0, false);
+    }
+  }
+  return CLOSED ? inner_min_closed_smem<L1>(A, L, ptab, w - __popc(o) - __popc(mid))
+                : inner_min_open_smem<L1>(A, L, ptab);
+}
+
+// A warp's scratch for an entry of the close list.
+struct SettleScratch {
+  int sdot[kMaxDot];
+  float sh[kMaxDot];
+  unsigned lst[4];
+  float rhi[2][kMaxDot], rlo[2][kMaxDot];
+  union {
+    struct {
+      __align__(16) float ptab[1 << kBnbL1];
+      float pm[kMaxDot * kLdM];
+      float vv[kMaxDot];
+    } bnb;
+    struct {
+      __align__(16) float colt[4 * kColStride];
+      __align__(16) float itab[(1 << kItMax) * kItStride];
+      __align__(16) float cslot[32][kItMax];
+    } team;
+  } u;
+};
+
+// The FP32 search's best candidate (m1, pattern over the slots b1) and
+// runner-up m2 among the blocks of the nl listed candidates (slot patterns in
+// t.lst), or among all of them (nl = 0), with the sums that the array's search
+// takes: its split (5 + 2 or 5 + 4, block-level teams) and team width say
+// which, and lane v of that team runs in lane v of the warp.
+template <bool CLOSED>
+static __device__ __noinline__ void listed_top2(const ArrayDesc& a, const float* sM,
+                                                const SlotView sv, SettleScratch& t, int nl,
+                                                float& m1, unsigned& b1, float& m2) {
+  const int lane = threadIdx.x & 31, T = a.cfg.T, k = sv.k;
+  const bool bnb = bnb_search(a.cfg.L1, a.cfg.L2);
+  unsigned blk = 0u;
+  if (lane < nl) blk = t.lst[lane] >> a.cfg.L1;
+  __syncwarp();
+  if (lane < nl) t.lst[lane] = blk;
+  __syncwarp();
+  m1 = m2 = kInf;
+  b1 = 0u;
+  if (bnb) {
+    // the tables of bnb_pair_build, an element per lane, and the inner pairs
+    float* pm = t.u.bnb.pm;
+#pragma unroll
+    for (int e = lane; e < kMaxDot * kMaxDot; e += 32) {
+      const int r = e >> 4, c = e & 15;
+      pm[r * kLdM + c] = (r < k && c < k) ? sM[sv.dot[r] * kLdM + sv.dot[c]] : 0.f;
+    }
+    if (lane < kMaxDot)
+      t.u.bnb.vv[lane] = lane < k ? sv.h[lane] + 0.5f * sM[sv.dot[lane] * (kLdM + 1)]
+                                  : (lane < kBnbL1 ? kBig : 0.f);
+    __syncwarp();
+    {
+      float r = 0.f;
+#pragma unroll
+      for (int j = 1; j < kBnbL1; ++j)
+#pragma unroll
+        for (int l = 0; l < j; ++l)
+          r = fmaf((((lane >> j) & 1) && ((lane >> l) & 1)) ? 1.f : 0.f, pm[j * kLdM + l], r);
+      t.u.bnb.ptab[lane] = r;
+    }
+    __syncwarp();
+    const int nout = max(k - kBnbIn, 0), nlb = min(__ffs(T) - 1, nout);
+    bool own = lane < nl;
+    for (int e = 0; e < min(lane, nl); ++e) own = own && t.lst[e] != blk;
+    const unsigned nblk = nl > 0 ? (own ? 1u : 0u) : (1u << (nout + kBnbL2)), first = nl > 0 ? blk : lane;
+    // (a middle pattern beyond the k slots holds no block)
+    const unsigned midmax = 1u << min(max(k - kBnbL1, 0), kBnbL2);
+#pragma unroll 1
+    for (unsigned q = nl > 0 ? 0u : (unsigned)lane, b = first; q < nblk; q += 32u, b += 32u) {
+      if ((b & 3u) >= midmax) continue;
+      const float e = bnb_block_min<CLOSED>(pm, t.u.bnb.vv, t.u.bnb.ptab, k, sv.w, nlb, b);
+      m2 = fminf(m2, fmaxf(m1, e));
+      if (e < m1) {
+        m1 = e;
+        b1 = b;
+      }
+    }
+  } else {
+    // split 5 + 4: block minima from the team tables
+    constexpr int L1 = 5, L2 = 4;
+    unsigned long long ev = 0;
+    col_build<L1, L2>(sM, sv, lane, 32, t.u.team.colt);
+    iter_build<L1, L2>(sM, sv, lane, T, t.u.team.itab, 32);
+    __syncwarp();
+    if (lane < T)
+      search_lane<L1, L2, CLOSED, false, true, 5, true>(
+          sM, sv, lane, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev, t.u.team.colt,
+          t.u.team.itab, t.u.team.cslot[lane], kInf, 0.f, t.lst, nl > 0 ? nl : -1);
+  }
+  for (int off = 1; off < 32; off <<= 1) {
+    const float o1 = __shfl_xor_sync(kFull, m1, off), o2 = __shfl_xor_sync(kFull, m2, off);
+    const unsigned ob = __shfl_xor_sync(kFull, b1, off);
+    top2_merge(m1, b1, m2, o1, ob, o2);
+  }
+  float e1, e2;
+  unsigned fb;
+  const unsigned best = m1 < kInf ? b1 : 0u;
+  if (bnb) team_finish<kBnbL1, kBnbL2, CLOSED>(sM, sv, lane & (T - 1), T, kFull, best, e1, fb, e2);
+  else team_finish<5, 4, CLOSED>(sM, sv, lane & (T - 1), T, kFull, best, e1, fb, e2);
+  if (m1 < kInf) {
+    m1 = e1;
+    b1 = fb;
+    m2 = fminf(m2, e2);
+  }
+}
+
+// One entry of the close list, by a warp: the argmin by the exact energies of
+// the listed candidates, the near-tie flag by the FP32 search's energies of the
+// same candidates (any other is further than the bound from the minimum in
+// every FP32 sum, so the flag and the charges are those of the FP32 search
+// and the resolve).  Without a list (nl = 0): the FP32 search over all of
+// them.  Returns 0 when the pixel is done, 1 when the resolve has to follow
+// (energies too close for double-float, or no list and a near tie), 2 for
+// the FP64 recheck (e: the entry for either).
+// What bounds it: latency, on cold instruction caches.  With the whole FP32
+// search as a kernel of its own and the resolve behind it, these few pixels
+// took 26 us of the 16-dot 100 x 100 diagram's 52; settled inside the sphere
+// search's warps they lengthened its tail by 23 us.
+template <bool CLOSED>
+__device__ inline int settle_entry(const GsLaunch& L, const ArrayDesc& a, const ModelConsts& cs,
+                                   SettleScratch& t, const CloseEntry& ce, ListEntry& e) {
+  const int n = a.n;
+  const int lane = threadIdx.x & 31, lt = lane & 15, half = lane >> 4;
+  const PixRec* rec = a.recs + ce.p;
+  const bool live = lt < n;
+  const int base = live ? rec->base[lt] : 0;
+  const df c = live ? df{rec->chi[lt], rec->clo[lt]} : df{0.f, 0.f};
+  const float h = live ? rec->h[lt] : 0.f;
+  const unsigned mask = rec->mask;
+  const float bound = rec->bound;
+  const int w = rec->w;
+  unsigned flags = rec->flags;
+  const int k = __popc(mask);
+  const bool amb = live && ((mask >> lt) & 1u);
+  const int nl = ce.nl;
+  // slots: dots in order, or (pruned search) by |h + M_ii / 2|
+  int slot = __popc(mask & ((1u << lt) - 1u));
+  if (bnb_search(a.cfg.L1, a.cfg.L2)) {
+    const float key = amb ? fabsf(h + 0.5f * cs.Mhi[lt * kLdM + lt]) : 0.f;
+    int rank = 0;
+#pragma unroll
+    for (int j = 0; j < kMaxDot; ++j) {
+      const float kj = __shfl_sync(kFull, key, j);
+      rank += (((mask >> j) & 1u) && (kj < key || (kj == key && j < lt))) ? 1 : 0;
+    }
+    slot = rank;
+  }
+  __syncwarp();
+  if (amb && half == 0) {
+    t.sdot[slot] = lt;
+    t.sh[slot] = h;
+  }
+  // exact energies, two candidates at a time (2 U)
+  df best = {kInf, 0.f}, second = {kInf, 0.f};
+  unsigned bbits = 0u;
+  auto take = [&](df u, unsigned b) {
+    const bool better = u.hi < best.hi || (u.hi == best.hi && u.lo < best.lo);
+    const df lose = better ? best : u;
+    if (lose.hi < second.hi || (lose.hi == second.hi && lose.lo < second.lo)) second = lose;
+    if (better) {
+      best = u;
+      bbits = b;
+    }
+  };
+  auto pattern = [&](int i) { return ((i < 2 ? ce.pat01 : ce.pat23) >> (16 * (i & 1))) & 0xffffu; };
+#pragma unroll 1
+  for (int i = 0; i < nl; i += 2) {
+    const unsigned b = pattern(i + half);
+    const df u = team_energy(cs, n, lt, kFull, live, base + (int)((b >> lt) & 1u), c, t.rhi[half],
+                             t.rlo[half]);
+    const unsigned sb =
+        __reduce_or_sync(half ? 0xffff0000u : 0xffffu, (amb && ((b >> lt) & 1u)) ? 1u << slot : 0u);
+    if (lt == 0 && i + half < nl) t.lst[i + half] = sb;
+    df u0, u1;
+    u0.hi = __shfl_sync(kFull, u.hi, 0);
+    u0.lo = __shfl_sync(kFull, u.lo, 0);
+    u1.hi = __shfl_sync(kFull, u.hi, 16);
+    u1.lo = __shfl_sync(kFull, u.lo, 16);
+    take(u0, pattern(i));
+    if (i + 1 < nl) take(u1, pattern(i + 1));
+  }
+  __syncwarp();
+  const SlotView sv{t.sdot, t.sh, k, CLOSED ? w : -1};
+  float m1, m2;
+  unsigned b1;
+  listed_top2<CLOSED>(a, cs.Mhi, sv, t, nl, m1, b1, m2);
+  const bool near = !(m2 - m1 > bound);
+  const bool boundary = (flags & (kFlagBoundary | kFlagQPCap | kFlagUnresolved)) != 0u;
+  // the resolve decides gaps of the energies below 1e-10 (1 + |U(base)|):
+  // leave it a hundred times that (U(base) <= U + S, and the bound is at least
+  // 24 2^-24 S)
+  const df gap2 = df_sub(second, best);
+  const bool exact = nl > 1 && 0.5f * gap2.hi > 1e-8f * (1.f + best.hi) + 1e-2f * bound;
+  const int next = boundary ? 2 : (near && !exact) ? 1 : 0;
+  // the FP32 search's candidate stands until what follows
+  const bool bit = amb && ((nl == 0 || (near && next != 0)) ? (b1 >> slot) & 1u
+                                                            : (bbits >> lt) & 1u);
+  const int ni = base + (bit ? 1 : 0);
+  if (nl == 0) best = team_energy(cs, n, lt, kFull, live, ni, c, t.rhi[half], t.rlo[half]);
+  if (near) flags |= kFlagNearTie | (next == 0 ? kFlagRechecked : 0u);
+  unsigned ov = 0u;
+  if (live && half == 0) store_charge(a, (long long)ce.p * n + lt, ni, ov);
+  if (__any_sync(kFull, ov != 0u)) flags |= kFlagOverflow;
+  if (lane == 0) {
+    if (a.out_U) a.out_U[ce.p] = 0.5 * df_to_double(best);
+    if (a.out_flags) a.out_flags[ce.p] = (uint8_t)flags;
+    if (boundary) atomicAdd(&L.cnt->boundary, 1ull);
+    else if (near) atomicAdd(&L.cnt->near_tie, 1ull);
+    if (near && next == 0) {
+      atomicAdd(&L.cnt->resolved, 1ull);
+      atomicMax(&L.cnt->shortlist_max, (unsigned long long)nl);
+    }
+    if (flags & kFlagOverflow) atomicAdd(&L.cnt->overflow, 1ull);
+  }
+  e = ListEntry{ce.array, ce.p, m1, (next == 2 && near) ? 1 : 0};
+  __syncwarp();
+  return next;
 }
 
 // ---------------------------------------------------------------------------

@@ -2,6 +2,8 @@
 // for prep and search (one kernel or two), grid-stride over the lists for
 // resolve and recheck.
 // The stages themselves live in qa_gs_tiles.cuh (shared with the batch).
+#include <algorithm>
+
 #include "qa_gs_tiles.cuh"
 
 namespace qa {
@@ -112,17 +114,54 @@ __global__ void __launch_bounds__(kSearchThreads, kBnbBlocks) k_search_bnb(GsLau
   search_only_tile<kBnbL1, kBnbL2, CLOSED, true>(L);
 }
 
-// The lists after the search, in one launch: near ties (resolve_entry) and
-// the FP64 recheck list (recheck_entry), grid-stride over both; a near tie
-// the resolve cannot settle is rechecked next by the same block.  The two
-// entries' shared layouts overlap, so each restages its model constants when
-// the other ran last.
+// Prep, sphere search and outputs of arrays of 9 to 16 dots: a persistent
+// grid whose warps take pixel pairs one at a time (no barrier between a
+// block's warps, so a slow pixel holds up its own warp only).
+template <bool CLOSED>
+__global__ void __launch_bounds__(kPrepThreads, kSphereBlocks)
+k_sphere(const __grid_constant__ GsLaunch L) {
+  __shared__ SphereShared sh;
+  const ArrayDesc& a = L.one;
+  grid_dep_signal();
+  if (blockIdx.x == 0) zero_accumulators(L.cnt);
+  sphere_zero_counts(sh);
+  sphere_stage_array(a, sh);
+  // whole rounds of pairs by the warp's place, what is left over from a counter
+  const unsigned pairs = (unsigned)((a.sc.P + 1) / 2), warps = gridDim.x * (kPrepThreads / 32);
+  const unsigned rounds = (pairs < warps ? 1u : pairs / warps) * warps;
+  for (unsigned q = blockIdx.x * (kPrepThreads / 32) + (threadIdx.x >> 5);;) {
+    if (q >= rounds || q >= pairs) {
+      if (rounds >= pairs) break;
+      if ((threadIdx.x & 31) == 0) q = rounds + atomicAdd(&L.cnt->next, 1u);
+      q = __shfl_sync(kFull, q, 0);
+      if (q >= pairs) break;
+    }
+    const long long p = 2ll * q + ((threadIdx.x >> 4) & 1);
+    sphere_pixel<CLOSED>(L, a, sh, 0, p, p < a.sc.P);
+    if (q < rounds) q += warps;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) sphere_counts(sh, L.bc_prep[blockIdx.x], L.bc_search[blockIdx.x]);
+}
+
+// The lists after the search, in one launch: what the sphere search left
+// (settle_entry, a warp per entry), near ties (resolve_entry) and the FP64
+// recheck list (recheck_entry), grid-stride over each; an entry that one
+// stage cannot settle goes on to the next with the same block.  The last
+// two entries' shared layouts overlap, so each restages its model constants
+// when the other ran last.
 static_assert(kResolveThreads == kRecheckThreads, "one block size for both lists");
-__global__ void __launch_bounds__(kResolveThreads) k_lists(GsLaunch L) {
+__global__ void __launch_bounds__(kResolveThreads)
+k_lists(const __grid_constant__ GsLaunch L) {
   __shared__ union ListShared {
     ResolveShared r;
     RecheckShared c;
   } S;
+  constexpr int kWarps = kResolveThreads / 32;
+  constexpr int kTodoRecheck = 1 << 30;  // beside the array's index (a batch has fewer)
+  __shared__ SettleScratch settle[kWarps];
+  __shared__ ListEntry todo[kWarps];
+  __shared__ int n_todo;
   int staged_r = -1, staged_c = -1;  // the array whose constants each layout holds
   if (!L.table) {  // one array: its model is known before the search ends
     stage_consts(&L.one.md->k, &S.r.cs);
@@ -137,13 +176,53 @@ __global__ void __launch_bounds__(kResolveThreads) k_lists(GsLaunch L) {
   if (pf) first = L.tie_list[blockIdx.x];
   const unsigned ntie = L.cnt->n_tie;
   const unsigned nflag = L.cnt->n_flag;
+  const unsigned nclose = L.cnt->n_close;
   unsigned my_res = 0, my_slmax = 0;
-  for (unsigned it = blockIdx.x; it < ntie + nflag; it += gridDim.x) {
-    ListEntry e = (pf && it == blockIdx.x && it < ntie)
-                      ? first
-                      : (it < ntie ? L.tie_list[it] : L.flag_list[it - ntie]);
+  // rounds of the close list (spread over the blocks first), then the two
+  // others; what a round of warps leaves, the block takes on before the next
+  const unsigned per = gridDim.x * kWarps, nlist = ntie + nflag;
+  const unsigned rounds = (nclose + per - 1) / per;
+  int at = 0, left = 0;
+#pragma unroll 1
+  for (unsigned r = 0, it = blockIdx.x;;) {
+    ListEntry e;
+    bool check;  // straight to the FP64 recheck
+    if (at < left) {
+      e = todo[at++];
+      check = (e.array & kTodoRecheck) != 0;
+      e.array &= ~kTodoRecheck;
+    } else if (r < rounds) {
+      __syncthreads();
+      if (threadIdx.x == 0) n_todo = 0;
+      __syncthreads();
+      const unsigned i = r * per + (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+      if (i < nclose) {
+        const CloseEntry ce = L.close_list[i];
+        const ArrayDesc& a = desc_of(L, ce.array);
+        const ModelConsts& cs = staged_r == ce.array ? S.r.cs : a.md->k;
+        const int next = a.mt.closed
+                             ? settle_entry<true>(L, a, cs, settle[threadIdx.x >> 5], ce, e)
+                             : settle_entry<false>(L, a, cs, settle[threadIdx.x >> 5], ce, e);
+        if (next && (threadIdx.x & 31) == 0) {
+          if (next == 2) e.array |= kTodoRecheck;
+          todo[atomicAdd(&n_todo, 1)] = e;
+        }
+      }
+      ++r;
+      __syncthreads();
+      at = 0;
+      left = n_todo;
+      continue;
+    } else if (it < nlist) {
+      e = (pf && it == blockIdx.x && it < ntie)
+              ? first
+              : (it < ntie ? L.tie_list[it] : L.flag_list[it - ntie]);
+      check = it >= ntie;
+      it += gridDim.x;
+    } else {
+      break;
+    }
     const ArrayDesc& a = desc_of(L, e.array);
-    bool check = it >= ntie;
     if (!check) {
       if (e.array != staged_r) {
         __syncthreads();
@@ -188,6 +267,8 @@ __global__ void __launch_bounds__(kResolveThreads) k_lists(GsLaunch L) {
     if (atomicAdd(&L.cnt->lists_done, 1u) == gridDim.x - 1) {
       L.cnt->n_flag = 0u;
       L.cnt->n_tie = 0u;
+      L.cnt->n_close = 0u;
+      L.cnt->next = 0u;
       L.cnt->lists_done = 0u;
     }
   }
@@ -228,6 +309,10 @@ cudaError_t launch_lists(const GsLaunch& L, cudaStream_t st) {
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+int sphere_blocks(const GsLaunch& L) {
+  const long long full = (L.one.sc.P + kSphereTeams - 1) / kSphereTeams;
+  return (int)std::min(full, (long long)L.num_sms * kSphereBlocks);
+}
 bool fused_tiles(const GsLaunch& L) {
   // a block preparing its own tile makes (prep_team / T) prep passes over it
   return L.one.prep_team <= 2 * L.one.cfg.T;
@@ -245,7 +330,11 @@ static cudaError_t run(const GsLaunch& L, cudaStream_t st) {
   // of its own, built for kBnbBlocks resident blocks per SM
   constexpr bool kBnb = bnb_search(L1, L2);
   const bool tf = L.one.cfg.T >= kTeamFinishMin;
-  if (fused_tiles(L)) {
+  if (L.one.sphere) {
+    k_sphere<CLOSED><<<sphere_blocks(L), kPrepThreads, 0, st>>>(L);
+    e = cudaGetLastError();
+    if (L.ev) cudaEventRecord(L.ev[1], st);
+  } else if (fused_tiles(L)) {
     if (L.ev) cudaEventRecord(L.ev[1], st);
     if (kBnb && tf)
       k_ground_state_bnb<CLOSED><<<search_blocks(L), kSearchThreads, 0, st>>>(L);

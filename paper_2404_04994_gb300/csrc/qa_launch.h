@@ -30,6 +30,7 @@ struct ArrayDesc {
   float bx_analytic;   // decision margin for double-float continuous minima
   float bx_qp_scale;   // ... per unit of (1 + max|c| + N_hat) for FP32 QP minima
   PixRec* recs;        // scratch [P]
+  int sphere;          // the sphere search instead of the FP32 search
   int8_t* out_n;
   int16_t* out_n16;    // int16 charge map instead of out_n when non-null
   double* out_U;
@@ -43,6 +44,7 @@ constexpr int kTeamFinishMin = 8;    // teams at least this wide finish the winn
 constexpr int kBnbL1 = 5, kBnbL2 = 2;
 constexpr int kBnbMinT = 16;
 constexpr int kBnbBlocks = 5;  // resident blocks per SM its kernels are built for
+constexpr int kSphereBlocks = 8;  // resident blocks per SM the sphere search's kernels are built for
 // Batched search kernel variants: 4 per split class (closed, team finish).
 constexpr int kBatchVariants = 20;
 static_assert(sizeof(((Counters*)nullptr)->q_var) / sizeof(unsigned) == kBatchVariants,
@@ -67,6 +69,7 @@ struct GsLaunch {
   int n_search_units;
   ListEntry* flag_list;        // scratch: pixels for the FP64 recheck
   ListEntry* tie_list;         // scratch: near-tie pixels for the list kernel's resolve
+  CloseEntry* close_list;      // scratch: pixels the sphere search left to the list kernel
   Counters* cnt;               // scratch; list heads zero at the start of each call
   BlockCounts* bc_prep;        // scratch [prep blocks]
   BlockCounts* bc_search;      // scratch [search blocks]
@@ -129,6 +132,7 @@ cudaError_t launch_prep(const GsLaunch& a, cudaStream_t st);
 cudaError_t launch_lists(const GsLaunch& a, cudaStream_t st);
 int prep_blocks(const GsLaunch& a);
 int search_blocks(const GsLaunch& a);
+int sphere_blocks(const GsLaunch& a);  // the sphere search's grid
 // true: one kernel prepares and searches each tile (block counts of both
 // stages per search block); false: k_prep then k_search
 bool fused_tiles(const GsLaunch& a);

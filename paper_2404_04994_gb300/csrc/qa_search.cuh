@@ -236,7 +236,9 @@ __device__ __forceinline__ float state_from_scratch(const float* sM,
 // sum min(0, g_m) + qneg (qneg: the model's bound of any pair-term sum, so
 // the bound holds for every candidate of the pattern) lies above lb_cut
 // holds no block to collect and is skipped.
-template <int L1, int L2, bool CLOSED, bool COLLECT, bool BLOCKS = false, int LANEBITS = 8>
+// ONLY: of the blocks just those in only[0 .. n_only) (n_only < 0: all).
+template <int L1, int L2, bool CLOSED, bool COLLECT, bool BLOCKS = false, int LANEBITS = 8,
+          bool ONLY = false>
 __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
                                             const SlotView sv, int t, int T,
                                             float thr, unsigned* blist,
@@ -246,7 +248,8 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
                                             const float* __restrict__ colt = nullptr,
                                             const float* __restrict__ itab = nullptr,
                                             float* __restrict__ cslot = nullptr,
-                                            float lb_cut = kInf, float qneg = 0.f) {
+                                            float lb_cut = kInf, float qneg = 0.f,
+                                            const unsigned* only = nullptr, int n_only = 0) {
   static_assert(L1 >= 2 && L1 <= 6 && L2 >= 0 && L2 <= 5, "search split");
   // block-level searches with at least 9 inner + middle slots take the
   // iteration slots' terms from the team table itab (iter_build): at most 7
@@ -377,6 +380,11 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
 
   for (unsigned it = 0; it < niter; ++it) {
     const unsigned o = (unsigned)t | (it << nlb);
+    if (ONLY && n_only >= 0) {
+      bool on = false;
+      for (int e = 0; e < n_only; ++e) on = on || (only[e] >> L2) == o;
+      if (!on) continue;
+    }
     float A = At;
     float q[L1 > 0 ? L1 : 1];
     float gm[L2 > 0 ? L2 : 1];
@@ -463,6 +471,11 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
             q[j] = up ? q[j] + Mim[j][mb] : q[j] - Mim[j][mb];
         }
       }
+      if (ONLY && n_only >= 0) {
+        bool on = false;
+        for (int e = 0; e < n_only; ++e) on = on || only[e] == (obase | gray_c((unsigned)s));
+        if (!on) continue;
+      }
       float mbk;
       if (!CLOSED) {
         mbk = inner_min_open<L1>(A, q, P);
@@ -528,14 +541,15 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
 // (at 1 + L1 + m).  Team-cooperative (lane lt of T); sync after.
 template <int L1, int L2>
 __device__ __forceinline__ void iter_build(const float* sM, const SlotView& sv, int lt, int T,
-                                           float* itab) {
+                                           float* itab, int step = 0) {
   const int k = sv.k;
   const int nmid = min(max(k - L1, 0), L2);
   const int nout = max(k - L1 - L2, 0);
   const int nlb = min(__ffs(T) - 1, nout);
   const int nit = nout - nlb;
   const int s0 = L1 + L2 + nlb;  // the first iteration slot
-  for (int e = lt; e < (1 << nit) * kItStride; e += T) {
+  if (step == 0) step = T;  // the lanes that build it
+  for (int e = lt; e < (1 << nit) * kItStride; e += step) {
     const unsigned it = (unsigned)(e / kItStride);
     const int v = e % kItStride;
     float acc = 0.f;

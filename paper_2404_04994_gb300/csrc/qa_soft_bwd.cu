@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
     if (tid == 0) {
       md->status = 1;
       md->k.model_bad = 1;
+      md->s.valid = 0;
     }
     return;
   }
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
       kc.qneg = qn;
       kc.pad2[0] = kc.pad2[1] = 0;
       kc.model_bad = 0;
+      md->s.valid = 0;  // the sphere search's factor is the host's
       kc.pad = 0;
     }
   }
