@@ -1375,6 +1375,8 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
     if (qa::bnb_search(d.cfg.L1, d.cfg.L2) && d.cfg.T < qa::kBnbMinT)
       d.cfg.T = qa::kBnbMinT;
     d.klass = qa::search_klass(d.cfg);
+    d.sphere = !m->host_stale && m->host.s.valid &&
+               use_sphere(m->n, it.threshold, 1LL << 40, it.closed != 0, d.cfg);
     d.prep_team = prep_team(m->n);
     d.bx_analytic = 4.0e-7f;
     d.bx_qp_scale = 0.f;
@@ -1396,16 +1398,45 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   qa::batch_occupancy(&pps, &sps);
   const double unit_target = 8.0;  // units per resident block
   double total_cost = 0.0;
-  for (int i = 0; i < count; ++i) total_cost += unit_cost(table[(size_t)i]) * (double)b->P[(size_t)i];
+  long long tile_pixels = 0, sphere_pixels = 0;
+  for (int i = 0; i < count; ++i) {
+    if (table[(size_t)i].sphere) {
+      sphere_pixels += b->P[(size_t)i];
+      continue;
+    }
+    tile_pixels += b->P[(size_t)i];
+    total_cost += unit_cost(table[(size_t)i]) * (double)b->P[(size_t)i];
+  }
   const long long prep_share =
-      (long long)std::ceil((double)b->pixels / (unit_target * b->num_sms * pps));
+      (long long)std::ceil((double)tile_pixels / (unit_target * b->num_sms * pps));
+  // sphere search: units of 8 to 256 pixels
+  const int sphere_full = b->num_sms * qa::kSphereBlocks;
+  const long long sphere_chunk =
+      std::min(256LL, std::max(8LL, sphere_pixels / (16LL * sphere_full) / 8 * 8));
+  // ... and at least two units per resident block of each variant, so that one
+  // with few or cheap pixels fills the chip, too (the 2-dot arrays of a batch
+  // of 192 ran on 110 blocks, 49 us for 3.5 M warp instructions)
   const double search_share =
       std::min(262144.0, std::max(16384.0, total_cost / (unit_target * b->num_sms * sps)));
-  std::vector<qa::WorkUnit> pu, su;
+  auto variant_of = [](const qa::ArrayDesc& d) {
+    return 4 * d.klass + 2 * (d.mt.closed ? 1 : 0) + (d.cfg.T >= qa::kTeamFinishMin ? 1 : 0);
+  };
+  long long var_tiles[qa::kBatchVariants] = {};
+  for (int i = 0; i < count; ++i)
+    if (!table[(size_t)i].sphere) {
+      const qa::ArrayDesc& d = table[(size_t)i];
+      var_tiles[variant_of(d)] += b->P[(size_t)i] * d.cfg.T / 128 + 1;
+    }
+  std::vector<qa::WorkUnit> pu, su, xu, xc;
   std::vector<double> scost;
   for (int i = 0; i < count; ++i) {
     const qa::ArrayDesc& d = table[(size_t)i];
     const long long P = b->P[(size_t)i];
+    if (d.sphere) {
+      for (long long f = 0; f < P; f += sphere_chunk)
+        (d.mt.closed ? xc : xu).push_back({i, (int)std::min(sphere_chunk, P - f), f});
+      continue;
+    }
     const long long tpb = 128 / d.prep_team;
     const long long pchunk = std::max(tpb, std::min(4096LL / tpb, (prep_share + tpb - 1) / tpb) * tpb);
     for (long long f = 0; f < P; f += pchunk)
@@ -1413,7 +1444,9 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
     const long long teams = 128 / d.cfg.T;
     const double c = unit_cost(d);
     long long k = (long long)std::max(1.0, std::floor(search_share / (c * (double)teams)));
-    k = std::min(k, 64LL);
+    const int v = variant_of(d);
+    k = std::min(k, std::max(1LL, std::min(64LL, var_tiles[v] / (2LL * b->num_sms *
+                                                                  qa::batch_search_occupancy(v)))));
     const long long schunk = teams * k;
     for (long long f = 0; f < P; f += schunk) {
       const long long cnt = std::min(schunk, P - f);
@@ -1424,8 +1457,7 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   // group the search units by kernel variant (4 klass + 2 closed + team
   // finish), largest first within a group; one persistent grid per variant
   auto variant = [&](const qa::WorkUnit& w) {
-    const qa::ArrayDesc& d = table[(size_t)w.array];
-    return 4 * d.klass + 2 * (d.mt.closed ? 1 : 0) + (d.cfg.T >= qa::kTeamFinishMin ? 1 : 0);
+    return variant_of(table[(size_t)w.array]);
   };
   std::vector<size_t> order(su.size());
   for (size_t i = 0; i < order.size(); ++i) order[i] = i;
@@ -1454,11 +1486,18 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   const size_t off_tab = align_up(sizeof(qa::Counters), 256);
   const size_t off_pu = align_up(off_tab + sizeof(qa::ArrayDesc) * (size_t)count, 256);
   const size_t off_su = align_up(off_pu + sizeof(qa::WorkUnit) * pu.size(), 256);
-  const size_t off_fl = align_up(off_su + sizeof(qa::WorkUnit) * su_sorted.size(), 256);
+  const int nsph[2] = {(int)xu.size(), (int)xc.size()};
+  xu.insert(xu.end(), xc.begin(), xc.end());
+  const int grid_sphere = std::min(sphere_full, nsph[0]) + std::min(sphere_full, nsph[1]);
+  const size_t off_xu = align_up(off_su + sizeof(qa::WorkUnit) * su_sorted.size(), 256);
+  const size_t off_fl = align_up(off_xu + sizeof(qa::WorkUnit) * xu.size(), 256);
   const size_t off_tl = align_up(off_fl + sizeof(qa::ListEntry) * Ptot, 256);
-  const size_t off_bcp = align_up(off_tl + sizeof(qa::ListEntry) * Ptot, 256);
-  const size_t off_bcs = align_up(off_bcp + sizeof(qa::BlockCounts) * (size_t)grid_prep, 256);
-  const size_t off_rec = align_up(off_bcs + sizeof(qa::BlockCounts) * (size_t)grid_search, 256);
+  const size_t off_cl = align_up(off_tl + sizeof(qa::ListEntry) * Ptot, 256);
+  const size_t off_bcp = align_up(off_cl + sizeof(qa::CloseEntry) * (size_t)sphere_pixels, 256);
+  const size_t off_bcs = align_up(
+      off_bcp + sizeof(qa::BlockCounts) * (size_t)(grid_prep + grid_sphere), 256);
+  const size_t off_rec = align_up(
+      off_bcs + sizeof(qa::BlockCounts) * (size_t)(grid_search + grid_sphere), 256);
   const size_t total = off_rec + sizeof(qa::PixRec) * Ptot;
   cudaError_t e = cudaMalloc(&b->mem, total);
   if (e != cudaSuccess) {
@@ -1478,6 +1517,10 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   if (e == cudaSuccess && !su_sorted.empty())
     e = cudaMemcpy(mem + off_su, su_sorted.data(), sizeof(qa::WorkUnit) * su_sorted.size(),
                    cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && !xu.empty())
+    e = cudaMemcpy(mem + off_xu, xu.data(), sizeof(qa::WorkUnit) * xu.size(), cudaMemcpyHostToDevice);
+  // (block counts of a grid that the batch does not launch read as zero)
+  if (e == cudaSuccess) e = cudaMemset(mem + off_bcp, 0, off_rec - off_bcp);
   if (e != cudaSuccess) {
     cudaFree(b->mem);
     delete b;
@@ -1490,6 +1533,14 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   L.n_prep_units = (int)pu.size();
   L.search_units = (const qa::WorkUnit*)(mem + off_su);
   L.n_search_units = (int)su_sorted.size();
+  L.sphere_units = (const qa::WorkUnit*)(mem + off_xu);
+  for (int f = 0; f < 2; ++f) {
+    L.sphere_first[f] = f ? nsph[0] : 0;
+    L.sphere_count[f] = nsph[f];
+    L.sphere_grid[f] = std::min(sphere_full, nsph[f]);
+    L.sphere_bc[f] = f ? L.sphere_grid[0] : 0;
+  }
+  L.close_list = (qa::CloseEntry*)(mem + off_cl);
   L.flag_list = (qa::ListEntry*)(mem + off_fl);
   L.tie_list = (qa::ListEntry*)(mem + off_tl);
   L.cnt = (qa::Counters*)(mem + off_cnt);
@@ -1526,7 +1577,8 @@ int qa_batch_stats(qa_batch* b, void* stream, qa_stats* out) {
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
   qa::Counters c;
   if (e == cudaSuccess) e = cudaMemcpy(&c, b->L.cnt, sizeof(c), cudaMemcpyDeviceToHost);
-  std::vector<qa::BlockCounts> bp((size_t)b->L.grid_prep), bs((size_t)b->L.grid_search);
+  const int gs = b->L.sphere_grid[0] + b->L.sphere_grid[1];
+  std::vector<qa::BlockCounts> bp((size_t)(b->L.grid_prep + gs)), bs((size_t)(b->L.grid_search + gs));
   if (e == cudaSuccess)
     e = cudaMemcpy(bp.data(), b->L.bc_prep, sizeof(qa::BlockCounts) * bp.size(), cudaMemcpyDeviceToHost);
   if (e == cudaSuccess)

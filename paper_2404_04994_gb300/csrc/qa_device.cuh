@@ -177,7 +177,7 @@ struct Counters {
   unsigned int n_close; // length of the close list
   unsigned int next;    // single array: the sphere search's work queue
   unsigned int q_prep;  // batched launch: work-queue heads
-  unsigned int q_search;
+  unsigned int q_sphere[2];  // ... the sphere search's, open and closed
   unsigned int q_var[20];  // batched launch: the search queue of each kernel variant
   unsigned int lists_done; // blocks of the list kernel that have finished
   unsigned int soft_done;  // blocks of the soft gradient reduction that have finished
@@ -208,12 +208,14 @@ struct ListEntry {
 };
 
 // A pixel the sphere search could not settle: the candidates within its
-// margin (nl of them, two to four; patterns over the dots), or none (nl = 0).
+// margin (nl of them, two to kCloseMax; 16-bit patterns over the dots, two to
+// a word), or none (nl = 0).
+constexpr int kCloseMax = 8;
 struct CloseEntry {
   int array;
   int p;
-  unsigned pat01, pat23;
   int nl;
+  unsigned pat[kCloseMax / 2];
 };
 
 // Copy the model's FP32 constants into shared memory (16-byte vectors).

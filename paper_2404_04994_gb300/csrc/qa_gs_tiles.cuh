@@ -1116,19 +1116,25 @@ __device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, Spher
       &sh.p.qx[tq], &sh.p.qz[tq], sh.lev[team], reinterpret_cast<uint2*>(&sh.p.qK[tq][0]), close,
       ev);
   const bool done = active && close == 1;
-  // candidates too close to tell apart (up to four): left, with their patterns
-  // over the dots, to the list kernel; so is a search that did not end
+  // candidates too close to tell apart: left, with their patterns over the
+  // dots, to the list kernel; so is a search that did not end
   if (__any_sync(kFull, active && close != 1)) {
     const unsigned* lst = reinterpret_cast<const unsigned*>(&sh.p.qz[tq]);
-    unsigned pat[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      pat[e] = (__ballot_sync(kFull, lt < n && e < close && ((lst[e] >> sh.m.pos[lt]) & 1u)) >> hw) &
-               0xffffu;
-    if (active && close != 1 && lt == 0) {
-      const unsigned at = atomicAdd(&L.cnt->n_close, 1u);
-      L.close_list[at] = CloseEntry{array, (int)p, pat[0] | (pat[1] << 16), pat[2] | (pat[3] << 16),
-                                    close <= 4 ? close : 0};
+    const bool leave = active && close != 1 && lt == 0;
+    CloseEntry* ce = nullptr;
+    if (leave) {
+      ce = L.close_list + atomicAdd(&L.cnt->n_close, 1u);
+      ce->array = array;
+      ce->p = (int)p;
+      ce->nl = close <= kCloseMax ? close : 0;
+    }
+#pragma unroll 1
+    for (int e = 0; e < kCloseMax; e += 2) {
+      const unsigned b0 = __ballot_sync(
+          kFull, lt < n && e < close && ((lst[e] >> sh.m.pos[lt]) & 1u));
+      const unsigned b1 = __ballot_sync(
+          kFull, lt < n && e + 1 < close && ((lst[e + 1] >> sh.m.pos[lt]) & 1u));
+      if (leave) ce->pat[e >> 1] = ((b0 >> hw) & 0xffffu) | (((b1 >> hw) & 0xffffu) << 16);
     }
     __syncwarp();
   }
@@ -1259,7 +1265,7 @@ __device__ __forceinline__ float bnb_block_min(const float* pm, const float* vv,
 struct SettleScratch {
   int sdot[kMaxDot];
   float sh[kMaxDot];
-  unsigned lst[4];
+  unsigned lst[kCloseMax];
   float rhi[2][kMaxDot], rlo[2][kMaxDot];
   union {
     struct {
@@ -1418,10 +1424,10 @@ __device__ inline int settle_entry(const GsLaunch& L, const ArrayDesc& a, const 
       bbits = b;
     }
   };
-  auto pattern = [&](int i) { return ((i < 2 ? ce.pat01 : ce.pat23) >> (16 * (i & 1))) & 0xffffu; };
+  auto pattern = [&](int i) { return (ce.pat[i >> 1] >> (16 * (i & 1))) & 0xffffu; };
 #pragma unroll 1
   for (int i = 0; i < nl; i += 2) {
-    const unsigned b = pattern(i + half);
+    const unsigned b = pattern(i + half);  // (zero past the list)
     const df u = team_energy(cs, n, lt, kFull, live, base + (int)((b >> lt) & 1u), c, t.rhi[half],
                              t.rlo[half]);
     const unsigned sb =

@@ -160,7 +160,7 @@ k_lists(const __grid_constant__ GsLaunch L) {
   constexpr int kWarps = kResolveThreads / 32;
   constexpr int kTodoRecheck = 1 << 30;  // beside the array's index (a batch has fewer)
   __shared__ SettleScratch settle[kWarps];
-  __shared__ ListEntry todo[kWarps];
+  __shared__ ListEntry todo[4 * kWarps];
   __shared__ int n_todo;
   int staged_r = -1, staged_c = -1;  // the array whose constants each layout holds
   if (!L.table) {  // one array: its model is known before the search ends
@@ -178,26 +178,27 @@ k_lists(const __grid_constant__ GsLaunch L) {
   const unsigned nflag = L.cnt->n_flag;
   const unsigned nclose = L.cnt->n_close;
   unsigned my_res = 0, my_slmax = 0;
-  // rounds of the close list (spread over the blocks first), then the two
-  // others; what a round of warps leaves, the block takes on before the next
+  // the close list, each warp its entries (spread over the blocks first), then
+  // the two others; what the warps leave, the block takes on (todo: before it
+  // could overflow)
   const unsigned per = gridDim.x * kWarps, nlist = ntie + nflag;
-  const unsigned rounds = (nclose + per - 1) / per;
+  unsigned ci = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  bool more = blockIdx.x < nclose;
   int at = 0, left = 0;
 #pragma unroll 1
-  for (unsigned r = 0, it = blockIdx.x;;) {
+  for (unsigned it = blockIdx.x;;) {
     ListEntry e;
     bool check;  // straight to the FP64 recheck
     if (at < left) {
       e = todo[at++];
       check = (e.array & kTodoRecheck) != 0;
       e.array &= ~kTodoRecheck;
-    } else if (r < rounds) {
+    } else if (more) {
       __syncthreads();
       if (threadIdx.x == 0) n_todo = 0;
       __syncthreads();
-      const unsigned i = r * per + (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-      if (i < nclose) {
-        const CloseEntry ce = L.close_list[i];
+      for (int q = 0; q < 4 && ci < nclose; ++q, ci += per) {
+        const CloseEntry& ce = L.close_list[ci];
         const ArrayDesc& a = desc_of(L, ce.array);
         const ModelConsts& cs = staged_r == ce.array ? S.r.cs : a.md->k;
         const int next = a.mt.closed
@@ -208,8 +209,7 @@ k_lists(const __grid_constant__ GsLaunch L) {
           todo[atomicAdd(&n_todo, 1)] = e;
         }
       }
-      ++r;
-      __syncthreads();
+      more = __syncthreads_or(ci < nclose) != 0;
       at = 0;
       left = n_todo;
       continue;

@@ -67,6 +67,11 @@ struct GsLaunch {
   int n_prep_units;
   const WorkUnit* search_units;
   int n_search_units;
+  // ... of the arrays that take the sphere search, open ones first: units
+  // [sphere_first, sphere_first + sphere_count) of each form, its grid, and
+  // its block counts from grid_prep (grid_search) + sphere_bc
+  const WorkUnit* sphere_units;
+  int sphere_first[2], sphere_count[2], sphere_grid[2], sphere_bc[2];
   ListEntry* flag_list;        // scratch: pixels for the FP64 recheck
   ListEntry* tie_list;         // scratch: near-tie pixels for the list kernel's resolve
   CloseEntry* close_list;      // scratch: pixels the sphere search left to the list kernel
