@@ -137,7 +137,12 @@ void fill_sphere(int n, qa::ModelData* md) {
   qa::SphereConsts& s = md->s;
   std::memset(&s, 0, sizeof(s));
   for (int i = 0; i < qa::kMaxDot; ++i) s.ord[i] = s.pos[i] = (unsigned char)i;
-  if (n < qa::kSphereMinDot) return;
+  double msum = 0.0;
+  for (int e = 0; e < n * n; ++e) msum += std::fabs(md->M[e]);
+  s.msum = (float)(msum * (1.0 + 1e-6));
+  s.valid = std::isfinite(s.msum);
+  if (n < qa::kSphereMinDot || !s.valid) return;
+  s.valid = 0;
   double A[qa::kMaxDot][qa::kMaxDot], L[qa::kMaxDot][qa::kMaxDot] = {}, W[qa::kMaxDot][qa::kMaxDot] = {};
   for (int i = 0; i < n; ++i)
     for (int j = 0; j < n; ++j) A[i][j] = md->Cdd[i * n + j];
@@ -157,7 +162,7 @@ void fill_sphere(int n, qa::ModelData* md) {
     for (int i = k + 1; i < n; ++i)
       for (int j = k + 1; j <= i; ++j) A[i][j] = A[j][i] = A[i][j] - L[i][k] * L[j][k];
   }
-  double ysq = 0.0, msum = 0.0;
+  double ysq = 0.0;
   for (int k = 0; k < n; ++k) {
     W[k][k] = std::sqrt(0.5) / L[k][k];
     for (int j = k - 1; j >= 0; --j) {
@@ -170,12 +175,10 @@ void fill_sphere(int n, qa::ModelData* md) {
     ysq += y * y;
     for (int j = 0; j < k; ++j) s.W[k][j] = (float)W[k][j];
     s.wd[k] = (float)W[k][k];
-    for (int j = 0; j < n; ++j) msum += std::fabs(md->M[k * n + j]);
   }
   for (int k = 0; k < n; ++k) s.pos[s.ord[k]] = (unsigned char)k;
   s.ysq = (float)(ysq * (1.0 + 1e-6));
-  s.msum = (float)(msum * (1.0 + 1e-6));
-  s.valid = std::isfinite(s.ysq) && std::isfinite(s.msum);
+  s.valid = std::isfinite(s.ysq);
 }
 
 // FP32 / double-float forms of the model used by every kernel.
@@ -448,27 +451,43 @@ qa::RasterK raster_constants(const qa_model* m, const qa::Scan& sc) {
 // while the sphere search's few close pixels take a longer list kernel, so
 // there the line is 13 dots (100 x 100: 12 dots 33 / 45, 13 dots 41 / 41, 14
 // dots 53 / 49, 16 dots 58 / 43; closed 12 dots 60 / 53).
-bool use_sphere(int n, double t, long long P, bool closed, const qa::SearchCfg& cfg) {
-  const double kexp = t >= 1.0 ? (double)n : (double)n * std::log2(1.0 + t);
+bool use_sphere(int n, double kexp, long long P, bool closed, const qa::SearchCfg& cfg) {
   return n >= qa::kSphereMinDot && cfg.T >= qa::kTeamFinishMin && cfg.L1 == 5 &&
          kexp >= (closed || P >= 30000 ? 11.01 : 12.6);
-}
-
-// The sphere search of a single-array call whose other fields are set: its
-// close list takes the block counts' room beyond the grid's entries (at most
-// ceil(P / 8) of P + 1).
-void set_sphere(const qa_model* m, qa::GsLaunch* a) {
-  static_assert(7 * sizeof(qa::BlockCounts) >= 8 * sizeof(qa::CloseEntry),
-                "eight pixels' entries in seven unused counts");
-  a->one.sphere = !m->host_stale && m->host.s.valid &&
-                  use_sphere(m->n, a->one.mt.t, a->one.sc.P, a->one.mt.closed != 0, a->one.cfg);
-  a->close_list = reinterpret_cast<qa::CloseEntry*>(a->bc_prep + qa::sphere_blocks(*a));
 }
 
 int prep_team(int n) {
   int t = 1;
   while (t < n) t <<= 1;
   return t;
+}
+
+// The search of an array whose other fields are set (P: the pixels that decide
+// how full the GPU is).
+int choose_search(const qa_model* m, const qa::ArrayDesc& d, long long P) {
+  if (m->host_stale || !m->host.s.valid) return qa::kSearchTiles;
+  const int n = m->n;
+  const double t = d.mt.t;
+  const bool closed = d.mt.closed != 0;
+  // (a closed array at t = 0 takes t = 1 wherever its set misses the total)
+  const double kexp = t >= 1.0 || (closed && t <= 0.0) ? (double)n : (double)n * std::log2(1.0 + t);
+  if (use_sphere(n, kexp, P, closed, d.cfg)) return qa::kSearchSphere;
+  // the list kernel repeats the sums of these configurations of the FP32 search
+  const bool listed = d.cfg.L1 >= 4 && (d.cfg.T < qa::kTeamFinishMin || d.cfg.L2 == 4);
+  if (n < 3 || !listed) return qa::kSearchTiles;
+  if (n <= 8) return qa::kSearchDense;
+  if (n < 12) return kexp < (closed ? 9.5 : 8.9) ? qa::kSearchDense : qa::kSearchTiles;
+  if (closed) return kexp < 11.01 || t <= 0.0 ? qa::kSearchMixed : qa::kSearchTiles;
+  return kexp < (P >= 30000 ? 9.4 : 4.6) ? qa::kSearchMixed : qa::kSearchTiles;
+}
+
+// The same for a single-array call; its close list takes the block counts' room
+// beyond the grid's entries (at most ceil(P / 8) of P + 1).
+void set_search(const qa_model* m, qa::GsLaunch* a) {
+  static_assert(7 * sizeof(qa::BlockCounts) >= 8 * sizeof(qa::CloseEntry),
+                "eight pixels' entries in seven unused counts");
+  a->one.search = choose_search(m, a->one, a->one.sc.P);
+  a->close_list = reinterpret_cast<qa::CloseEntry*>(a->bc_prep + qa::pixel_blocks(*a));
 }
 
 struct ScanIn {
@@ -619,7 +638,7 @@ int run_ground_state(qa_model* m, const ScanIn& in, double t, int closed,
   a.bc_search = m->d_bc_search;
   a.cnt = m->d_cnt;
   a.num_sms = m->num_sms;
-  set_sphere(m, &a);
+  set_search(m, &a);
   a.one.out_n = out_n;
   a.one.out_n16 = out_n16;
   a.one.out_U = out_U;
@@ -628,8 +647,8 @@ int run_ground_state(qa_model* m, const ScanIn& in, double t, int closed,
   m->last_P = P;
   a.ev = m->timing ? m->ev : nullptr;
   m->last_kind = 1;
-  if (a.one.sphere) {
-    m->n_bc_prep = m->n_bc_search = qa::sphere_blocks(a);
+  if (a.one.search != qa::kSearchTiles) {
+    m->n_bc_prep = m->n_bc_search = qa::pixel_blocks(a);
   } else {
     m->n_bc_prep = qa::fused_tiles(a) ? qa::search_blocks(a) : qa::prep_blocks(a);
     m->n_bc_search = qa::search_blocks(a);
@@ -1300,7 +1319,7 @@ extern "C" int qa_ground_state_open_static(qa_model* m, const qa_raster* r,
   a.bc_search = (qa::BlockCounts*)(ws + kStOffBcs);
   a.cnt = cnt;
   a.num_sms = m->num_sms;
-  set_sphere(m, &a);
+  set_search(m, &a);
   a.one.out_n = out_n;
   a.one.out_U = out_U;
   a.one.out_flags = out_flags;
@@ -1375,8 +1394,7 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
     if (qa::bnb_search(d.cfg.L1, d.cfg.L2) && d.cfg.T < qa::kBnbMinT)
       d.cfg.T = qa::kBnbMinT;
     d.klass = qa::search_klass(d.cfg);
-    d.sphere = !m->host_stale && m->host.s.valid &&
-               use_sphere(m->n, it.threshold, 1LL << 40, it.closed != 0, d.cfg);
+    d.search = choose_search(m, d, 1LL << 40);
     d.prep_team = prep_team(m->n);
     d.bx_analytic = 4.0e-7f;
     d.bx_qp_scale = 0.f;
@@ -1398,21 +1416,29 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   qa::batch_occupancy(&pps, &sps);
   const double unit_target = 8.0;  // units per resident block
   double total_cost = 0.0;
-  long long tile_pixels = 0, sphere_pixels = 0;
+  // one-pass arrays: by variant (search and team width, form)
+  auto pixel_variant = [](const qa::ArrayDesc& d) {
+    const int w = d.search == qa::kSearchSphere  ? 0
+                  : d.search == qa::kSearchMixed ? 1
+                  : d.prep_team == 16            ? 2
+                  : d.prep_team == 8             ? 3
+                                                 : 4;
+    return 2 * w + (d.mt.closed ? 1 : 0);
+  };
+  long long tile_pixels = 0, one_pass = 0, var_pixels[qa::kPixelVariants] = {};
   for (int i = 0; i < count; ++i) {
-    if (table[(size_t)i].sphere) {
-      sphere_pixels += b->P[(size_t)i];
+    const qa::ArrayDesc& d = table[(size_t)i];
+    if (d.search != qa::kSearchTiles) {
+      one_pass += b->P[(size_t)i];
+      var_pixels[pixel_variant(d)] += b->P[(size_t)i];
       continue;
     }
     tile_pixels += b->P[(size_t)i];
-    total_cost += unit_cost(table[(size_t)i]) * (double)b->P[(size_t)i];
+    total_cost += unit_cost(d) * (double)b->P[(size_t)i];
   }
   const long long prep_share =
       (long long)std::ceil((double)tile_pixels / (unit_target * b->num_sms * pps));
-  // sphere search: units of 8 to 256 pixels
-  const int sphere_full = b->num_sms * qa::kSphereBlocks;
-  const long long sphere_chunk =
-      std::min(256LL, std::max(8LL, sphere_pixels / (16LL * sphere_full) / 8 * 8));
+  const int pixel_full = b->num_sms * qa::kPixelBlocks;
   // ... and at least two units per resident block of each variant, so that one
   // with few or cheap pixels fills the chip, too (the 2-dot arrays of a batch
   // of 192 ran on 110 blocks, 49 us for 3.5 M warp instructions)
@@ -1423,18 +1449,23 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   };
   long long var_tiles[qa::kBatchVariants] = {};
   for (int i = 0; i < count; ++i)
-    if (!table[(size_t)i].sphere) {
+    if (table[(size_t)i].search == qa::kSearchTiles) {
       const qa::ArrayDesc& d = table[(size_t)i];
       var_tiles[variant_of(d)] += b->P[(size_t)i] * d.cfg.T / 128 + 1;
     }
-  std::vector<qa::WorkUnit> pu, su, xu, xc;
+  std::vector<qa::WorkUnit> pu, su, xu, xv[qa::kPixelVariants];
   std::vector<double> scost;
   for (int i = 0; i < count; ++i) {
     const qa::ArrayDesc& d = table[(size_t)i];
     const long long P = b->P[(size_t)i];
-    if (d.sphere) {
-      for (long long f = 0; f < P; f += sphere_chunk)
-        (d.mt.closed ? xc : xu).push_back({i, (int)std::min(sphere_chunk, P - f), f});
+    if (d.search != qa::kSearchTiles) {
+      // units of 2 to 32 rounds of a block's teams, sixteen to a resident block
+      const int v = pixel_variant(d);
+      const long long teams = 128 / d.prep_team;
+      const long long chunk =
+          teams * std::min(32LL, std::max(2LL, var_pixels[v] / (16LL * pixel_full * teams)));
+      for (long long f = 0; f < P; f += chunk)
+        xv[v].push_back({i, (int)std::min(chunk, P - f), f});
       continue;
     }
     const long long tpb = 128 / d.prep_team;
@@ -1486,18 +1517,22 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   const size_t off_tab = align_up(sizeof(qa::Counters), 256);
   const size_t off_pu = align_up(off_tab + sizeof(qa::ArrayDesc) * (size_t)count, 256);
   const size_t off_su = align_up(off_pu + sizeof(qa::WorkUnit) * pu.size(), 256);
-  const int nsph[2] = {(int)xu.size(), (int)xc.size()};
-  xu.insert(xu.end(), xc.begin(), xc.end());
-  const int grid_sphere = std::min(sphere_full, nsph[0]) + std::min(sphere_full, nsph[1]);
+  int pix_first[qa::kPixelVariants], pix_grid[qa::kPixelVariants], grid_pixel = 0;
+  for (int v = 0; v < qa::kPixelVariants; ++v) {
+    pix_first[v] = (int)xu.size();
+    xu.insert(xu.end(), xv[v].begin(), xv[v].end());
+    pix_grid[v] = std::min(pixel_full, (int)xv[v].size());
+    grid_pixel += pix_grid[v];
+  }
   const size_t off_xu = align_up(off_su + sizeof(qa::WorkUnit) * su_sorted.size(), 256);
   const size_t off_fl = align_up(off_xu + sizeof(qa::WorkUnit) * xu.size(), 256);
   const size_t off_tl = align_up(off_fl + sizeof(qa::ListEntry) * Ptot, 256);
   const size_t off_cl = align_up(off_tl + sizeof(qa::ListEntry) * Ptot, 256);
-  const size_t off_bcp = align_up(off_cl + sizeof(qa::CloseEntry) * (size_t)sphere_pixels, 256);
+  const size_t off_bcp = align_up(off_cl + sizeof(qa::CloseEntry) * (size_t)one_pass, 256);
   const size_t off_bcs = align_up(
-      off_bcp + sizeof(qa::BlockCounts) * (size_t)(grid_prep + grid_sphere), 256);
+      off_bcp + sizeof(qa::BlockCounts) * (size_t)(grid_prep + grid_pixel), 256);
   const size_t off_rec = align_up(
-      off_bcs + sizeof(qa::BlockCounts) * (size_t)(grid_search + grid_sphere), 256);
+      off_bcs + sizeof(qa::BlockCounts) * (size_t)(grid_search + grid_pixel), 256);
   const size_t total = off_rec + sizeof(qa::PixRec) * Ptot;
   cudaError_t e = cudaMalloc(&b->mem, total);
   if (e != cudaSuccess) {
@@ -1533,12 +1568,13 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
   L.n_prep_units = (int)pu.size();
   L.search_units = (const qa::WorkUnit*)(mem + off_su);
   L.n_search_units = (int)su_sorted.size();
-  L.sphere_units = (const qa::WorkUnit*)(mem + off_xu);
-  for (int f = 0; f < 2; ++f) {
-    L.sphere_first[f] = f ? nsph[0] : 0;
-    L.sphere_count[f] = nsph[f];
-    L.sphere_grid[f] = std::min(sphere_full, nsph[f]);
-    L.sphere_bc[f] = f ? L.sphere_grid[0] : 0;
+  L.pixel_units = (const qa::WorkUnit*)(mem + off_xu);
+  for (int v = 0, at = 0; v < qa::kPixelVariants; ++v) {
+    L.pix_first[v] = pix_first[v];
+    L.pix_count[v] = (int)xv[v].size();
+    L.pix_grid[v] = pix_grid[v];
+    L.pix_bc[v] = at;
+    at += pix_grid[v];
   }
   L.close_list = (qa::CloseEntry*)(mem + off_cl);
   L.flag_list = (qa::ListEntry*)(mem + off_fl);
@@ -1577,7 +1613,8 @@ int qa_batch_stats(qa_batch* b, void* stream, qa_stats* out) {
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
   qa::Counters c;
   if (e == cudaSuccess) e = cudaMemcpy(&c, b->L.cnt, sizeof(c), cudaMemcpyDeviceToHost);
-  const int gs = b->L.sphere_grid[0] + b->L.sphere_grid[1];
+  int gs = 0;
+  for (int v = 0; v < qa::kPixelVariants; ++v) gs += b->L.pix_grid[v];
   std::vector<qa::BlockCounts> bp((size_t)(b->L.grid_prep + gs)), bs((size_t)(b->L.grid_search + gs));
   if (e == cudaSuccess)
     e = cudaMemcpy(bp.data(), b->L.bc_prep, sizeof(qa::BlockCounts) * bp.size(), cudaMemcpyDeviceToHost);

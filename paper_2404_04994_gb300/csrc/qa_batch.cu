@@ -44,44 +44,6 @@ __global__ void __launch_bounds__(kPrepThreads) k_prep_batch(GsLaunch L) {
   }
 }
 
-// Prep, sphere search and outputs of the arrays that take it, the open and the
-// closed ones in a launch of their own: with both forms' code in one kernel
-// its warps miss the instruction cache (10 stalls per issue instead of 1.7,
-// 1,600 us instead of about 1,000 us for the 65 arrays of 12 to 16 dots of a
-// batch of 192).  Blocks take units as above; a unit's pixel pairs go round
-// the block's warps.
-template <bool CLOSED>
-__global__ void __launch_bounds__(kPrepThreads, kSphereBlocks)
-k_sphere_batch(const __grid_constant__ GsLaunch L) {
-  __shared__ SphereShared sh;
-  __shared__ int s_unit;
-  const int f = CLOSED ? 1 : 0;
-  int staged = -1;
-  sphere_zero_counts(sh);
-  for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) s_unit = (int)atomicAdd(&L.cnt->q_sphere[f], 1u);
-    __syncthreads();
-    const int u = s_unit;
-    if (u >= L.sphere_count[f]) break;
-    const WorkUnit wu = L.sphere_units[L.sphere_first[f] + u];
-    const ArrayDesc& a = L.table[wu.array];
-    if (wu.array != staged) {
-      sphere_stage_array(a, sh);
-      staged = wu.array;
-    }
-    const long long end = wu.first + wu.count;
-    for (long long q = wu.first + (threadIdx.x >> 5) * 2; q < end; q += kSphereTeams) {
-      const long long p = q + ((threadIdx.x >> 4) & 1);
-      sphere_pixel<CLOSED>(L, a, sh, wu.array, p, p < end);
-    }
-  }
-  if (threadIdx.x == 0) {
-    const int b = L.sphere_bc[f] + blockIdx.x;
-    sphere_counts(sh, L.bc_prep[L.grid_prep + b], L.bc_search[L.grid_search + b]);
-  }
-}
-
 // The search of one kernel variant (split, form, team finish): a persistent
 // grid over that variant's units, so that every variant runs with its own
 // register count (one kernel over all of them needs the largest).
@@ -168,8 +130,7 @@ void batch_occupancy(int* prep_per_sm, int* search_per_sm) {
 cudaError_t launch_ground_state_batch(const GsLaunch& L, cudaStream_t st) {
   if (L.ev) cudaEventRecord(L.ev[0], st);
   cudaMemsetAsync(L.cnt, 0, sizeof(Counters), st);
-  if (L.sphere_count[0] > 0) k_sphere_batch<false><<<L.sphere_grid[0], kPrepThreads, 0, st>>>(L);
-  if (L.sphere_count[1] > 0) k_sphere_batch<true><<<L.sphere_grid[1], kPrepThreads, 0, st>>>(L);
+  launch_pixels_batch(L, st);
   if (L.n_prep_units > 0) k_prep_batch<<<L.grid_prep, kPrepThreads, 0, st>>>(L);
   if (L.ev) cudaEventRecord(L.ev[1], st);
   for (int v = 0; v < kBatchVariants; ++v)

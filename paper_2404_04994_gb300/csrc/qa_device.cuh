@@ -126,8 +126,8 @@ struct __align__(16) SphereConsts {
   unsigned char ord[kMaxDot];           // dot of each level
   unsigned char pos[kMaxDot];           // level of each dot
   float ysq;                            // sum_k (sum_l |W_kl|)^2
-  float msum;                           // sum_ij |M_ij|
-  int valid;                            // 0: no factor (few dots, or updated on the device)
+  float msum;                           // sum_ij |M_ij| (any number of dots)
+  int valid;                            // 0: updated on the device, or no factor
   int pad;
 };
 
@@ -175,9 +175,9 @@ struct Counters {
   unsigned int n_flag;  // length of the FP64 recheck list
   unsigned int n_tie;   // length of the near-tie list
   unsigned int n_close; // length of the close list
-  unsigned int next;    // single array: the sphere search's work queue
+  unsigned int next;    // single array: the one-pass kernel's work queue
   unsigned int q_prep;  // batched launch: work-queue heads
-  unsigned int q_sphere[2];  // ... the sphere search's, open and closed
+  unsigned int q_pixel[10];  // ... of each one-pass variant
   unsigned int q_var[20];  // batched launch: the search queue of each kernel variant
   unsigned int lists_done; // blocks of the list kernel that have finished
   unsigned int soft_done;  // blocks of the soft gradient reduction that have finished
@@ -207,7 +207,7 @@ struct ListEntry {
   int tie;  // 1 when the order of the best two candidates is in doubt
 };
 
-// A pixel the sphere search could not settle: the candidates within its
+// A pixel the one-pass search could not settle: the candidates within its
 // margin (nl of them, two to kCloseMax; 16-bit patterns over the dots, two to
 // a word), or none (nl = 0).
 constexpr int kCloseMax = 8;

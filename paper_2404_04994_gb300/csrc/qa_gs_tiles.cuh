@@ -203,14 +203,14 @@ struct PrepPixel {
   unsigned qp_set; // QP pixels: the active set the QP settled on
 };
 
-template <bool CLOSED>
+template <bool CLOSED, int W = 0>
 __device__ __forceinline__ PrepPixel prep_set(const ArrayDesc& a, PrepShared& sh, long long p,
                                               bool active) {
   const int n = a.n;
   const float bx_qp_scale = a.bx_qp_scale > 0.f ? a.bx_qp_scale : sh.cs.bx_qp_scale;
   const bool model_bad = sh.cs.model_bad != 0;
 
-  const int TP = a.prep_team;
+  const int TP = W ? W : a.prep_team;  // W: the team width where it is known
   const int lt = threadIdx.x & (TP - 1);
   const int lane = threadIdx.x & 31;
   const int tbase = lane & ~(TP - 1);                   // team's first lane
@@ -442,12 +442,13 @@ __device__ __forceinline__ PrepPixel prep_set(const ArrayDesc& a, PrepShared& sh
 
 // The second half: h of the lane's dot (returned) and S, the sum of the
 // magnitudes entering a candidate's energy (per team).
+template <int W = 0>
 __device__ __forceinline__ float prep_h(const ArrayDesc& a, PrepShared& sh, const PrepPixel& q,
                                         float& S) {
   const int n = a.n;
   const float* sMhi = sh.cs.Mhi;
   const float* sMlo = sh.cs.Mlo;
-  const int TP = a.prep_team;
+  const int TP = W ? W : a.prep_team;
   const int lt = threadIdx.x & (TP - 1);
   const int tbase = threadIdx.x & 31 & ~(TP - 1);
   const unsigned tmask = (TP == 32 ? 0xffffffffu : ((1u << TP) - 1u)) << tbase;
@@ -934,6 +935,7 @@ __device__ inline void search_tile(const GsLaunch& L, const ArrayDesc& a, Search
 // U = r^T M r of the lane's charges ni: a row per lane, as in search_tile's
 // wide teams, summed over the team (every lane of tmask calls; rhi, rlo: the
 // team's scratch rows).
+template <int W>
 __device__ __forceinline__ df team_energy(const ModelConsts& cs, int n, int lt, unsigned tmask,
                                           bool live, int ni, df c, float* rhi, float* rlo) {
   const df r = live ? df_sub({(float)ni, 0.f}, c) : df{0.f, 0.f};
@@ -958,62 +960,83 @@ __device__ __forceinline__ df team_energy(const ModelConsts& cs, int n, int lt, 
     u = df_mul(fast_two_sum(shi, slo), r);
   }
 #pragma unroll
-  for (int off = 1; off < kSphT; off <<= 1) {
+  for (int off = 1; off < W; off <<= 1) {
     df o;
-    o.hi = __shfl_xor_sync(tmask, u.hi, off, kSphT);
-    o.lo = __shfl_xor_sync(tmask, u.lo, off, kSphT);
+    o.hi = __shfl_xor_sync(tmask, u.hi, off, W);
+    o.lo = __shfl_xor_sync(tmask, u.lo, off, W);
     u = df_add(u, o);
   }
   return u;
 }
 
 // ---------------------------------------------------------------------------
-// (a1)-(a6), (a8) in one pass for arrays of 9 to 16 dots: a team of 16 lanes,
-// lane i owning dot i, prepares a pixel, searches its candidate set with the
-// sphere search and writes its outputs; c, the candidate set and h stay in
-// the lanes.  A pixel with candidates too close to call, or whose search does
-// not end (no factor, or too many nodes), gets its record and goes on the
-// close list (settle_entry); one whose candidate set is in doubt gets its
-// record and goes on the FP64 list.
-// What bounds it: instruction issue (1,430 warp instructions per 16-dot pixel,
-// 2.4 - 3 a cycle; the tile kernels' 3,061, three quarters of them in the
-// FP32 search).  Sixteen lanes a pixel as in the prep, so that a pixel's whole
-// way keeps its lanes.  Whole calls, before / after: 16 dots 100 x 100 57 / 42
-// us (closed 93 / 60), 16-dot list of 10^4 vectors 71 / 54 us, 12 dots
-// 400 x 301 241 / 172 us.
+// (a1)-(a6), (a8) in one pass: a team of W = 4, 8 or 16 lanes, lane i owning
+// dot i, prepares a pixel, searches its candidate set and writes its outputs;
+// c and the candidate set stay in the lanes.  The search is the sphere search
+// where many dots are expected ambiguous, else the enumeration below.  A pixel
+// with candidates too close to call, or whose search does not end, gets its
+// record and goes on the close list (settle_entry); one whose candidate set is
+// in doubt gets its record and goes on the FP64 list.
+// What bounds it: instruction issue (1,430 warp instructions per 16-dot pixel
+// of the sphere search, 2.4 - 3 a cycle; the tile kernels' 3,061, three
+// quarters of them in the FP32 search).  Whole calls, before / after: 16 dots
+// 100 x 100 57 / 42 us (closed 93 / 60), 16-dot list of 10^4 vectors 71 / 54
+// us, 12 dots 400 x 301 241 / 172 us.
 // ---------------------------------------------------------------------------
-constexpr int kSphereTeams = kPrepThreads / kSphT;
-struct SphereShared {
+template <int W>
+struct PixelShared {
+  static constexpr int kTeams = kPrepThreads / W;
   PrepShared p;
-  SphereModel m;
-  float4 lev[kSphereTeams][kMaxDot / 2];
-  unsigned long long cand[kSphereTeams], ev[kSphereTeams];
-  unsigned qp[kSphereTeams], doubled[kSphereTeams], boundary[kSphereTeams],
-      overflow[kSphereTeams];
+  unsigned long long cand[kTeams], ev[kTeams];
+  unsigned qp[kTeams], doubled[kTeams], boundary[kTeams], overflow[kTeams];
   int valid;
 };
+struct SphereShared : PixelShared<kSphT> {
+  SphereModel m;
+  float4 lev[kTeams][kMaxDot / 2];
+};
+// The search of a kernel's pixels: the enumeration, the sphere search, or the
+// one that a pixel's ambiguous dots call for (a warp's pixels alike: the
+// sphere search from kMixedDots on, where the enumeration's 2^k / 256 blocks
+// cost more).
+enum : int { kPixDense = 0, kPixSphere = 1, kPixMixed = 2 };
+constexpr int kMixedDots = 12;
+template <int W, int MODE>
+struct PixelSharedOf { typedef PixelShared<W> type; };
+template <>
+struct PixelSharedOf<kSphT, kPixSphere> { typedef SphereShared type; };
+template <>
+struct PixelSharedOf<kSphT, kPixMixed> { typedef SphereShared type; };
 static_assert(kSphT * sizeof(float) * kQPRow >= kSphStack * sizeof(uint2),
               "the team's QP rows hold its waiting nodes");
 
 // Block set-up (all threads), once per array.
-__device__ inline void sphere_stage_array(const ArrayDesc& a, SphereShared& sh) {
+__device__ inline void pixel_stage_search(const ArrayDesc& a, SphereShared& sh) {
   sphere_stage(a.md->s, sh.m);
+}
+template <int W>
+__device__ inline void pixel_stage_search(const ArrayDesc&, PixelShared<W>&) {}
+template <typename SH>
+__device__ inline void pixel_stage_array(const ArrayDesc& a, SH& sh) {
+  pixel_stage_search(a, sh);
   if (threadIdx.x == 0) sh.valid = a.md->s.valid;
   prep_stage_array(a, sh.p);  // ends with a barrier
 }
-__device__ inline void sphere_zero_counts(SphereShared& sh) {
-  if (threadIdx.x < kSphereTeams) {
+template <int W>
+__device__ inline void pixel_zero_counts(PixelShared<W>& sh) {
+  if (threadIdx.x < sh.kTeams) {
     sh.cand[threadIdx.x] = sh.ev[threadIdx.x] = 0ull;
     sh.qp[threadIdx.x] = sh.doubled[threadIdx.x] = 0u;
     sh.boundary[threadIdx.x] = sh.overflow[threadIdx.x] = 0u;
   }
 }
 // The block's counts (thread 0 after a barrier).
-__device__ inline void sphere_counts(const SphereShared& sh, BlockCounts& prep,
-                                     BlockCounts& search) {
+template <int W>
+__device__ inline void pixel_counts(const PixelShared<W>& sh, BlockCounts& prep,
+                                    BlockCounts& search) {
   PrepAcc p;
   SearchAcc s;
-  for (int t = 0; t < kSphereTeams; ++t) {
+  for (int t = 0; t < sh.kTeams; ++t) {
     p.candidates += sh.cand[t];
     p.qp += sh.qp[t];
     p.doubled += sh.doubled[t];
@@ -1030,16 +1053,177 @@ __device__ inline void sphere_counts(const SphereShared& sh, BlockCounts& prep,
   search.overflow = s.overflow;
 }
 
-// One warp's two pixels, p its team's (active: below the end).
-template <bool CLOSED>
-__device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, SphereShared& sh,
-                                    int array, long long p, bool active) {
+// The enumeration: the candidate energies relative to the base,
+//     E(b) = sum_{s in b} v_s + sum_{s < s' in b} M_ss',  v = h + M_ss / 2,
+// of one pixel by its team.  The first kIn slots are inner (2^kIn energies at
+// a time by doubling), the next log2 W the lane's, further ones a loop of the
+// whole team; a state of the lane and loop slots is summed from scratch.  Two
+// passes: the minimum, then the patterns within G of it (by each lane's best
+// block alone unless another block of some lane is that close).  The same
+// arguments and results as sphere_search, patterns over the dots; v: the
+// dot's single-flip energy; sd, sv, lst: W (lst: 16) words of scratch each.
+// What bounds it: instruction issue, about 140 warp instructions a pixel at
+// up to kIn + log2 W slots against 320 of the tile kernels' thread per pixel
+// or two, which hold 32 pair terms in registers (four blocks per SM).
+template <int W, bool CLOSED>
+__device__ __forceinline__ unsigned dense_search(const float* sM, int n, int lt, bool active,
+                                                 float v, unsigned mask, int w, float G, int* sd,
+                                                 float* sv, unsigned* lst, int& close,
+                                                 unsigned& evaluated) {
+  constexpr int LB = W == 16 ? 4 : W == 8 ? 3 : 2;
+  constexpr int kIn = W == 4 ? 2 : 4, NI = 1 << kIn;
+  const unsigned hw = threadIdx.x & 31u & ~(unsigned)(W - 1);
+  constexpr unsigned kW = W == 32 ? 0xffffffffu : (1u << W) - 1u;
+  auto team = [&](bool pred) { return (__ballot_sync(kFull, pred) >> hw) & kW; };
+  const int k = active ? __popc(mask) : 0;
+  const bool amb = active && ((mask >> lt) & 1u);
+  const int slot = __popc(mask & ((1u << lt) - 1u));
+  __syncwarp();
+  sd[lt] = 0;
+  sv[lt] = 0.f;
+  __syncwarp();
+  if (amb) {
+    sd[slot] = lt;
+    sv[slot] = v;
+  }
+  __syncwarp();
+  const int nlb = min(max(k - kIn, 0), LB), nout = max(k - kIn - LB, 0);
+  // the lane's state: A, q; the inner pair terms P
+  int dI[kIn];  // inner dots (as columns)
+  float q0[kIn], P[NI], A0 = 0.f, wl[LB];
+  int rl[LB];
+#pragma unroll
+  for (int j = 0; j < kIn; ++j) {
+    dI[j] = sd[j];
+    q0[j] = j < k ? sv[j] : kBig;
+  }
+#pragma unroll
+  for (int b = 0; b < NI; ++b) P[b] = 0.f;
+#pragma unroll
+  for (int j = 1; j < kIn; ++j) {
+    const float* row = sM + sd[j] * kLdM;
+#pragma unroll
+    for (int l = 0; l < j; ++l) {
+      const float m = row[dI[l]];
+#pragma unroll
+      for (int b = 0; b < NI; ++b)
+        if (((b >> j) & 1) && ((b >> l) & 1)) P[b] += m;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < LB; ++i) {
+    rl[i] = sd[kIn + i];
+    wl[i] = (i < nlb && ((lt >> i) & 1)) ? 1.f : 0.f;
+    const float* row = sM + rl[i] * kLdM;
+    float add = sv[kIn + i];
+#pragma unroll
+    for (int l = 0; l < i; ++l) add = fmaf(wl[l], row[rl[l]], add);
+    A0 = fmaf(wl[i], add, A0);
+#pragma unroll
+    for (int j = 0; j < kIn; ++j) q0[j] = fmaf(wl[i], row[dI[j]], q0[j]);
+  }
+  const bool own = active && (lt >> nlb) == 0;
+  const int r0 = w - __popc((unsigned)lt);  // closed: weight left
+  // the energies of one block: loop pattern o
+  auto block = [&](unsigned o, float* e) {
+    float A = A0, q[kIn];
+#pragma unroll
+    for (int j = 0; j < kIn; ++j) q[j] = q0[j];
+    for (unsigned m = o; m; m &= m - 1u) {
+      const int s1 = kIn + LB + __ffs(m) - 1;
+      const float* row = sM + sd[s1] * kLdM;
+      float add = sv[s1];
+#pragma unroll
+      for (int i = 0; i < LB; ++i) add = fmaf(wl[i], row[rl[i]], add);
+      for (unsigned l = o & ((m & (0u - m)) - 1u); l; l &= l - 1u)
+        add += row[sd[kIn + LB + __ffs(l) - 1]];
+      A += add;
+#pragma unroll
+      for (int j = 0; j < kIn; ++j) q[j] += row[dI[j]];
+    }
+    e[0] = A;
+#pragma unroll
+    for (int j = 0; j < kIn; ++j)
+#pragma unroll
+      for (int b = 0; b < (1 << j); ++b) e[b + (1 << j)] = e[b] + q[j];
+    const int r = r0 - __popc(o);
+#pragma unroll
+    for (int b = 0; b < NI; ++b) {
+      e[b] += P[b];
+      if (CLOSED && popc_c((unsigned)b) != r) e[b] = kInf;
+    }
+  };
+  float g1 = kInf, g2 = kInf;
+  unsigned o1 = 0u;
+  const unsigned no = own ? 1u << nout : 0u;
+#pragma unroll 1
+  for (unsigned o = 0; o < no; ++o) {
+    float e[NI];
+    block(o, e);
+    float m = e[0];
+#pragma unroll
+    for (int b = 1; b < NI; ++b) m = fminf(m, e[b]);
+    g2 = fminf(g2, fmaxf(g1, m));
+    if (m < g1) {
+      g1 = m;
+      o1 = o;
+    }
+  }
+  evaluated += no * (unsigned)NI;
+  __syncwarp();
+  float m1 = g1;
+#pragma unroll
+  for (int off = W / 2; off > 0; off >>= 1) m1 = fminf(m1, __shfl_xor_sync(kFull, m1, off));
+  const float thr = m1 + G;
+  // the patterns within the margin: inner bits of a block at a time
+  const bool wide = __any_sync(kFull, own && g2 <= thr);
+  int nl = 0;
+  unsigned b1 = 0u;
+#pragma unroll 1
+  for (unsigned o = 0;; ++o) {
+    const unsigned oo = wide ? o : o1;
+    unsigned hit = 0u;
+    if (own && oo < no && (wide || g1 <= thr)) {
+      float e[NI];
+      block(oo, e);
+#pragma unroll
+      for (int b = 0; b < NI; ++b) hit |= e[b] <= thr ? 1u << b : 0u;
+    }
+    __syncwarp();
+    while (true) {  // one candidate of each lane at a time
+      const unsigned has = team(hit != 0u);
+      if (!__any_sync(kFull, hit != 0u)) break;
+      if (hit) {
+        const unsigned sb = (unsigned)(__ffs(hit) - 1) | ((unsigned)lt << kIn) | (oo << (kIn + LB));
+        const int at = nl + __popc(has & ((1u << lt) - 1u));
+        // slots to dots
+        unsigned db = 0u;
+        for (unsigned m = sb; m; m &= m - 1u) db |= 1u << sd[__ffs(m) - 1];
+        if (at < kSphList) lst[at] = db;
+        hit &= hit - 1u;
+      }
+      nl += __popc(has);
+    }
+    if (!wide || !__any_sync(kFull, own && o + 1 < no)) break;
+  }
+  __syncwarp();
+  b1 = nl > 0 ? lst[0] : 0u;
+  close = (!(m1 < kBig) || nl > kSphList || nl < 1) ? 0 : nl;
+  return b1;
+}
+
+// One warp's pixels, p its team's (active: below the end).
+template <int W, bool CLOSED, int MODE>
+__device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
+                                    typename PixelSharedOf<W, MODE>::type& sh, int array,
+                                    long long p, bool active) {
   const int n = a.n;
-  const int lt = threadIdx.x & (kSphT - 1);
-  const int tq = threadIdx.x & ~(kSphT - 1);
-  const int team = threadIdx.x / kSphT;
-  const unsigned hw = threadIdx.x & 16u;
-  const PrepPixel q = prep_set<CLOSED>(a, sh.p, p, active);
+  const int lt = threadIdx.x & (W - 1);
+  const int tq = threadIdx.x & ~(W - 1);
+  const int team = threadIdx.x / W;
+  const unsigned hw = threadIdx.x & 31u & ~(unsigned)(W - 1);
+  constexpr unsigned kW = (1u << W) - 1u;
+  const PrepPixel q = prep_set<CLOSED, W>(a, sh.p, p, active);
   const bool amb = q.live && ((q.mask >> lt) & 1u);
   const int k = __popc(q.mask);
   const bool qp = (q.flags & kFlagQP) != 0u;
@@ -1056,11 +1240,11 @@ __device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, Spher
   sh.p.qx[threadIdx.x] = r0;
   sh.p.qz[threadIdx.x] = q.live ? __fadd_rn(__fsub_rn(q.x.hi, q.c.hi), q.x.lo - q.c.lo) : 0.f;
   __syncwarp();
-  float S = 0.f;
+  float S = 0.f, v = 0.f;
   {
     float h0 = 0.f, h1 = 0.f;
 #pragma unroll
-    for (int j = 0; j < kMaxDot; j += 4) {
+    for (int j = 0; j < W; j += 4) {
       const float4 r4 = *reinterpret_cast<const float4*>(&sh.p.qx[tq + j]);
       h0 = fmaf(Mrow[j], r4.x, h0);
       h1 = fmaf(Mrow[j + 1], r4.y, h1);
@@ -1068,6 +1252,7 @@ __device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, Spher
       h1 = fmaf(Mrow[j + 3], r4.w, h1);
     }
     const unsigned below = q.mask & ((1u << lt) - 1u);
+    v = (h0 + h1) + 0.5f * Mrow[lt];
     if (amb) {
       S = fabsf(h0 + h1);
       if (below == (1u << lt) - 1u) {
@@ -1075,51 +1260,76 @@ __device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, Spher
       } else {
         S += 0.5f * Mrow[lt];
 #pragma unroll
-        for (int j = 0; j < kMaxDot; ++j) S += ((below >> j) & 1u) ? fabsf(Mrow[j]) : 0.f;
+        for (int j = 0; j < W; ++j) S += ((below >> j) & 1u) ? fabsf(Mrow[j]) : 0.f;
       }
     }
   }
 #pragma unroll
-  for (int off = 8; off > 0; off >>= 1) S += __shfl_xor_sync(kFull, S, off);
-  // the gradient M (x - c) where a constraint is active (else zero, closed: a
-  // multiple of 1)
-  float a1 = 0.f, neg = 0.f, rmax = 1.f;
-  if (__any_sync(kFull, qp)) {
-    float z = 0.f;
-#pragma unroll
-    for (int j = 0; j < kMaxDot; ++j) z = fmaf(Mrow[j], sh.p.qz[tq + j], z);
-    rmax = fmaxf(fabsf(r0), fabsf(sh.p.qz[threadIdx.x]));
-    if (CLOSED) {  // the multiple of 1: the least entry, a free dot's
-      float zm = q.live ? z : kInf;
-#pragma unroll
-      for (int off = 8; off > 0; off >>= 1) zm = fminf(zm, __shfl_xor_sync(kFull, zm, off));
-      z -= zm;
-    }
-    a1 = (qp && amb) ? fmaxf(z, 0.f) : 0.f;
-    neg = (qp && amb) ? fmaxf(-z, 0.f) : 0.f;
-#pragma unroll
-    for (int off = 8; off > 0; off >>= 1) {
-      neg += __shfl_xor_sync(kFull, neg, off);
-      rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
-    }
-  }
-  const float ez = u24 * a.md->s.msum * fmaxf(rmax, 1.f);  // u sum |M| |r|
-  const float bound = pixel_bound(a, S * 1.00001f + 20.f * ez, k);
-  neg += (qp ? 24.f : 2.f) * ez;
-  // no factor, or a centre outside [-1, 1] (an unsettled QP): left to the
-  // FP32 search
-  const bool far = ((__ballot_sync(kFull, !(fabsf(f) <= 1.f)) >> hw) & 0xffffu) != 0u;
+  for (int off = W / 2; off > 0; off >>= 1) S += __shfl_xor_sync(kFull, S, off);
+  const unsigned any_qp = __any_sync(kFull, qp);
+  float rmax = 1.f;
   int close = 0;
-  unsigned ev = 0;
-  const unsigned bits = sphere_search<CLOSED>(
-      a.md->s, sh.m, n, lt, active && sh.valid && !far, f, a1, q.mask, q.w, bound, neg,
-      &sh.p.qx[tq], &sh.p.qz[tq], sh.lev[team], reinterpret_cast<uint2*>(&sh.p.qK[tq][0]), close,
-      ev);
+  unsigned ev = 0, bits = 0u;
+  const bool sphere =
+      MODE == kPixSphere || (MODE == kPixMixed && __any_sync(kFull, active && k >= kMixedDots));
+  if constexpr (MODE != kPixDense) if (sphere) {
+    // the gradient M (x - c) where a constraint is active (else zero, closed: a
+    // multiple of 1)
+    float a1 = 0.f, neg = 0.f;
+    if (any_qp) {
+      float z = 0.f;
+#pragma unroll
+      for (int j = 0; j < W; ++j) z = fmaf(Mrow[j], sh.p.qz[tq + j], z);
+      rmax = fmaxf(fabsf(r0), fabsf(sh.p.qz[threadIdx.x]));
+      if (CLOSED) {  // the multiple of 1: the least entry, a free dot's
+        float zm = q.live ? z : kInf;
+#pragma unroll
+        for (int off = W / 2; off > 0; off >>= 1) zm = fminf(zm, __shfl_xor_sync(kFull, zm, off));
+        z -= zm;
+      }
+      a1 = (qp && amb) ? fmaxf(z, 0.f) : 0.f;
+      neg = (qp && amb) ? fmaxf(-z, 0.f) : 0.f;
+#pragma unroll
+      for (int off = W / 2; off > 0; off >>= 1) {
+        neg += __shfl_xor_sync(kFull, neg, off);
+        rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
+      }
+    }
+    const float ez = u24 * a.md->s.msum * fmaxf(rmax, 1.f);  // u sum |M| |r|
+    const float bound = pixel_bound(a, S * 1.00001f + 20.f * ez, k);
+    neg += (qp ? 24.f : 2.f) * ez;
+    // no factor, or a centre outside [-1, 1] (an unsettled QP): left to the
+    // FP32 search
+    const bool far = ((__ballot_sync(kFull, !(fabsf(f) <= 1.f)) >> hw) & kW) != 0u;
+    bits = sphere_search<CLOSED>(a.md->s, sh.m, n, lt, active && sh.valid && !far, f, a1, q.mask,
+                                 q.w, bound, neg, &sh.p.qx[tq], &sh.p.qz[tq], sh.lev[team],
+                                 reinterpret_cast<uint2*>(&sh.p.qK[tq][0]), close, ev);
+  }
+  // (the candidates within the margin: level patterns of the sphere search,
+  // dot patterns of the enumeration)
+  unsigned* lst =
+      reinterpret_cast<unsigned*>(MODE == kPixDense ? &sh.p.qK[tq][0] : &sh.p.qz[tq]);
+  if constexpr (MODE != kPixSphere) if (!sphere) {
+    if (any_qp) {
+      rmax = fabsf(r0);
+#pragma unroll
+      for (int off = W / 2; off > 0; off >>= 1)
+        rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
+    }
+    const float ez = u24 * a.md->s.msum * fmaxf(rmax, 1.f);
+    // twice the near-tie bound as in the sphere search, once more for this
+    // search's own sums (at most 2 k + 8 additions), and the error of the
+    // plain h on both sides
+    const float G = 3.f * pixel_bound(a, S * 1.00001f + 20.f * ez, k) + 40.f * ez;
+    bits = dense_search<W, CLOSED>(sh.p.cs.Mhi, n, lt, active && sh.valid, v, q.mask, q.w, G,
+                                   &sh.p.qa[tq], &sh.p.qc[tq], lst, close, ev);
+  }
   const bool done = active && close == 1;
   // candidates too close to tell apart: left, with their patterns over the
   // dots, to the list kernel; so is a search that did not end
   if (__any_sync(kFull, active && close != 1)) {
-    const unsigned* lst = reinterpret_cast<const unsigned*>(&sh.p.qz[tq]);
+    int pos = lt;
+    if constexpr (MODE != kPixDense) pos = sphere ? sh.m.pos[lt] : lt;
     const bool leave = active && close != 1 && lt == 0;
     CloseEntry* ce = nullptr;
     if (leave) {
@@ -1131,38 +1341,45 @@ __device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, Spher
 #pragma unroll 1
     for (int e = 0; e < kCloseMax; e += 2) {
       const unsigned b0 = __ballot_sync(
-          kFull, lt < n && e < close && ((lst[e] >> sh.m.pos[lt]) & 1u));
+          kFull, lt < n && e < close && ((lst[e] >> pos) & 1u));
       const unsigned b1 = __ballot_sync(
-          kFull, lt < n && e + 1 < close && ((lst[e + 1] >> sh.m.pos[lt]) & 1u));
-      if (leave) ce->pat[e >> 1] = ((b0 >> hw) & 0xffffu) | (((b1 >> hw) & 0xffffu) << 16);
+          kFull, lt < n && e + 1 < close && ((lst[e + 1] >> pos) & 1u));
+      if (leave) ce->pat[e >> 1] = ((b0 >> hw) & kW) | (((b1 >> hw) & kW) << 16);
     }
     __syncwarp();
   }
 
   // n* = base + bits and U(n*) = 1/2 r^T M r
   int ni = q.base + (int)((bits >> lt) & 1u);
-  const df u = team_energy(sh.p.cs, n, lt, kFull, q.live, ni, q.c, &sh.p.qx[tq], &sh.p.qz[tq]);
+  const df u = team_energy<W>(sh.p.cs, n, lt, kFull, q.live, ni, q.c, &sh.p.qx[tq], &sh.p.qz[tq]);
   unsigned flags = q.flags, ov = 0u;
-  // int8 maps of 16 dots: the team's charges as one 16-byte store
-  const bool vec = !a.out_n16 && n == 16 && (reinterpret_cast<uintptr_t>(a.out_n) & 15u) == 0;
+  // int8 maps of W dots: the team's charges as one W-byte store
+  const bool vec =
+      !a.out_n16 && n == W && (reinterpret_cast<uintptr_t>(a.out_n) & (W - 1)) == 0;
   if (vec) {
     if (ni > 127) {
       ni = 127;
       ov = kFlagOverflow;
     }
-    unsigned word = ((unsigned)ni & 0xffu) << (8 * (lt & 3));
-    word |= __shfl_xor_sync(kFull, word, 1);
-    word |= __shfl_xor_sync(kFull, word, 2);
-    const unsigned w1 = __shfl_sync(kFull, word, hw + 4), w2 = __shfl_sync(kFull, word, hw + 8);
-    const unsigned w3 = __shfl_sync(kFull, word, hw + 12);
-    const unsigned w0 = word;
-    if (done && lt == 0)
-      *reinterpret_cast<int4*>(a.out_n + p * n) =
-          make_int4((int)w0, (int)w1, (int)w2, (int)w3);
+    unsigned w0 = ((unsigned)ni & 0xffu) << (8 * (lt & 3));
+    w0 |= __shfl_xor_sync(kFull, w0, 1);
+    w0 |= __shfl_xor_sync(kFull, w0, 2);
+    int8_t* dst = a.out_n + p * n;
+    if constexpr (W == 16) {
+      const unsigned w1 = __shfl_sync(kFull, w0, hw + 4), w2 = __shfl_sync(kFull, w0, hw + 8);
+      const unsigned w3 = __shfl_sync(kFull, w0, hw + 12);
+      if (done && lt == 0)
+        *reinterpret_cast<int4*>(dst) = make_int4((int)w0, (int)w1, (int)w2, (int)w3);
+    } else if constexpr (W == 8) {
+      const unsigned w1 = __shfl_sync(kFull, w0, hw + 4);
+      if (done && lt == 0) *reinterpret_cast<int2*>(dst) = make_int2((int)w0, (int)w1);
+    } else {
+      if (done && lt == 0) *reinterpret_cast<int*>(dst) = (int)w0;
+    }
   } else if (done && q.live) {
     store_charge(a, p * n + lt, ni, ov);
   }
-  if ((__ballot_sync(kFull, ov != 0u) >> hw) & 0xffffu) flags |= kFlagOverflow;
+  if ((__ballot_sync(kFull, ov != 0u) >> hw) & kW) flags |= kFlagOverflow;
   const unsigned evw = __reduce_add_sync(kFull, ev);
   if (active && lt == 0) {
     sh.cand[team] += CLOSED ? binom(k, q.w) : (1ull << k);
@@ -1173,7 +1390,7 @@ __device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, Spher
   const bool listed = done && (flags & (kFlagBoundary | kFlagQPCap | kFlagUnresolved)) != 0u;
   if (active && (close != 1 || listed)) {
     float Sx;
-    const float h = prep_h(a, sh.p, q, Sx);
+    const float h = prep_h<W>(a, sh.p, q, Sx);
     store_record<CLOSED>(a.recs + p, q, lt, h, pixel_bound(a, Sx, k));
   }
   if (done && lt == 0) {
@@ -1188,7 +1405,7 @@ __device__ inline void sphere_pixel(const GsLaunch& L, const ArrayDesc& a, Spher
 }
 
 // ---------------------------------------------------------------------------
-// Pixels that the sphere search left (the close list): the FP32 search's
+// Pixels that search_pixel left (the close list): the FP32 search's
 // near-tie flag and, where it is set, the argmin by exact energies.
 // ---------------------------------------------------------------------------
 // The pruned FP32 search's minimum of one block (an outer pattern with its
@@ -1281,11 +1498,13 @@ struct SettleScratch {
   } u;
 };
 
+template <int N>
+struct SplitSize { static constexpr int value = N; };
 // The FP32 search's best candidate (m1, pattern over the slots b1) and
 // runner-up m2 among the blocks of the nl listed candidates (slot patterns in
 // t.lst), or among all of them (nl = 0), with the sums that the array's search
-// takes: its split (5 + 2 or 5 + 4, block-level teams) and team width say
-// which, and lane v of that team runs in lane v of the warp.
+// takes: its split and team width say which, and lane v of that team runs in
+// lane v of the warp.
 template <bool CLOSED>
 static __device__ __noinline__ void listed_top2(const ArrayDesc& a, const float* sM,
                                                 const SlotView sv, SettleScratch& t, int nl,
@@ -1299,6 +1518,10 @@ static __device__ __noinline__ void listed_top2(const ArrayDesc& a, const float*
   __syncwarp();
   m1 = m2 = kInf;
   b1 = 0u;
+  // listed: lane e takes block e, each block once
+  bool own = lane < nl;
+  for (int e = 0; e < min(lane, nl); ++e) own = own && t.lst[e] != blk;
+  const int nlb = min(__ffs(T) - 1, max(k - a.cfg.L1 - a.cfg.L2, 0));  // the team's lane bits
   if (bnb) {
     // the tables of bnb_pair_build, an element per lane, and the inner pairs
     float* pm = t.u.bnb.pm;
@@ -1321,9 +1544,7 @@ static __device__ __noinline__ void listed_top2(const ArrayDesc& a, const float*
       t.u.bnb.ptab[lane] = r;
     }
     __syncwarp();
-    const int nout = max(k - kBnbIn, 0), nlb = min(__ffs(T) - 1, nout);
-    bool own = lane < nl;
-    for (int e = 0; e < min(lane, nl); ++e) own = own && t.lst[e] != blk;
+    const int nout = max(k - kBnbIn, 0);
     const unsigned nblk = nl > 0 ? (own ? 1u : 0u) : (1u << (nout + kBnbL2)), first = nl > 0 ? blk : lane;
     // (a middle pattern beyond the k slots holds no block)
     const unsigned midmax = 1u << min(max(k - kBnbL1, 0), kBnbL2);
@@ -1337,6 +1558,32 @@ static __device__ __noinline__ void listed_top2(const ArrayDesc& a, const float*
         b1 = b;
       }
     }
+  } else if (T < kTeamFinishMin) {
+    // narrow teams: the best candidate of each of the team's lanes, of its
+    // other blocks the minimum
+    unsigned long long ev = 0;
+    const bool run = nl > 0 ? own : lane < T;
+    const unsigned v = nl > 0 ? (blk >> a.cfg.L2) & ((1u << nlb) - 1u) : (unsigned)lane;
+    float g = kInf;
+    auto lanes = [&](auto l1, auto l2) {
+      search_lane<decltype(l1)::value, decltype(l2)::value, CLOSED, false, false, 5, true>(
+          sM, sv, (int)v, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev, nullptr, nullptr, nullptr,
+          kInf, 0.f, nl > 0 ? (int)blk : -1, &g);
+    };
+    if (run) {
+      if (a.cfg.L2 == 0) lanes(SplitSize<4>{}, SplitSize<0>{});
+      else if (a.cfg.L2 == 3) lanes(SplitSize<4>{}, SplitSize<3>{});
+      else lanes(SplitSize<5>{}, SplitSize<4>{});
+    }
+    for (int e = 0; e < nl; ++e) {
+      const float ge = __shfl_sync(kFull, g, e);
+      const unsigned ve = __shfl_sync(kFull, v, e);
+      const bool oe = __shfl_sync(kFull, own ? 1 : 0, e) != 0;
+      if (own && oe && e != lane && ve == v && (ge < g || (ge == g && e < lane))) {
+        m1 = kInf;  // that block is this team lane's best
+        m2 = g;
+      }
+    }
   } else {
     // split 5 + 4: block minima from the team tables
     constexpr int L1 = 5, L2 = 4;
@@ -1344,16 +1591,18 @@ static __device__ __noinline__ void listed_top2(const ArrayDesc& a, const float*
     col_build<L1, L2>(sM, sv, lane, 32, t.u.team.colt);
     iter_build<L1, L2>(sM, sv, lane, T, t.u.team.itab, 32);
     __syncwarp();
-    if (lane < T)
+    const int v = nl > 0 ? (int)((blk >> L2) & ((1u << nlb) - 1u)) : lane;
+    if (nl > 0 ? own : lane < T)
       search_lane<L1, L2, CLOSED, false, true, 5, true>(
-          sM, sv, lane, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev, t.u.team.colt,
-          t.u.team.itab, t.u.team.cslot[lane], kInf, 0.f, t.lst, nl > 0 ? nl : -1);
+          sM, sv, v, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev, t.u.team.colt, t.u.team.itab,
+          t.u.team.cslot[lane], kInf, 0.f, nl > 0 ? (int)blk : -1);
   }
   for (int off = 1; off < 32; off <<= 1) {
     const float o1 = __shfl_xor_sync(kFull, m1, off), o2 = __shfl_xor_sync(kFull, m2, off);
     const unsigned ob = __shfl_xor_sync(kFull, b1, off);
     top2_merge(m1, b1, m2, o1, ob, o2);
   }
+  if (T < kTeamFinishMin) return;
   float e1, e2;
   unsigned fb;
   const unsigned best = m1 < kInf ? b1 : 0u;
@@ -1428,7 +1677,7 @@ __device__ inline int settle_entry(const GsLaunch& L, const ArrayDesc& a, const 
 #pragma unroll 1
   for (int i = 0; i < nl; i += 2) {
     const unsigned b = pattern(i + half);  // (zero past the list)
-    const df u = team_energy(cs, n, lt, kFull, live, base + (int)((b >> lt) & 1u), c, t.rhi[half],
+    const df u = team_energy<kMaxDot>(cs, n, lt, kFull, live, base + (int)((b >> lt) & 1u), c, t.rhi[half],
                              t.rlo[half]);
     const unsigned sb =
         __reduce_or_sync(half ? 0xffff0000u : 0xffffu, (amb && ((b >> lt) & 1u)) ? 1u << slot : 0u);
@@ -1458,7 +1707,7 @@ __device__ inline int settle_entry(const GsLaunch& L, const ArrayDesc& a, const 
   const bool bit = amb && ((nl == 0 || (near && next != 0)) ? (b1 >> slot) & 1u
                                                             : (bbits >> lt) & 1u);
   const int ni = base + (bit ? 1 : 0);
-  if (nl == 0) best = team_energy(cs, n, lt, kFull, live, ni, c, t.rhi[half], t.rlo[half]);
+  if (nl == 0) best = team_energy<kMaxDot>(cs, n, lt, kFull, live, ni, c, t.rhi[half], t.rlo[half]);
   if (near) flags |= kFlagNearTie | (next == 0 ? kFlagRechecked : 0u);
   unsigned ov = 0u;
   if (live && half == 0) store_charge(a, (long long)ce.p * n + lt, ni, ov);

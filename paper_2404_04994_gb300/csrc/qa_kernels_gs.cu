@@ -2,8 +2,6 @@
 // for prep and search (one kernel or two), grid-stride over the lists for
 // resolve and recheck.
 // The stages themselves live in qa_gs_tiles.cuh (shared with the batch).
-#include <algorithm>
-
 #include "qa_gs_tiles.cuh"
 
 namespace qa {
@@ -114,43 +112,15 @@ __global__ void __launch_bounds__(kSearchThreads, kBnbBlocks) k_search_bnb(GsLau
   search_only_tile<kBnbL1, kBnbL2, CLOSED, true>(L);
 }
 
-// Prep, sphere search and outputs of arrays of 9 to 16 dots: a persistent
-// grid whose warps take pixel pairs one at a time (no barrier between a
-// block's warps, so a slow pixel holds up its own warp only).
-template <bool CLOSED>
-__global__ void __launch_bounds__(kPrepThreads, kSphereBlocks)
-k_sphere(const __grid_constant__ GsLaunch L) {
-  __shared__ SphereShared sh;
-  const ArrayDesc& a = L.one;
-  grid_dep_signal();
-  if (blockIdx.x == 0) zero_accumulators(L.cnt);
-  sphere_zero_counts(sh);
-  sphere_stage_array(a, sh);
-  // whole rounds of pairs by the warp's place, what is left over from a counter
-  const unsigned pairs = (unsigned)((a.sc.P + 1) / 2), warps = gridDim.x * (kPrepThreads / 32);
-  const unsigned rounds = (pairs < warps ? 1u : pairs / warps) * warps;
-  for (unsigned q = blockIdx.x * (kPrepThreads / 32) + (threadIdx.x >> 5);;) {
-    if (q >= rounds || q >= pairs) {
-      if (rounds >= pairs) break;
-      if ((threadIdx.x & 31) == 0) q = rounds + atomicAdd(&L.cnt->next, 1u);
-      q = __shfl_sync(kFull, q, 0);
-      if (q >= pairs) break;
-    }
-    const long long p = 2ll * q + ((threadIdx.x >> 4) & 1);
-    sphere_pixel<CLOSED>(L, a, sh, 0, p, p < a.sc.P);
-    if (q < rounds) q += warps;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) sphere_counts(sh, L.bc_prep[blockIdx.x], L.bc_search[blockIdx.x]);
-}
-
 // The lists after the search, in one launch: what the sphere search left
 // (settle_entry, a warp per entry), near ties (resolve_entry) and the FP64
 // recheck list (recheck_entry), grid-stride over each; an entry that one
 // stage cannot settle goes on to the next with the same block.  The last
 // two entries' shared layouts overlap, so each restages its model constants
-// when the other ran last.
+// when the other ran last.  CLOSE: a pixel-by-pixel kernel may have left a
+// close list (its code costs a call without one 2.5 us).
 static_assert(kResolveThreads == kRecheckThreads, "one block size for both lists");
+template <bool CLOSE>
 __global__ void __launch_bounds__(kResolveThreads)
 k_lists(const __grid_constant__ GsLaunch L) {
   __shared__ union ListShared {
@@ -159,8 +129,8 @@ k_lists(const __grid_constant__ GsLaunch L) {
   } S;
   constexpr int kWarps = kResolveThreads / 32;
   constexpr int kTodoRecheck = 1 << 30;  // beside the array's index (a batch has fewer)
-  __shared__ SettleScratch settle[kWarps];
-  __shared__ ListEntry todo[4 * kWarps];
+  __shared__ SettleScratch settle[CLOSE ? kWarps : 1];
+  __shared__ ListEntry todo[CLOSE ? 4 * kWarps : 1];
   __shared__ int n_todo;
   int staged_r = -1, staged_c = -1;  // the array whose constants each layout holds
   if (!L.table) {  // one array: its model is known before the search ends
@@ -176,7 +146,7 @@ k_lists(const __grid_constant__ GsLaunch L) {
   if (pf) first = L.tie_list[blockIdx.x];
   const unsigned ntie = L.cnt->n_tie;
   const unsigned nflag = L.cnt->n_flag;
-  const unsigned nclose = L.cnt->n_close;
+  const unsigned nclose = CLOSE ? L.cnt->n_close : 0u;
   unsigned my_res = 0, my_slmax = 0;
   // the close list, each warp its entries (spread over the blocks first), then
   // the two others; what the warps leave, the block takes on (todo: before it
@@ -189,11 +159,11 @@ k_lists(const __grid_constant__ GsLaunch L) {
   for (unsigned it = blockIdx.x;;) {
     ListEntry e;
     bool check;  // straight to the FP64 recheck
-    if (at < left) {
+    if (CLOSE && at < left) {
       e = todo[at++];
       check = (e.array & kTodoRecheck) != 0;
       e.array &= ~kTodoRecheck;
-    } else if (more) {
+    } else if (CLOSE && more) {
       __syncthreads();
       if (threadIdx.x == 0) n_todo = 0;
       __syncthreads();
@@ -305,14 +275,14 @@ static cudaError_t launch_dependent(void (*kern)(KArgs...), unsigned grid, unsig
 }
 
 cudaError_t launch_lists(const GsLaunch& L, cudaStream_t st) {
-  cudaError_t e = launch_dependent(k_lists, (unsigned)L.num_sms, kResolveThreads, st, L);
+  // (of a batch, only where an array is searched pixel by pixel)
+  bool close = L.one.search != kSearchTiles;
+  for (int v = 0; v < kPixelVariants; ++v) close = close || L.pix_count[v] > 0;
+  cudaError_t e = launch_dependent(close ? k_lists<true> : k_lists<false>, (unsigned)L.num_sms,
+                                   kResolveThreads, st, L);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-int sphere_blocks(const GsLaunch& L) {
-  const long long full = (L.one.sc.P + kSphereTeams - 1) / kSphereTeams;
-  return (int)std::min(full, (long long)L.num_sms * kSphereBlocks);
-}
 bool fused_tiles(const GsLaunch& L) {
   // a block preparing its own tile makes (prep_team / T) prep passes over it
   return L.one.prep_team <= 2 * L.one.cfg.T;
@@ -330,9 +300,8 @@ static cudaError_t run(const GsLaunch& L, cudaStream_t st) {
   // of its own, built for kBnbBlocks resident blocks per SM
   constexpr bool kBnb = bnb_search(L1, L2);
   const bool tf = L.one.cfg.T >= kTeamFinishMin;
-  if (L.one.sphere) {
-    k_sphere<CLOSED><<<sphere_blocks(L), kPrepThreads, 0, st>>>(L);
-    e = cudaGetLastError();
+  if (L.one.search != kSearchTiles) {
+    e = launch_pixels(L, st);
     if (L.ev) cudaEventRecord(L.ev[1], st);
   } else if (fused_tiles(L)) {
     if (L.ev) cudaEventRecord(L.ev[1], st);

@@ -16,6 +16,11 @@ struct SearchCfg {
   int T;   // lanes per pixel (1..32)
 };
 
+// How an array is searched: prep and FP32 search by tiles, or pixel by pixel
+// (search_pixel) with the sphere search, the enumeration, or either by the
+// pixel's ambiguous dots.
+enum : int { kSearchTiles = 0, kSearchSphere = 1, kSearchDense = 2, kSearchMixed = 3 };
+
 // One array of a ground-state call: its model, voltages, method settings,
 // scratch records and outputs.
 struct ArrayDesc {
@@ -30,7 +35,7 @@ struct ArrayDesc {
   float bx_analytic;   // decision margin for double-float continuous minima
   float bx_qp_scale;   // ... per unit of (1 + max|c| + N_hat) for FP32 QP minima
   PixRec* recs;        // scratch [P]
-  int sphere;          // the sphere search instead of the FP32 search
+  int search;          // kSearchTiles, kSearchSphere, kSearchDense or kSearchMixed
   int8_t* out_n;
   int16_t* out_n16;    // int16 charge map instead of out_n when non-null
   double* out_U;
@@ -44,7 +49,8 @@ constexpr int kTeamFinishMin = 8;    // teams at least this wide finish the winn
 constexpr int kBnbL1 = 5, kBnbL2 = 2;
 constexpr int kBnbMinT = 16;
 constexpr int kBnbBlocks = 5;  // resident blocks per SM its kernels are built for
-constexpr int kSphereBlocks = 8;  // resident blocks per SM the sphere search's kernels are built for
+constexpr int kPixelBlocks = 8;  // resident blocks per SM the one-pass kernels are built for
+constexpr int kPixelVariants = 10;  // batched one-pass kernels (qa_pixels_batch.cu)
 // Batched search kernel variants: 4 per split class (closed, team finish).
 constexpr int kBatchVariants = 20;
 static_assert(sizeof(((Counters*)nullptr)->q_var) / sizeof(unsigned) == kBatchVariants,
@@ -67,14 +73,15 @@ struct GsLaunch {
   int n_prep_units;
   const WorkUnit* search_units;
   int n_search_units;
-  // ... of the arrays that take the sphere search, open ones first: units
-  // [sphere_first, sphere_first + sphere_count) of each form, its grid, and
-  // its block counts from grid_prep (grid_search) + sphere_bc
-  const WorkUnit* sphere_units;
-  int sphere_first[2], sphere_count[2], sphere_grid[2], sphere_bc[2];
+  // ... of the arrays searched pixel by pixel, grouped by variant: units
+  // [pix_first, pix_first + pix_count) of each, its grid, and its block counts
+  // from grid_prep (grid_search) + pix_bc
+  const WorkUnit* pixel_units;
+  int pix_first[kPixelVariants], pix_count[kPixelVariants], pix_grid[kPixelVariants],
+      pix_bc[kPixelVariants];
   ListEntry* flag_list;        // scratch: pixels for the FP64 recheck
   ListEntry* tie_list;         // scratch: near-tie pixels for the list kernel's resolve
-  CloseEntry* close_list;      // scratch: pixels the sphere search left to the list kernel
+  CloseEntry* close_list;      // scratch: pixels the one-pass search left to the list kernel
   Counters* cnt;               // scratch; list heads zero at the start of each call
   BlockCounts* bc_prep;        // scratch [prep blocks]
   BlockCounts* bc_search;      // scratch [search blocks]
@@ -137,7 +144,11 @@ cudaError_t launch_prep(const GsLaunch& a, cudaStream_t st);
 cudaError_t launch_lists(const GsLaunch& a, cudaStream_t st);
 int prep_blocks(const GsLaunch& a);
 int search_blocks(const GsLaunch& a);
-int sphere_blocks(const GsLaunch& a);  // the sphere search's grid
+// The one-pass ground state (prep, search and outputs of the pixels) of one
+// array, its grid, and of a batch's arrays that take it.
+int pixel_blocks(const GsLaunch& a);
+cudaError_t launch_pixels(const GsLaunch& a, cudaStream_t st);
+cudaError_t launch_pixels_batch(const GsLaunch& a, cudaStream_t st);
 // true: one kernel prepares and searches each tile (block counts of both
 // stages per search block); false: k_prep then k_search
 bool fused_tiles(const GsLaunch& a);

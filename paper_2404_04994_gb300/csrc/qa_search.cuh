@@ -236,7 +236,7 @@ __device__ __forceinline__ float state_from_scratch(const float* sM,
 // sum min(0, g_m) + qneg (qneg: the model's bound of any pair-term sum, so
 // the bound holds for every candidate of the pattern) lies above lb_cut
 // holds no block to collect and is skipped.
-// ONLY: of the blocks just those in only[0 .. n_only) (n_only < 0: all).
+// ONLY: of the lane's blocks just block `only` (< 0: all); *gmin: its minimum.
 template <int L1, int L2, bool CLOSED, bool COLLECT, bool BLOCKS = false, int LANEBITS = 8,
           bool ONLY = false>
 __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
@@ -249,7 +249,7 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
                                             const float* __restrict__ itab = nullptr,
                                             float* __restrict__ cslot = nullptr,
                                             float lb_cut = kInf, float qneg = 0.f,
-                                            const unsigned* only = nullptr, int n_only = 0) {
+                                            int only = -1, float* gmin = nullptr) {
   static_assert(L1 >= 2 && L1 <= 6 && L2 >= 0 && L2 <= 5, "search split");
   // block-level searches with at least 9 inner + middle slots take the
   // iteration slots' terms from the team table itab (iter_build): at most 7
@@ -378,13 +378,10 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
     }
   }
 
-  for (unsigned it = 0; it < niter; ++it) {
+  const unsigned it0 = (ONLY && only >= 0) ? ((unsigned)only >> L2) >> nlb : 0u;
+  const unsigned it1 = (ONLY && only >= 0) ? it0 + 1u : niter;
+  for (unsigned it = it0; it < it1; ++it) {
     const unsigned o = (unsigned)t | (it << nlb);
-    if (ONLY && n_only >= 0) {
-      bool on = false;
-      for (int e = 0; e < n_only; ++e) on = on || (only[e] >> L2) == o;
-      if (!on) continue;
-    }
     float A = At;
     float q[L1 > 0 ? L1 : 1];
     float gm[L2 > 0 ? L2 : 1];
@@ -471,11 +468,7 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
             q[j] = up ? q[j] + Mim[j][mb] : q[j] - Mim[j][mb];
         }
       }
-      if (ONLY && n_only >= 0) {
-        bool on = false;
-        for (int e = 0; e < n_only; ++e) on = on || only[e] == (obase | gray_c((unsigned)s));
-        if (!on) continue;
-      }
+      if (ONLY && only >= 0 && (unsigned)only != (obase | gray_c((unsigned)s))) continue;
       float mbk;
       if (!CLOSED) {
         mbk = inner_min_open<L1>(A, q, P);
@@ -499,6 +492,7 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
   }
   evaluated += (unsigned long long)niter * (unsigned)nsteps * (unsigned)NI;
   if (COLLECT) return;
+  if (ONLY && gmin) *gmin = g1;
   if (BLOCKS) {  // block level only: the team finishes the winning block
     m1 = g1;
     b1 = blk;

@@ -1,4 +1,4 @@
-"""The sphere search (arrays of many ambiguous dots) against the FP32 search:
+"""The one-pass searches (sphere search, enumeration) against the FP32 search:
 the same model updated from device matrices has no host factor and takes the
 general path, so both run on the same inputs.  Charges and flags are equal;
 energies differ by the rounding of double-float sums of at most 256 terms
@@ -48,7 +48,16 @@ def _same(a, b, label):
     (13, False, 1.0, 19, 7, 0), (14, False, 1.0, 64, 33, 0), (16, False, 0.8, 100, 99, 0),
     (12, False, 1.0, 200, 151, 0), (16, False, 0.65, 201, 150, 0), (13, False, 0.8, 183, 167, 0),
     (12, True, 1.0, 41, 23, 1), (13, True, 0.8, 64, 31, 13), (15, True, 1.0, 57, 40, 30),
-    (16, True, 1.0, 100, 31, 16), (16, True, 0.65, 211, 143, 20)])
+    (16, True, 1.0, 100, 31, 16), (16, True, 0.65, 211, 143, 20),
+    # the enumeration by 4, 8 and 16 lanes
+    (3, False, 1.0, 1, 1, 0), (3, True, 1.0, 33, 5, 4), (4, False, 1.0, 67, 31, 0),
+    (4, True, 0.5, 67, 31, 3), (5, False, 1.0, 17, 1, 0), (6, True, 1.0, 50, 41, 12),
+    (8, False, 1.0, 101, 67, 0), (8, True, 0.25, 101, 67, 8), (8, True, 0.0, 31, 67, 5),
+    (9, True, 1.0, 90, 67, 9), (9, False, 0.5, 90, 67, 0), (11, False, 0.65, 90, 45, 0),
+    (11, True, 0.65, 90, 45, 7),
+    # either by the pixel's dots
+    (12, False, 0.5, 190, 160, 0), (14, False, 0.25, 60, 41, 0), (16, False, 0.5, 257, 193, 0),
+    (12, True, 0.5, 60, 41, 12), (16, True, 0.5, 60, 41, 16), (14, True, 0.0, 60, 41, 14)])
 def test_sphere_matches_fp32_search(qa, n, closed, t, W, H, N):
     Cdd, Cgd, gx, gy, V = _model(n, 7 * n + W)
     ras = inputs.raster(n, gx, gy, V, lo=-1.0, hi=6.0, W=W, H=H)
@@ -93,17 +102,19 @@ def test_sphere_forms(qa, form, carrier, i16):
         _same(a, b, f"{form} carrier {carrier} closed {closed}")
 
 
-@pytest.mark.parametrize("ng,closed", [(16, False), (20, False), (16, True)])
-def test_sphere_points(qa, ng, closed):
-    Cdd, Cgd, *_ = _model(16, 11, extra=ng - 16)
+@pytest.mark.parametrize("n,ng,closed", [(16, 16, False), (16, 20, False), (16, 16, True),
+                                         (4, 4, False), (7, 9, True)])
+def test_sphere_points(qa, n, ng, closed):
+    Cdd, Cgd, *_ = _model(n, 11, extra=ng - n)
     V = torch.rand((1501, ng), dtype=torch.float64, device="cuda",
                    generator=torch.Generator(device="cuda").manual_seed(3)) * 7 - 1
     a, b = _both(qa, Cdd, Cgd, lambda m: m.ground_state_points(V, closed=closed,
-                                                               n_charges=16 if closed else 0))
+                                                               n_charges=n if closed else 0))
     _same(a, b, f"points {ng}")
 
 
-@pytest.mark.parametrize("n,closed", [(13, False), (16, False), (14, True)])
+@pytest.mark.parametrize("n,closed", [(13, False), (16, False), (14, True), (4, False),
+                                      (8, False), (8, True)])
 def test_exact_ties(qa, n, closed):
     # identical, uncoupled dots, all of one charge: half-integer voltages tie
     # every pattern, more than the search lists; the rest ties none or all
