@@ -251,9 +251,9 @@ __device__ __forceinline__ PrepPixel prep_set(const ArrayDesc& a, PrepShared& sh
     if (a.sc.kind == 0) {
       int ix, iy;
       if (a.sc.P <= 0xffffffffLL) {  // 32-bit division when the raster allows it
-        const unsigned pu = (unsigned)p, W = (unsigned)a.sc.W;
-        iy = (int)(pu / W);
-        ix = (int)(pu - (unsigned)iy * W);
+        const unsigned pu = (unsigned)p, width = (unsigned)a.sc.W;
+        iy = (int)(pu / width);
+        ix = (int)(pu - (unsigned)iy * width);
       } else {
         ix = (int)(p % a.sc.W);
         iy = (int)(p / a.sc.W);
@@ -1484,125 +1484,274 @@ struct SettleScratch {
   float sh[kMaxDot];
   unsigned lst[kCloseMax];
   float rhi[2][kMaxDot], rlo[2][kMaxDot];
-  union {
-    struct {
-      __align__(16) float ptab[1 << kBnbL1];
-      float pm[kMaxDot * kLdM];
-      float vv[kMaxDot];
-    } bnb;
-    struct {
-      __align__(16) float colt[4 * kColStride];
-      __align__(16) float itab[(1 << kItMax) * kItStride];
-      __align__(16) float cslot[32][kItMax];
-    } team;
-  } u;
+  __align__(16) float ptab[1 << kBnbL1];  // the pruned search's tables
+  float pm[kMaxDot * kLdM];
+  float vv[kMaxDot];
+};
+
+// The exhaustive search's sums for a block (a pattern of the outer and middle
+// slots), by a warp: lane c < in keeps the coefficient of walked slot c, every
+// lane the block's energy A, and lane b forms inner pattern b.  The terms are
+// added in search_lane's order, so the results are its to the bit; rolled
+// loops over the set slots, because an entry's code runs once per launch on
+// cold instruction caches (search_lane itself, unrolled for registers, took
+// the list kernel of the 16-dot 257 x 193 diagram at t = 0.5 26.6 us, this
+// 16.0).
+struct SettleWarp {
+  const float* sM;
+  const int* dot;   // of each slot
+  const float* h;
+  int k, L1, in;    // slots; inner, inner + middle slots
+  int lane, mydot;
+  float v0;         // h + M / 2 of the lane's walked slot (a slot beyond k: never wins)
+
+  __device__ __forceinline__ void init(const float* M, const SlotView& sv, int l1, int l2) {
+    sM = M;
+    dot = sv.dot;
+    h = sv.h;
+    k = sv.k;
+    L1 = l1;
+    in = l1 + l2;
+    lane = threadIdx.x & 31;
+    mydot = lane < min(in, k) ? dot[lane] : 0;
+    v0 = lane < min(in, k) ? h[lane] + 0.5f * sM[mydot * (kLdM + 1)] : (lane < L1 ? kBig : 0.f);
+  }
+  // A and the lane's coefficient after the slots `bits` (each with its pair
+  // terms with those of `bits` below it)
+  __device__ __forceinline__ void add_slots(unsigned bits, float& A, float& val) const {
+#pragma unroll 1
+    for (unsigned m = bits; m; m &= m - 1u) {
+      const int s = __ffs(m) - 1;
+      const float* row = sM + dot[s] * kLdM;
+      float add = h[s] + 0.5f * row[dot[s]];
+#pragma unroll 1
+      for (unsigned l = bits & ((1u << s) - 1u); l; l &= l - 1u) add += row[dot[__ffs(l) - 1]];
+      A += add;
+      if (lane < min(in, k)) val += row[mydot];
+    }
+  }
+  // The inner pair terms of pattern `lane`, summed dot by dot.
+  __device__ __forceinline__ float pairs() const {
+    float P = 0.f;
+#pragma unroll 1
+    for (int j = 1; j < min(L1, k); ++j) {
+      if (!((lane >> j) & 1)) continue;
+      float r = 0.f;
+#pragma unroll 1
+      for (int l = 0; l < j; ++l)
+        if ((lane >> l) & 1) r += sM[dot[j] * kLdM + dot[l]];
+      P += r;
+    }
+    return P;
+  }
+  // The energy of inner pattern `lane` (+inf: not a candidate).
+  __device__ __forceinline__ float inner(float A, float val, float P, int r) const {
+    float e = A;
+#pragma unroll 1
+    for (int j = 0; j < L1; ++j) {
+      const float q = __shfl_sync(kFull, val, j);
+      if ((lane >> j) & 1) e += q;
+    }
+    e += P;
+    return (lane >> L1) != 0 || (r >= 0 && __popc((unsigned)lane) != r) ? kInf : e;
+  }
+  // The block's minimum as the walk finds it.  split: the outer slots' sums
+  // in two groups, those of the team's nlb lane bits and the others.
+  __device__ __forceinline__ float walk_min(unsigned blk, int nlb, bool split, float P,
+                                            int w) const {
+    const int L2 = in - L1;
+    const unsigned o = blk >> L2, mid = blk & ((1u << L2) - 1u);
+    const unsigned lm = split ? o & ((1u << nlb) - 1u) : o, im = o & ~lm;
+    float A = 0.f, val = v0;
+    add_slots(lm << in, A, val);
+    if (split) {
+      float A2 = 0.f, val2 = 0.f, x = 0.f;
+      add_slots(im << in, A2, val2);
+#pragma unroll 1
+      for (unsigned m = im; m; m &= m - 1u) {
+        const float* row = sM + dot[in + __ffs(m) - 1] * kLdM;
+        float c = 0.f;
+#pragma unroll 1
+        for (unsigned l = lm; l; l &= l - 1u) c += row[dot[in + __ffs(l) - 1]];
+        x += c;
+      }
+      A = (A + x) + A2;
+      val += val2;
+    }
+#pragma unroll 1
+    for (unsigned s = 1, g = 0; g != mid; ++s) {  // the Gray walk to the middle pattern
+      const int mb = __ffs(s) - 1;
+      g = s ^ (s >> 1);
+      const bool up = (g >> mb) & 1u;
+      const float gm = __shfl_sync(kFull, val, L1 + mb);
+      A = up ? A + gm : A - gm;
+      if (lane < min(in, k) && lane != L1 + mb) {
+        const float d = sM[mydot * kLdM + dot[L1 + mb]];
+        val = up ? val + d : val - d;
+      }
+    }
+    float e = inner(A, val, P, w < 0 ? -1 : max(w - __popc(blk), 0));
+    if (w >= 0 && w < __popc(blk)) e = kInf;
+    for (int off = 16; off > 0; off >>= 1) e = fminf(e, __shfl_xor_sync(kFull, e, off));
+    return e;
+  }
 };
 
 template <int N>
 struct SplitSize { static constexpr int value = N; };
+// The exhaustive search of a pixel without a list, by a warp: the same kind of
+// results over all its candidates.
+template <bool CLOSED>
+static __device__ __noinline__ void full_top2(const ArrayDesc& a, const float* sM, const SlotView sv,
+                                              const SettleWarp& sw, int nlb, bool split, float P,
+                                              float& m1, unsigned& b1, float& m2) {
+  const int lane = threadIdx.x & 31, T = a.cfg.T, k = sv.k, L1 = a.cfg.L1, L2 = a.cfg.L2;
+  m1 = m2 = kInf;
+  b1 = 0u;
+  if (T >= kTeamFinishMin) {
+    const unsigned nmid = 1u << min(max(k - L1, 0), L2), no = 1u << max(k - L1 - L2, 0);
+#pragma unroll 1
+    for (unsigned o = 0; o < no; ++o)
+#pragma unroll 1
+      for (unsigned mid = 0; mid < nmid; ++mid) {
+        const unsigned blk = (o << L2) | mid;
+        const float e = sw.walk_min(blk, nlb, split, P, sv.w);
+        if (lane == 0) {
+          m2 = fminf(m2, fmaxf(m1, e));
+          if (e < m1) {
+            m1 = e;
+            b1 = blk;
+          }
+        }
+      }
+    return;
+  }
+  unsigned long long ev = 0;
+  auto lanes = [&](auto l1, auto l2) {
+    search_lane<decltype(l1)::value, decltype(l2)::value, CLOSED, false, false, 5>(
+        sM, sv, lane, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev);
+  };
+  if (lane < T) {
+    if (L2 == 0) lanes(SplitSize<4>{}, SplitSize<0>{});
+    else if (L2 == 3) lanes(SplitSize<4>{}, SplitSize<3>{});
+    else lanes(SplitSize<5>{}, SplitSize<4>{});
+  }
+}
+
 // The FP32 search's best candidate (m1, pattern over the slots b1) and
 // runner-up m2 among the blocks of the nl listed candidates (slot patterns in
 // t.lst), or among all of them (nl = 0), with the sums that the array's search
-// takes: its split and team width say which, and lane v of that team runs in
-// lane v of the warp.
+// takes: its split and team width say which.
 template <bool CLOSED>
-static __device__ __noinline__ void listed_top2(const ArrayDesc& a, const float* sM,
-                                                const SlotView sv, SettleScratch& t, int nl,
-                                                float& m1, unsigned& b1, float& m2) {
-  const int lane = threadIdx.x & 31, T = a.cfg.T, k = sv.k;
-  const bool bnb = bnb_search(a.cfg.L1, a.cfg.L2);
-  unsigned blk = 0u;
-  if (lane < nl) blk = t.lst[lane] >> a.cfg.L1;
-  __syncwarp();
-  if (lane < nl) t.lst[lane] = blk;
-  __syncwarp();
+__device__ __forceinline__ void listed_top2(const ArrayDesc& a, const float* sM, const SlotView sv,
+                                            SettleScratch& t, int nl, float& m1, unsigned& b1,
+                                            float& m2) {
+  const int lane = threadIdx.x & 31, T = a.cfg.T, L1 = a.cfg.L1, L2 = a.cfg.L2, k = sv.k;
+  const bool bnb = bnb_search(L1, L2), tf = T >= kTeamFinishMin;
+  const int nlb = min(__ffs(T) - 1, max(k - L1 - L2, 0));  // the team's lane bits
+  unsigned blk = lane < nl ? t.lst[lane] >> L1 : 0u;
+  bool own = lane < nl;  // lane e holds block e, each block once
+  for (int e = 0; e < nl; ++e) own = own && (e >= lane || (t.lst[e] >> L1) != blk);
   m1 = m2 = kInf;
   b1 = 0u;
-  // listed: lane e takes block e, each block once
-  bool own = lane < nl;
-  for (int e = 0; e < min(lane, nl); ++e) own = own && t.lst[e] != blk;
-  const int nlb = min(__ffs(T) - 1, max(k - a.cfg.L1 - a.cfg.L2, 0));  // the team's lane bits
   if (bnb) {
-    // the tables of bnb_pair_build, an element per lane, and the inner pairs
-    float* pm = t.u.bnb.pm;
+    // the tables of bnb_pair_build, an element per lane, and the inner pairs;
+    // a block per lane
 #pragma unroll
     for (int e = lane; e < kMaxDot * kMaxDot; e += 32) {
       const int r = e >> 4, c = e & 15;
-      pm[r * kLdM + c] = (r < k && c < k) ? sM[sv.dot[r] * kLdM + sv.dot[c]] : 0.f;
+      t.pm[r * kLdM + c] = (r < k && c < k) ? sM[sv.dot[r] * kLdM + sv.dot[c]] : 0.f;
     }
     if (lane < kMaxDot)
-      t.u.bnb.vv[lane] = lane < k ? sv.h[lane] + 0.5f * sM[sv.dot[lane] * (kLdM + 1)]
-                                  : (lane < kBnbL1 ? kBig : 0.f);
+      t.vv[lane] = lane < k ? sv.h[lane] + 0.5f * sM[sv.dot[lane] * (kLdM + 1)]
+                            : (lane < kBnbL1 ? kBig : 0.f);
     __syncwarp();
-    {
-      float r = 0.f;
+    float r = 0.f;
 #pragma unroll
-      for (int j = 1; j < kBnbL1; ++j)
+    for (int j = 1; j < kBnbL1; ++j)
 #pragma unroll
-        for (int l = 0; l < j; ++l)
-          r = fmaf((((lane >> j) & 1) && ((lane >> l) & 1)) ? 1.f : 0.f, pm[j * kLdM + l], r);
-      t.u.bnb.ptab[lane] = r;
-    }
+      for (int l = 0; l < j; ++l)
+        r = fmaf((((lane >> j) & 1) && ((lane >> l) & 1)) ? 1.f : 0.f, t.pm[j * kLdM + l], r);
+    t.ptab[lane] = r;
     __syncwarp();
-    const int nout = max(k - kBnbIn, 0);
-    const unsigned nblk = nl > 0 ? (own ? 1u : 0u) : (1u << (nout + kBnbL2)), first = nl > 0 ? blk : lane;
     // (a middle pattern beyond the k slots holds no block)
     const unsigned midmax = 1u << min(max(k - kBnbL1, 0), kBnbL2);
+    const unsigned nblk = nl > 0 ? (own ? 1u : 0u) : 1u << (max(k - kBnbIn, 0) + kBnbL2);
 #pragma unroll 1
-    for (unsigned q = nl > 0 ? 0u : (unsigned)lane, b = first; q < nblk; q += 32u, b += 32u) {
+    for (unsigned q = nl > 0 ? 0u : (unsigned)lane; q < nblk; q += 32u) {
+      const unsigned b = nl > 0 ? blk : q;
       if ((b & 3u) >= midmax) continue;
-      const float e = bnb_block_min<CLOSED>(pm, t.u.bnb.vv, t.u.bnb.ptab, k, sv.w, nlb, b);
+      const float e = bnb_block_min<CLOSED>(t.pm, t.vv, t.ptab, k, sv.w, nlb, b);
       m2 = fminf(m2, fmaxf(m1, e));
       if (e < m1) {
         m1 = e;
         b1 = b;
       }
     }
-  } else if (T < kTeamFinishMin) {
-    // narrow teams: the best candidate of each of the team's lanes, of its
-    // other blocks the minimum
-    unsigned long long ev = 0;
-    const bool run = nl > 0 ? own : lane < T;
-    const unsigned v = nl > 0 ? (blk >> a.cfg.L2) & ((1u << nlb) - 1u) : (unsigned)lane;
-    float g = kInf;
-    auto lanes = [&](auto l1, auto l2) {
-      search_lane<decltype(l1)::value, decltype(l2)::value, CLOSED, false, false, 5, true>(
-          sM, sv, (int)v, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev, nullptr, nullptr, nullptr,
-          kInf, 0.f, nl > 0 ? (int)blk : -1, &g);
-    };
-    if (run) {
-      if (a.cfg.L2 == 0) lanes(SplitSize<4>{}, SplitSize<0>{});
-      else if (a.cfg.L2 == 3) lanes(SplitSize<4>{}, SplitSize<3>{});
-      else lanes(SplitSize<5>{}, SplitSize<4>{});
-    }
+  } else {
+    const bool split = tf && L1 + L2 >= 9;
+    SettleWarp sw;
+    sw.init(sM, sv, L1, L2);
+    const float P = sw.pairs();
+    if (nl == 0) full_top2<CLOSED>(a, sM, sv, sw, nlb, split, P, m1, b1, m2);
+#pragma unroll 1
     for (int e = 0; e < nl; ++e) {
-      const float ge = __shfl_sync(kFull, g, e);
-      const unsigned ve = __shfl_sync(kFull, v, e);
-      const bool oe = __shfl_sync(kFull, own ? 1 : 0, e) != 0;
-      if (own && oe && e != lane && ve == v && (ge < g || (ge == g && e < lane))) {
-        m1 = kInf;  // that block is this team lane's best
-        m2 = g;
+      const float m = sw.walk_min(__shfl_sync(kFull, blk, e), nlb, split, P, sv.w);
+      if (lane == e && own) m1 = m;
+    }
+    if (nl > 0) b1 = blk;
+    if (!tf && nl > 0) {
+      // narrow teams: the best block of each of the team's lanes (v) candidate
+      // by candidate, of its other blocks the minimum
+      const unsigned v = (blk >> L2) & ((1u << nlb) - 1u);
+      bool first = own;
+      const float g = m1;
+#pragma unroll 1
+      for (int e = 0; e < nl; ++e) {
+        const float ge = __shfl_sync(kFull, g, e);
+        const unsigned ve = __shfl_sync(kFull, v, e);
+        if (__shfl_sync(kFull, own ? 1 : 0, e) && e != lane && ve == v &&
+            (ge < g || (ge == g && e < lane)))
+          first = false;
+      }
+      if (own && !first) {
+        m2 = m1;
+        m1 = kInf;
+      }
+#pragma unroll 1
+      for (int e = 0; e < nl; ++e) {
+        if (!__shfl_sync(kFull, first ? 1 : 0, e)) continue;
+        const unsigned S = __shfl_sync(kFull, blk, e) << L1;
+        float A = 0.f, val = sw.v0;
+        sw.add_slots(S, A, val);
+        const int r = CLOSED ? sv.w - __popc(S) : -1;
+        float x1 = sw.inner(A, val, P, r), x2 = kInf;
+        if (CLOSED && r < 0) x1 = kInf;
+        unsigned xb = (unsigned)lane;
+        for (int off = 16; off > 0; off >>= 1) {
+          const float o1 = __shfl_xor_sync(kFull, x1, off), o2 = __shfl_xor_sync(kFull, x2, off);
+          const unsigned ob = __shfl_xor_sync(kFull, xb, off);
+          x2 = fminf(fminf(x2, o2), fmaxf(x1, o1));
+          if (o1 < x1 || (o1 == x1 && ob < xb)) {
+            x1 = o1;
+            xb = ob;
+          }
+        }
+        if (lane == e) {
+          m1 = x1;
+          m2 = x2;
+          b1 = S | xb;
+        }
       }
     }
-  } else {
-    // split 5 + 4: block minima from the team tables
-    constexpr int L1 = 5, L2 = 4;
-    unsigned long long ev = 0;
-    col_build<L1, L2>(sM, sv, lane, 32, t.u.team.colt);
-    iter_build<L1, L2>(sM, sv, lane, T, t.u.team.itab, 32);
-    __syncwarp();
-    const int v = nl > 0 ? (int)((blk >> L2) & ((1u << nlb) - 1u)) : lane;
-    if (nl > 0 ? own : lane < T)
-      search_lane<L1, L2, CLOSED, false, true, 5, true>(
-          sM, sv, v, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev, t.u.team.colt, t.u.team.itab,
-          t.u.team.cslot[lane], kInf, 0.f, nl > 0 ? (int)blk : -1);
   }
+#pragma unroll 1
   for (int off = 1; off < 32; off <<= 1) {
     const float o1 = __shfl_xor_sync(kFull, m1, off), o2 = __shfl_xor_sync(kFull, m2, off);
     const unsigned ob = __shfl_xor_sync(kFull, b1, off);
     top2_merge(m1, b1, m2, o1, ob, o2);
   }
-  if (T < kTeamFinishMin) return;
+  if (!tf) return;
   float e1, e2;
   unsigned fb;
   const unsigned best = m1 < kInf ? b1 : 0u;

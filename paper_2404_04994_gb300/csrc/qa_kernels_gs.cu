@@ -153,7 +153,7 @@ k_lists(const __grid_constant__ GsLaunch L) {
   // could overflow)
   const unsigned per = gridDim.x * kWarps, nlist = ntie + nflag;
   unsigned ci = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-  bool more = blockIdx.x < nclose;
+  bool more = CLOSE && blockIdx.x < nclose;
   int at = 0, left = 0;
 #pragma unroll 1
   for (unsigned it = blockIdx.x;;) {
@@ -163,7 +163,7 @@ k_lists(const __grid_constant__ GsLaunch L) {
       e = todo[at++];
       check = (e.array & kTodoRecheck) != 0;
       e.array &= ~kTodoRecheck;
-    } else if (CLOSE && more) {
+    } else if (more) {
       __syncthreads();
       if (threadIdx.x == 0) n_todo = 0;
       __syncthreads();

@@ -236,9 +236,7 @@ __device__ __forceinline__ float state_from_scratch(const float* sM,
 // sum min(0, g_m) + qneg (qneg: the model's bound of any pair-term sum, so
 // the bound holds for every candidate of the pattern) lies above lb_cut
 // holds no block to collect and is skipped.
-// ONLY: of the lane's blocks just block `only` (< 0: all); *gmin: its minimum.
-template <int L1, int L2, bool CLOSED, bool COLLECT, bool BLOCKS = false, int LANEBITS = 8,
-          bool ONLY = false>
+template <int L1, int L2, bool CLOSED, bool COLLECT, bool BLOCKS = false, int LANEBITS = 8>
 __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
                                             const SlotView sv, int t, int T,
                                             float thr, unsigned* blist,
@@ -248,8 +246,7 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
                                             const float* __restrict__ colt = nullptr,
                                             const float* __restrict__ itab = nullptr,
                                             float* __restrict__ cslot = nullptr,
-                                            float lb_cut = kInf, float qneg = 0.f,
-                                            int only = -1, float* gmin = nullptr) {
+                                            float lb_cut = kInf, float qneg = 0.f) {
   static_assert(L1 >= 2 && L1 <= 6 && L2 >= 0 && L2 <= 5, "search split");
   // block-level searches with at least 9 inner + middle slots take the
   // iteration slots' terms from the team table itab (iter_build): at most 7
@@ -378,9 +375,7 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
     }
   }
 
-  const unsigned it0 = (ONLY && only >= 0) ? ((unsigned)only >> L2) >> nlb : 0u;
-  const unsigned it1 = (ONLY && only >= 0) ? it0 + 1u : niter;
-  for (unsigned it = it0; it < it1; ++it) {
+  for (unsigned it = 0; it < niter; ++it) {
     const unsigned o = (unsigned)t | (it << nlb);
     float A = At;
     float q[L1 > 0 ? L1 : 1];
@@ -468,7 +463,6 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
             q[j] = up ? q[j] + Mim[j][mb] : q[j] - Mim[j][mb];
         }
       }
-      if (ONLY && only >= 0 && (unsigned)only != (obase | gray_c((unsigned)s))) continue;
       float mbk;
       if (!CLOSED) {
         mbk = inner_min_open<L1>(A, q, P);
@@ -492,7 +486,6 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
   }
   evaluated += (unsigned long long)niter * (unsigned)nsteps * (unsigned)NI;
   if (COLLECT) return;
-  if (ONLY && gmin) *gmin = g1;
   if (BLOCKS) {  // block level only: the team finishes the winning block
     m1 = g1;
     b1 = blk;
