@@ -1847,10 +1847,11 @@ __device__ inline int settle_entry(const GsLaunch& L, const ArrayDesc& a, const 
   const bool near = !(m2 - m1 > bound);
   const bool boundary = (flags & (kFlagBoundary | kFlagQPCap | kFlagUnresolved)) != 0u;
   // the resolve decides gaps of the energies below 1e-10 (1 + |U(base)|):
-  // leave it a hundred times that (U(base) <= U + S, and the bound is at least
-  // 24 2^-24 S)
+  // leave it four times that (U(base) <= U + S, and the bound is at least
+  // 24 2^-24 S; a wider margin would send a near tie in a hundred through the
+  // resolve, 18 us of latency in most diagrams)
   const df gap2 = df_sub(second, best);
-  const bool exact = nl > 1 && 0.5f * gap2.hi > 1e-8f * (1.f + best.hi) + 1e-2f * bound;
+  const bool exact = nl > 1 && 0.5f * gap2.hi > 4e-10f * (1.f + best.hi + bound * (16777216.f / 24.f));
   const int next = boundary ? 2 : (near && !exact) ? 1 : 0;
   // the FP32 search's candidate stands until what follows
   const bool bit = amb && ((nl == 0 || (near && next != 0)) ? (b1 >> slot) & 1u

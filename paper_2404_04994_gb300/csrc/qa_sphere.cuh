@@ -38,7 +38,8 @@ constexpr int kSphT = 16;                  // lanes per pixel
 constexpr int kSphRow = 4 * kMaxDot + 17;  // table row: four 16-entry tables; odd, and rows of
                                            // neighbouring levels start 17 banks apart
 constexpr int kSphStack = 160;             // waiting nodes per pixel
-constexpr int kSphSteps = 96;              // expansion steps per pixel at most
+constexpr int kSphRoom = 3 * kMaxDot / 2;  // what one node's descendants add at most
+constexpr int kSphSteps = 512;             // expansion steps per pixel at most
 constexpr int kSphList = 16;               // candidates within the margin that are listed
 
 // A block's copy of a model's factor: for each level k and each group g of
@@ -239,7 +240,9 @@ __device__ __forceinline__ unsigned sphere_search(const SphereConsts& g, const S
 #pragma unroll 1
     for (int step = 0; step < kSphSteps; ++step) {
       if (!__any_sync(kAll, sp > 0)) break;
-      const int take = min(sp, kSphT);
+      // as many as leave room for one node's way down (three more a level), so
+      // the stack cannot overflow
+      const int take = min(min(sp, kSphT), max(1, (kSphStack - kSphRoom - sp) / 3));
       bool valid = lt < take;
       uint2 nd = make_uint2(0u, 2u << 16);
       if (valid) nd = stk[sp - 1 - lt];
@@ -290,10 +293,6 @@ __device__ __forceinline__ unsigned sphere_search(const SphereConsts& g, const S
         if (keep && at < kSphStack)
           stk[at] = make_uint2(__float_as_uint(c[j]),
                                (nb | ((unsigned)j << (2 * p))) | ((unsigned)(p + 1) << 16));
-      }
-      if (sp > kSphStack) {  // no room: not settled
-        hard = true;
-        sp = 0;
       }
       __syncwarp();
     }
