@@ -1524,8 +1524,8 @@ static cudaError_t dispatch_soft(const SoftLaunch& a, cudaStream_t st) {
   if constexpr (!BWD) {
     return cl ? run_soft_mode<true, kDenseFwd>(a, st) : run_soft_mode<false, kDenseFwd>(a, st);
   } else {
-    if (a.fit_target)
-      return cl ? run_soft_mode<true, kDenseFit>(a, st) : run_soft_mode<false, kDenseFit>(a, st);
+    if (a.fit_target)  // up to 8 dots (beyond: k_soft_fit)
+      return cl ? run_soft_dense<true, kDenseFit>(a, st) : run_soft_dense<false, kDenseFit>(a, st);
     if (a.ctx_in)
       return cl ? run_soft_mode<true, kDenseBwdCtx>(a, st)
                 : run_soft_mode<false, kDenseBwdCtx>(a, st);

@@ -1,10 +1,12 @@
 // qa_soft_bwd.cu -- soft occupation backward pass (instantiations) and the
 // device model update.
-#include "qa_soft.cuh"
+#include "qa_soft_fit.cuh"
 
 namespace qa {
 
 cudaError_t launch_soft_backward(const SoftLaunch& a, cudaStream_t st) {
+  if (a.fit_target && a.n > kDenseMax)
+    return a.mt.closed ? run_soft_fit<true>(a, st) : run_soft_fit<false>(a, st);
   return dispatch_soft<true>(a, st);
 }
 
