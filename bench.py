@@ -242,39 +242,28 @@ def run_ours(args):
     api.qa_model_set_timing(h, False)
     st = m.stats()
     L1, L2 = st["inner_bits"], st["middle_bits"]
-    # FP32 lane-operations per evaluated inner slot: tree add + pair-term add +
-    # one comparison, plus the middle Gray step (L1 + L2 adds and a 3-op top-two
-    # update) shared by the 2^L1 slots of a block
-    ops_per_slot = 3.0 + (L1 + L2 + 3.0) / (1 << L1)
-    # the pruned search (5 + 2 split) also bounds every outer pattern of every
-    # pixel: 2^(k - 7) patterns (k = 16 ambiguous dots at t = 1), each bound
-    # A + sum_j min(0, L_j) costing about 25 FP32 lane-operations (the lane's
-    # iteration-slot pair terms ~2.5, A 2, the seven L_j 7, their minima with
-    # 0 7, the sum 6, the pair-term floor 1)
-    pruned = (L1, L2) == (5, 2)
-    ops_per_bound = 25.0
-    bounds = P * (1 << max(n_dot - L1 - L2, 0)) if pruned else 0
-    ops = st["evaluated"] * ops_per_slot + bounds * ops_per_bound
-    ms_s = statistics.mean(search_ms)
+    # FP32 lane-operations of the sphere search per evaluated child: a node's
+    # four children take two rows of four table sums and the centre (10), the
+    # three further row sums (3), six squares with their additions (12) and
+    # three gradient terms
+    ops_per_child = 28.0 / 4.0
+    ops = st["evaluated"] * ops_per_child
+    ms_s = statistics.mean(a + b for a, b in zip(prep_ms, search_ms))
     achieved = ops / (ms_s * 1e-3) / 1e12
     sm_max = (clk.get("sm_max_mhz") or peaks.get("sm_max_mhz") or 2070.0)
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
     peak = n_sm * 128 * sm_max * 1e6 / 1e12   # FP32 lanes x clock
-    # the same diagram searched exhaustively by the split walk (every one of
-    # the 2^16 candidates at 3.375 lane-operations): what the pruning saves
+    # the same diagram searched exhaustively (every one of the 2^16 candidates
+    # at the split walk's 3.375 lane-operations): what the search saves
     exh = st["candidates"] * 3.375 / (ms_s * 1e-3) / 1e12
     roofline = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak, 3),
                 "unit": "Tops/s", "frac": round(achieved / peak, 4), "traffic": search_traffic(),
-                "kernel": ("k_ground_state_bnb<open> (prep + pruned search of each tile)"
-                           if pruned else f"k_ground_state<{L1},{L2},open> (prep + search)"),
-                "ops_per_launch": ops,
-                "ops_per_evaluated_slot": ops_per_slot,
-                "bounds_per_launch": bounds, "ops_per_bound": ops_per_bound,
+                "kernel": "k_pixels<16,open,sphere> (prep, sphere search and outputs)",
+                "ops_per_launch": ops, "ops_per_evaluated_child": ops_per_child,
                 "exhaustive_equivalent_tops": round(exh, 3),
-                # k_ground_state runs the prep and the search of each tile, so
-                # its time covers both; the separate prep kernel does not run
+                # one kernel prepares and searches: the events put its time in
+                # the first of the two intervals
                 "kernel_ms": round(ms_s, 5),
-                "separate_prep_ms": round(statistics.mean(prep_ms), 5),
                 "resolve_recheck_ms": round(statistics.mean(recheck_ms), 5),
                 "peak_basis": f"{n_sm} SMs x 128 FP32 lanes x {sm_max:.0f} MHz (of nominal "
                               "unit counts and max clock; MEASURED_PEAKS.json has no FP32 figure)"}
@@ -346,8 +335,8 @@ def run_ours(args):
             "roofline": roofline, "cpu_baseline": cpu,
             "e2e": {"value": world * P / e2e_s, "unit": UNIT,
                     "h2d_bytes_per_step": int(bi), "d2h_bytes_per_step": int(bo)},
-            # per step: k_ground_state_bnb (prep + pruned search of each
-            # tile) and k_lists (near-tie resolve and FP64 recheck)
+            # per step: k_pixels (prep, search and outputs) and k_lists (close
+            # candidates, near-tie resolve and FP64 recheck)
             "gpu_launches": 2 * args.steps, "clocks": clk, "extra": extra}
     if rank == 0:
         print(json.dumps(line))
