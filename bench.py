@@ -107,8 +107,8 @@ def search_traffic():
         return None
     csrc = os.path.join(ROOT, "paper_2404_04994_gb300", "csrc")
     h = hashlib.sha256()
-    for f in ("qa_search.cuh", "qa_gs_tiles.cuh", "qa_kernels_gs.cu", "qa_device.cuh",
-              "qa_prep.cuh"):
+    for f in ("qa_search.cuh", "qa_sphere.cuh", "qa_gs_tiles.cuh", "qa_pixels.cu",
+              "qa_kernels_gs.cu", "qa_device.cuh", "qa_prep.cuh"):
         h.update(open(os.path.join(csrc, f), "rb").read())
     return int(m_traf.group(1)) if h.hexdigest()[:16] == m_hash.group(1) else None
 
