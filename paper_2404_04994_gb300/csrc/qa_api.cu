@@ -222,6 +222,9 @@ void fill_consts(int n, qa::ModelData* md) {
   fill_sphere(n, md);
 }
 
+// ModelData::gen of the host copy that makes a model's generation `gen`.
+unsigned host_gen(unsigned long long gen) { return (unsigned)(gen % 0xffffffffull) + 1u; }
+
 // Validate + convert host matrices into a ModelData (Maxwell form).
 int build_model(int n, int ng, int form, const double* Cdd_in,
                 const double* Cgd_in, qa::ModelData* md) {
@@ -437,7 +440,7 @@ qa::RasterK raster_constants(const qa_model* m, const qa::Scan& sc) {
     rk.du[i] = split(b);
     rk.dw[i] = split(c);
   }
-  rk.valid = 1;
+  rk.gen = m->host.gen;
   return rk;
 }
 
@@ -809,6 +812,7 @@ int qa_model_create(const double* Cdd, const double* Cgd, int n_dot, int n_gate,
   qa_model* m = new qa_model();
   int rc = build_model(n_dot, n_gate, form, Cdd, Cgd, &m->host);
   if (rc) { delete m; return rc; }
+  m->host.gen = host_gen(m->gen);
   m->n = n_dot;
   m->ng = n_gate;
   m->form = form;
@@ -833,6 +837,7 @@ int qa_model_update(qa_model* m, const double* Cdd, const double* Cgd) {
   qa::ModelData md;
   int rc = build_model(m->n, m->ng, m->form, Cdd, Cgd, &md);
   if (rc) return rc;
+  md.gen = host_gen(m->gen + 1);
   if ((rc = select_device(m))) return rc;
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess)
@@ -858,6 +863,7 @@ int qa_model_update_async(qa_model* m, const double* Cdd, const double* Cgd, voi
     if (e != cudaSuccess) return cuda_fail(e, "staging buffer");
   }
   if ((rc = build_model(m->n, m->ng, m->form, Cdd, Cgd, m->staging))) return rc;
+  m->staging->gen = host_gen(m->gen + 1);
   e = cudaMemcpyAsync(m->d_md, m->staging, sizeof(qa::ModelData), cudaMemcpyHostToDevice,
                       (cudaStream_t)stream);
   if (e == cudaSuccess) e = cudaEventRecord(m->staged, (cudaStream_t)stream);

@@ -139,7 +139,7 @@ struct __align__(16) ModelData {
   double vs[kMaxDot];                 // Cdd 1 / (1^T Cdd 1)   (Appendix D)
   double cond;                        // ||Cdd||_1 ||M||_1
   int status;                         // 0 ok; nonzero: Cdd not PD on update
-  int pad;
+  unsigned gen;                       // which host copy this is; 0: updated on the device
   ModelConsts k;                      // FP32 forms of the above
   SphereConsts s;
 };
@@ -155,9 +155,11 @@ struct Scan {
 };
 
 // Raster induced-charge constants c0, du, dw (double-float), computed on the
-// host when the host copy of the model is current.
+// host when the host copy of the model is current.  A launch that runs after
+// the model changed (a batch's next run, the replay of a graph) finds another
+// `gen` in the model and forms them from the device copy instead.
 struct RasterK {
-  int valid;
+  unsigned gen;  // ModelData::gen of the host copy they come from; 0: none
   int pad;
   df c0[kMaxDot], du[kMaxDot], dw[kMaxDot];
 };

@@ -127,6 +127,7 @@ struct PrepShared {
 // Stage an array's FP32 model constants and raster constants (all threads);
 // one thread converts the FP64 threshold for the whole block.
 __device__ inline void prep_stage_array(const ArrayDesc& a, PrepShared& sh) {
+  const bool rk = a.rk.gen != 0u && a.rk.gen == a.md->gen;
   stage_consts(&a.md->k, &sh.cs);
   if (threadIdx.x == 0) {
     sh.th0 = __double2float_rn(0.5 * a.mt.t);
@@ -139,7 +140,7 @@ __device__ inline void prep_stage_array(const ArrayDesc& a, PrepShared& sh) {
     }
   }
   if (a.sc.kind == 0) {
-    if (a.rk.valid) {
+    if (rk) {
       if (threadIdx.x < kMaxDot) {
         sh.sc0[threadIdx.x] = a.rk.c0[threadIdx.x];
         sh.sdu[threadIdx.x] = a.rk.du[threadIdx.x];

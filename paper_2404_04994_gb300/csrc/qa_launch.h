@@ -27,7 +27,7 @@ struct ArrayDesc {
   const ModelData* md;
   int n, ng;
   Scan sc;
-  RasterK rk;          // host-computed raster constants (rk.valid = 0: device)
+  RasterK rk;          // host-computed raster constants
   Method mt;
   SearchCfg cfg;
   int prep_team;       // lanes per pixel in the prep stage (pow2 >= n, <= 16)

@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
   if (!ok) {
     if (tid == 0) {
       md->status = 1;
+      md->gen = 0u;
       md->k.model_bad = 1;
       md->s.valid = 0;
     }
@@ -130,6 +131,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
     if (tid == 0) {
       md->cond = cond;
       md->status = 0;
+      md->gen = 0u;
       kc.s_s = __double2float_rn(tot);
       const double e1 = cond * (n + 1) * 5.9604644775390625e-8;
       kc.bx_qp_scale = __double2float_rn(8.0 * e1);

@@ -155,3 +155,49 @@ def test_autotuned_batch_matches_oracle_at_the_tuned_thresholds(qa):
                 f.cpu().numpy().reshape(-1), rec, sp["Cdd"],
                 f"tuned N={nd} t={sp['threshold']:.3f} team={sp['team']}", closed=sp["closed"])
     b.close()
+
+
+def test_batch_and_graph_see_a_model_update(qa):
+    # capacitances may change between a batch's runs: the next run, and the
+    # replay of a captured one, take the new Cgd with the new M
+    import torch
+    old, new = _mixed_specs(15, sides=(23,), seed=7), _mixed_specs(15, sides=(23,), seed=7)
+    r = np.random.Generator(np.random.PCG64(1))
+    for sp in new:
+        sp["Cdd"] = sp["Cdd"] + 0.1 * np.diag(r.random(sp["Cdd"].shape[0]))
+        sp["Cgd"] = sp["Cgd"] * r.uniform(0.6, 1.4, sp["Cgd"].shape)
+    want = []
+    for sp in new:
+        m = qa.Model(sp["Cdd"], sp["Cgd"])
+        call = m.ground_state_closed if sp["closed"] else m.ground_state_open
+        arg = (sp["n_charges"],) if sp["closed"] else ()
+        n, U, _ = call(sp["raster"], *arg, threshold=sp["threshold"])
+        want.append((n.cpu().numpy(), U.cpu().numpy().reshape(n.shape[:2])))
+        m.close()
+
+    def check(label):
+        torch.cuda.synchronize()
+        for (n, U, _), (n0, U0) in zip(b.outputs, want):
+            np.testing.assert_array_equal(n.cpu().numpy(), n0, err_msg=label)
+            np.testing.assert_allclose(U.cpu().numpy(), U0, rtol=1e-9, atol=1e-12, err_msg=label)
+
+    b = qa.Batch(old)
+    b.run()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        b.run()
+    for m, sp in zip(b.models, new):
+        qa.qa_model_update(m.handle, sp["Cdd"], sp["Cgd"])
+    b.run()
+    check("run after an update")
+    for o in b.outputs:
+        o[0].fill_(-1)
+    g.replay()
+    check("replay after an update")
+    for m, sp in zip(b.models, new):
+        qa.qa_model_update_dev(m.handle, torch.tensor(sp["Cdd"], device="cuda"),
+                               torch.tensor(sp["Cgd"], device="cuda"))
+    g.replay()
+    check("replay after an update on the device")
+    b.close()
