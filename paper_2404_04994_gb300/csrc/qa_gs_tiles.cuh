@@ -1268,7 +1268,18 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
 #pragma unroll
   for (int off = W / 2; off > 0; off >>= 1) S += __shfl_xor_sync(kFull, S, off);
   const unsigned any_qp = __any_sync(kFull, qp);
+  // max_j |base_j - c_j|, |x_j - c_j|, which scales the rounding of M r: at most
+  // 1 on an open pixel without active constraints (x = c), but a closed one
+  // moves every dot by lambda v
   float rmax = 1.f;
+  if (CLOSED || any_qp) {
+    rmax = fmaxf(fabsf(r0), fabsf(sh.p.qz[threadIdx.x]));
+#pragma unroll
+    for (int off = W / 2; off > 0; off >>= 1)
+      rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
+    rmax = fmaxf(rmax, 1.f);
+  }
+  const float ez = u24 * a.md->s.msum * rmax;  // u sum |M| |r|
   int close = 0;
   unsigned ev = 0, bits = 0u;
   const bool sphere =
@@ -1281,7 +1292,6 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
       float z = 0.f;
 #pragma unroll
       for (int j = 0; j < W; ++j) z = fmaf(Mrow[j], sh.p.qz[tq + j], z);
-      rmax = fmaxf(fabsf(r0), fabsf(sh.p.qz[threadIdx.x]));
       if (CLOSED) {  // the multiple of 1: the least entry, a free dot's
         float zm = q.live ? z : kInf;
 #pragma unroll
@@ -1291,12 +1301,8 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
       a1 = (qp && amb) ? fmaxf(z, 0.f) : 0.f;
       neg = (qp && amb) ? fmaxf(-z, 0.f) : 0.f;
 #pragma unroll
-      for (int off = W / 2; off > 0; off >>= 1) {
-        neg += __shfl_xor_sync(kFull, neg, off);
-        rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
-      }
+      for (int off = W / 2; off > 0; off >>= 1) neg += __shfl_xor_sync(kFull, neg, off);
     }
-    const float ez = u24 * a.md->s.msum * fmaxf(rmax, 1.f);  // u sum |M| |r|
     const float bound = pixel_bound(a, S * 1.00001f + 20.f * ez, k);
     neg += (qp ? 24.f : 2.f) * ez;
     // no factor, or a centre outside [-1, 1] (an unsettled QP): left to the
@@ -1311,13 +1317,6 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
   unsigned* lst =
       reinterpret_cast<unsigned*>(MODE == kPixDense ? &sh.p.qK[tq][0] : &sh.p.qz[tq]);
   if constexpr (MODE != kPixSphere) if (!sphere) {
-    if (any_qp) {
-      rmax = fabsf(r0);
-#pragma unroll
-      for (int off = W / 2; off > 0; off >>= 1)
-        rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
-    }
-    const float ez = u24 * a.md->s.msum * fmaxf(rmax, 1.f);
     // twice the near-tie bound as in the sphere search, once more for this
     // search's own sums (at most 2 k + 8 additions), and the error of the
     // plain h on both sides

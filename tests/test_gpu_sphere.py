@@ -142,3 +142,28 @@ def test_exact_ties(qa, n, closed):
                                    atol=1e-12)
     np.testing.assert_allclose(a[1], b[1], rtol=1e-11, atol=1e-12)
     np.testing.assert_array_equal(a[2], b[2])
+
+
+@pytest.mark.parametrize("n,a,N,t", [(4, 0.999, 20000, 1.0), (6, 0.99, 30000, 1.0),
+                                     (8, 0.999, 50000, 1.0), (8, 0.999, 50000, 0.5),
+                                     (11, 0.999, 60000, 0.6), (12, 0.999, 60000, 0.5),
+                                     (14, 0.999, 60000, 1.0)])
+def test_closed_far_from_the_induced_charge(qa, n, a, N, t):
+    # a closed array whose total is far from sum c (lambda large, no dot at
+    # zero) and whose off-diagonal capacitances are positive, so that h = M r
+    # cancels: the FP32 rounding of h is 10^3 u |h| and more.  U is large
+    # against its gaps: energies to the rounding of the double-float sum,
+    # 2^-44 sum |r| |M| |r|
+    r = np.random.Generator(np.random.PCG64(n))
+    Cdd = (1.0 - a) * np.diag(r.uniform(0.8, 1.2, n)) + a
+    Cgd = inputs.dense_cgd(r, n)
+    ras = inputs.raster(n, *inputs.swept_gates(n), r.uniform(1.0, 3.0, n), lo=0.0, hi=3.0,
+                        W=100, H=60)
+    x, y = _both(qa, Cdd, Cgd, lambda m: m.ground_state_i16(ras, threshold=t, closed=True,
+                                                            n_charges=N))
+    assert (x[0].astype(np.int64).sum(-1) == N).all()
+    assert not (x[2] & 4).any()
+    np.testing.assert_array_equal(x[0], y[0])
+    np.testing.assert_array_equal(x[2], y[2])
+    mag = np.abs(np.linalg.inv(Cdd)).sum() * (2.0 * N / n) ** 2
+    np.testing.assert_allclose(x[1], y[1], rtol=0, atol=2.0 ** -44 * mag)
