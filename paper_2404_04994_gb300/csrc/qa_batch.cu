@@ -130,15 +130,18 @@ void batch_occupancy(int* prep_per_sm, int* search_per_sm) {
 cudaError_t launch_ground_state_batch(const GsLaunch& L, cudaStream_t st) {
   if (L.ev) cudaEventRecord(L.ev[0], st);
   cudaMemsetAsync(L.cnt, 0, sizeof(Counters), st);
-  launch_pixels_batch(L, st);
+  // each stage's own error: a launcher that reports one has cleared it
+  cudaError_t e = launch_pixels_batch(L, st);
+  if (e != cudaSuccess) return e;
   if (L.n_prep_units > 0) k_prep_batch<<<L.grid_prep, kPrepThreads, 0, st>>>(L);
   if (L.ev) cudaEventRecord(L.ev[1], st);
   for (int v = 0; v < kBatchVariants; ++v)
     if (L.var_count[v] > 0) batch_search_kernel(v)<<<L.var_grid[v], kSearchThreads, 0, st>>>(L, v);
   if (L.ev) cudaEventRecord(L.ev[2], st);
-  launch_lists(L, st);
+  e = launch_lists(L, st);
   if (L.ev) cudaEventRecord(L.ev[3], st);
-  return cudaGetLastError();
+  const cudaError_t last = cudaGetLastError();
+  return e != cudaSuccess ? e : last;
 }
 
 }  // namespace qa

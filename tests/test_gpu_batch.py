@@ -201,3 +201,30 @@ def test_batch_and_graph_see_a_model_update(qa):
     g.replay()
     check("replay after an update on the device")
     b.close()
+
+
+@pytest.mark.parametrize("launcher", ["_ZN2qa19launch_pixels_batchERKNS_8GsLaunchEP11CUstream_st",
+                                      "_ZN2qa12launch_listsERKNS_8GsLaunchEP11CUstream_st"])
+def test_batch_reports_the_error_of_each_stage(tmp_path, launcher):
+    # a stand-in for one launcher that launches nothing and fails
+    import os
+    import shutil
+    import subprocess
+    import sys
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no g++")
+    src = tmp_path / "fail.cpp"
+    src.write_text(f'extern "C" int {launcher}(const void*, void*) {{ return 1; }}\n')
+    lib = tmp_path / "fail.so"
+    subprocess.check_call([gxx, "-shared", "-fPIC", "-o", str(lib), str(src)])
+    code = ("import numpy as np\n"
+            "from paper_2404_04994_gb300 import api, inputs\n"
+            "ras = inputs.raster(4, 0, 1, np.ones(4), W=9, H=7)\n"
+            "b = api.Batch([dict(Cdd=np.eye(4), Cgd=np.eye(4), raster=ras)])\n"
+            "try:\n    b.run()\nexcept api.QAError as e:\n    print('code', e.code)\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, LD_PRELOAD=str(lib), PYTHONPATH=root)
+    r = subprocess.run([sys.executable, "-c", code], env=env, cwd=root, capture_output=True,
+                       text=True, timeout=300)
+    assert r.stdout.strip() == "code -7", r.stdout + r.stderr
