@@ -1467,10 +1467,15 @@ static cudaError_t run_soft_wide(const SoftLaunch& a, cudaStream_t st) {
   constexpr int teams = kSoftThreads / 32;
   const unsigned grid = (unsigned)((a.sc.P + teams - 1) / teams);
   const size_t smem = WideSmem<NIT>(BWD, contrib_len(a.n)).total;
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      k_soft_wide<CLOSED, MODE, NIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      (int)WideSmem<NIT>(BWD, contrib_len(kMaxDot)).total);
-  if (attr != cudaSuccess) return attr;
+  // the backward of 13 to 16 dots takes more than the default limit, which
+  // belongs to the current device and context: raised on each of its calls, to
+  // the largest size, so that calls of other threads need no more
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_soft_wide<CLOSED, MODE, NIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)WideSmem<NIT>(BWD, contrib_len(kMaxDot)).total);
+    if (e != cudaSuccess) return e;
+  }
   if (a.ev) cudaEventRecord(a.ev[0], st);
   k_soft_wide<CLOSED, MODE, NIT><<<grid, kSoftThreads, smem, st>>>(a);
   if (BWD) k_soft_reduce<<<contrib_len(a.n), 256, 0, st>>>(a, (int)grid);

@@ -1,0 +1,131 @@
+"""The library's host path on a machine of several GPUs, without one: its
+objects linked against a stand-in for the CUDA runtime whose memory is host
+memory and whose kernels do nothing.  It keeps the attributes of each device's
+kernels, and refuses a launch that asks for more dynamic shared memory than
+they allow, as the runtime does."""
+import glob
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+from paper_2404_04994_gb300 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+RUNTIME = r"""
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <utility>
+#define API extern "C" __attribute__((visibility("default")))
+struct dim3 { unsigned x, y, z; };
+static int dev = 0, last = 0;
+static std::map<std::pair<int, const void*>, int> limit;  // dynamic shared memory
+static dim3 grid, block;
+static size_t smem;
+static void* stream;
+static int fail(int e) { return last = e; }
+static int launch(const void* f, size_t bytes) {
+  auto it = limit.find({dev, f});
+  return bytes > (it == limit.end() ? 48 * 1024 : (size_t)it->second) ? fail(1) : 0;
+}
+API int cudaGetDevice(int* d) { *d = dev; return 0; }
+API int cudaSetDevice(int d) { dev = d; return 0; }
+API int cudaFuncSetAttribute(const void* f, int attr, int v) {
+  if (attr == 8) limit[{dev, f}] = v;
+  return 0;
+}
+API unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t s, void* st) {
+  grid = g; block = b; smem = s; stream = st;
+  return 0;
+}
+API int __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* s, void* st) {
+  *g = grid; *b = block; *s = smem; *(void**)st = stream;
+  return 0;
+}
+API int __cudaGetKernel(void** k, const void* f) { *k = (void*)f; return 0; }
+API int __cudaLaunchKernel(void* k, dim3, dim3, void**, size_t s, void*) { return launch(k, s); }
+struct Config { dim3 g, b; size_t s; };
+API int cudaLaunchKernelExC(const Config* c, const void* f, void**) { return launch(f, c->s); }
+API int cudaGetLastError() { int e = last; last = 0; return e; }
+API const char* cudaGetErrorString(int) { return "error"; }
+API int cudaMalloc(void** p, size_t n) { *p = calloc(n, 1); return 0; }
+API int cudaHostAlloc(void** p, size_t n, unsigned) { *p = calloc(n, 1); return 0; }
+API int cudaFree(void* p) { free(p); return 0; }
+API int cudaFreeHost(void* p) { free(p); return 0; }
+API int cudaMemcpy(void* d, const void* s, size_t n, int) { memcpy(d, s, n); return 0; }
+API int cudaMemcpyAsync(void* d, const void* s, size_t n, int, void*) { memcpy(d, s, n); return 0; }
+API int cudaMemset(void* d, int v, size_t n) { memset(d, v, n); return 0; }
+API int cudaMemsetAsync(void* d, int v, size_t n, void*) { memset(d, v, n); return 0; }
+API int cudaDeviceGetAttribute(int* v, int, int) { *v = 152; return 0; }
+API int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t,
+                                                               unsigned) { *n = 1; return 0; }
+API int cudaGetSymbolAddress(void** p, const void* s) { *p = (void*)s; return 0; }
+API int cudaDeviceSynchronize() { return 0; }
+API int cudaStreamSynchronize(void*) { return 0; }
+API int cudaEventCreate(void** e) { *e = &dev; return 0; }
+API int cudaEventCreateWithFlags(void** e, unsigned) { *e = &dev; return 0; }
+API int cudaEventDestroy(void*) { return 0; }
+API int cudaEventRecord(void*, void*) { return 0; }
+API int cudaEventSynchronize(void*) { return 0; }
+API int cudaEventElapsedTime(float* t, void*, void*) { *t = 0.f; return 0; }
+API void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
+API void __cudaRegisterFatBinaryEnd(void**) {}
+API void __cudaUnregisterFatBinary(void**) {}
+API void __cudaRegisterFunction(void**, const char*, char*, const char*, int, void*, void*, void*,
+                                void*, int*) {}
+API void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
+"""
+
+
+@pytest.fixture(scope="module")
+def library(tmp_path_factory):
+    objs = sorted(glob.glob(os.path.join(build.OUT_DIR, "*.o")))
+    gxx = shutil.which("g++")
+    if gxx is None or not objs or build.stale():
+        pytest.skip("needs g++ and the objects of an up-to-date build")
+    d = tmp_path_factory.mktemp("host_path")
+    (d / "runtime.cpp").write_text(RUNTIME)
+    lib = str(d / "libqarray_host.so")
+    subprocess.check_call([gxx, "-std=c++17", "-shared", "-fPIC", "-o", lib, *objs,
+                           str(d / "runtime.cpp")])
+    return lib
+
+
+def _run(library, code):
+    env = dict(os.environ, QARRAY_LIB=library, PYTHONPATH=ROOT)
+    r = subprocess.run([sys.executable, "-c", code], env=env, cwd=ROOT, capture_output=True,
+                       text=True, timeout=120)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout.split()
+
+
+@pytest.mark.parametrize("n", [8, 12, 13, 16])
+def test_soft_calls_on_each_device(library, n):
+    # the backward of 13 to 16 dots needs more than the default limit, on
+    # whichever device it runs
+    out = _run(library, f"""
+import ctypes
+import numpy as np
+from paper_2404_04994_gb300 import api, inputs
+lib, n = api.load(), {n}
+r = np.random.Generator(np.random.PCG64(2))
+Cdd, Cgd = inputs.chain_cdd(r, n), inputs.dense_cgd(r, n)
+ras = api.make_raster(inputs.raster(n, 0, 1, np.ones(n), W=8, H=4), n)
+g, d = np.ones((32, n), dtype=np.float32), np.zeros((n, n))
+for dev in (0, 1, 0):
+    lib.cudaSetDevice(dev)
+    m = api.qa_model_create(Cdd, Cgd)
+    for rc in (lib.qa_soft_occupation(m, ctypes.byref(ras), 0.05, 1.0, 0, 0, g.ctypes.data, None,
+                                      None),
+               lib.qa_soft_occupation_backward(m, ctypes.byref(ras), 0.05, 1.0, 0, 0,
+                                               g.ctypes.data, d.ctypes.data, d.ctypes.data, None),
+               lib.qa_soft_occupation_backward(m, ctypes.byref(ras), 0.05, 1.0, 1, n,
+                                               g.ctypes.data, d.ctypes.data, d.ctypes.data, None)):
+        print(rc)
+    api.qa_model_destroy(m)
+""")
+    assert out == ["0"] * 9
