@@ -370,8 +370,9 @@ typedef struct {
     double threshold;     /* Eq. "threshold", [0, 1]                          */
     int closed;           /* 0 open, 1 closed with n_charges carriers         */
     int n_charges;
-    int team;             /* lanes per pixel of the search (1..32, power of
-                             two); 0 = the library's choice                   */
+    int team;             /* lanes per pixel of the search by tiles (1..32,
+                             power of two; at least 16 where the pruned search
+                             runs); 0 = the library's choice of search        */
     int8_t* out_n;        /* DEVICE [H, W, n_dot]                              */
     double* out_U;        /* DEVICE [H, W] (nullable)                          */
     uint8_t* out_flags;   /* DEVICE [H, W] (nullable)                          */

@@ -10,8 +10,11 @@ sample rasters of the group; the smallest admitted value wins, else t = 1.
 The chosen t is an output of the tuning and the batch is then exact with
 respect to the method at that t (the oracle is run at the same t).
 
-Team: every power of two from 1 to 32 is timed on the sample at the chosen
-t (CUDA events, median of a few runs) and the fastest wins.
+Team: the library's own choice (0: for most arrays a search with lanes of its
+own) and every power of two from 1 to 32 are timed at the chosen t (CUDA
+events, median of a few runs) and the fastest wins.  The sample is repeated
+until its pixels fill the GPU, as the batch does: a few small arrays alone time
+launches.
 
 The decision logic takes a ``runner(specs, reps) -> (maps, ms)`` so that it can
 be exercised on the CPU with a fake; the default runner drives the library's
@@ -24,7 +27,8 @@ import math
 
 import numpy as np
 
-TEAMS = (1, 2, 4, 8, 16, 32)
+TEAMS = (0, 1, 2, 4, 8, 16, 32)
+TIMED_PIXELS = 32768  # about four to each team of lanes the GPU holds
 
 
 def delta_matrix(Cdd):
@@ -82,9 +86,10 @@ def tune(specs, runner=None, sample_side=24, arrays_per_group=4, teams=TEAMS, re
                 chosen = t
                 break
             rejected[t] = bad
+        copies = -(-TIMED_PIXELS // sum(b["raster"]["W"] * b["raster"]["H"] for b in base))
         team_ms = {}
         for T in teams:
-            _, ms = runner([dict(b, threshold=chosen, team=T) for b in base], reps)
+            _, ms = runner([dict(b, threshold=chosen, team=T) for b in base] * copies, reps)
             team_ms[T] = ms
         best_team = min(team_ms, key=lambda T: (team_ms[T], T))
         table[key] = {"threshold": chosen, "team": int(best_team), "arrays": idx,

@@ -1400,7 +1400,8 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
     if (qa::bnb_search(d.cfg.L1, d.cfg.L2) && d.cfg.T < qa::kBnbMinT)
       d.cfg.T = qa::kBnbMinT;
     d.klass = qa::search_klass(d.cfg);
-    d.search = choose_search(m, d, 1LL << 40);
+    // (a width asked for is the tile search's, the one that has a choice of it)
+    d.search = it.team ? (int)qa::kSearchTiles : choose_search(m, d, 1LL << 40);
     d.prep_team = prep_team(m->n);
     d.bx_analytic = 4.0e-7f;
     d.bx_qp_scale = 0.f;

@@ -1,8 +1,8 @@
 """The library's host path on a machine of several GPUs, without one: its
 objects linked against a stand-in for the CUDA runtime whose memory is host
 memory and whose kernels do nothing.  It keeps the attributes of each device's
-kernels, and refuses a launch that asks for more dynamic shared memory than
-they allow, as the runtime does."""
+kernels, refuses a launch that asks for more dynamic shared memory than they
+allow, as the runtime does, and lists what was launched."""
 import glob
 import os
 import shutil
@@ -19,6 +19,7 @@ RUNTIME = r"""
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <string>
 #include <utility>
 #define API extern "C" __attribute__((visibility("default")))
 struct dim3 { unsigned x, y, z; };
@@ -28,7 +29,19 @@ static dim3 grid, block;
 static size_t smem;
 static void* stream;
 static int fail(int e) { return last = e; }
+static std::map<const void*, std::string>& names() {  // filled while the library loads
+  static auto* m = new std::map<const void*, std::string>;
+  return *m;
+}
+static std::string& log_ = *new std::string;
+API const char* launched() {
+  static std::string s;
+  s.swap(log_);
+  log_.clear();
+  return s.c_str();
+}
 static int launch(const void* f, size_t bytes) {
+  log_ += names()[f] + " ";
   auto it = limit.find({dev, f});
   return bytes > (it == limit.end() ? 48 * 1024 : (size_t)it->second) ? fail(1) : 0;
 }
@@ -75,8 +88,8 @@ API int cudaEventElapsedTime(float* t, void*, void*) { *t = 0.f; return 0; }
 API void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
 API void __cudaRegisterFatBinaryEnd(void**) {}
 API void __cudaUnregisterFatBinary(void**) {}
-API void __cudaRegisterFunction(void**, const char*, char*, const char*, int, void*, void*, void*,
-                                void*, int*) {}
+API void __cudaRegisterFunction(void**, const char* f, char*, const char* name, int, void*, void*,
+                                void*, void*, int*) { names()[f] = name; }
 API void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 """
 
@@ -129,3 +142,34 @@ for dev in (0, 1, 0):
     api.qa_model_destroy(m)
 """)
     assert out == ["0"] * 9
+
+
+@pytest.mark.parametrize("team", [0, 1, 4, 8, 32])
+def test_batch_item_team_is_the_tile_search(library, team):
+    # lanes asked for are lanes of the search by tiles; the library's own
+    # choice is a one-pass kernel for arrays of 3 dots and more
+    out = _run(library, f"""
+import ctypes
+import numpy as np
+from paper_2404_04994_gb300 import api, inputs
+lib = api.load()
+lib.launched.restype = ctypes.c_char_p
+for n in (3, 5, 8, 11, 12, 16):
+    for closed in (0, 1):
+        for t in (0.5, 1.0):
+            r = np.random.Generator(np.random.PCG64(2))
+            item = api.qa_batch_item()
+            m = api.qa_model_create(inputs.chain_cdd(r, n), inputs.dense_cgd(r, n))
+            out = np.zeros((32, n), dtype=np.int8)
+            item.model, item.out_n = m.value, out.ctypes.data
+            ras = api.make_raster(inputs.raster(n, 0, 1, np.ones(n), W=8, H=4), n)
+            item.raster, item.threshold, item.closed, item.n_charges = ras, t, closed, n
+            item.team = {team}
+            b = ctypes.c_void_p()
+            assert lib.qa_batch_create(ctypes.byref(item), 1, ctypes.byref(b)) == 0
+            assert lib.qa_batch_run(b, None) == 0
+            names = lib.launched().decode()
+            print(int("k_pixels_batch" in names), int("k_search_batch" in names))
+""")
+    pairs = set(zip(out[::2], out[1::2]))
+    assert pairs == {("0", "1")} if team else ("1", "0") in pairs
