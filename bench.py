@@ -261,8 +261,7 @@ def run_ours(args):
                 "kernel": "k_pixels<16,open,sphere> (prep, sphere search and outputs)",
                 "ops_per_launch": ops, "ops_per_evaluated_child": ops_per_child,
                 "exhaustive_equivalent_tops": round(exh, 3),
-                # one kernel prepares and searches: the events put its time in
-                # the first of the two intervals
+                # one kernel prepares and searches
                 "kernel_ms": round(ms_s, 5),
                 "resolve_recheck_ms": round(statistics.mean(recheck_ms), 5),
                 "peak_basis": f"{n_sm} SMs x 128 FP32 lanes x {sm_max:.0f} MHz (of nominal "
@@ -454,7 +453,8 @@ def search_profile(api, m, fn, flush, tag):
     api.qa_model_set_timing(m.handle, False)
     st = m.stats()
     L1, L2 = st["inner_bits"], st["middle_bits"]
-    ops = st["evaluated"] * (3.0 + (L1 + L2 + 3.0) / (1 << L1))
+    # (no inner slots: the sphere search, 7 operations a child as above)
+    ops = st["evaluated"] * (3.0 + (L1 + L2 + 3.0) / (1 << L1) if L1 else 7.0)
     ms = statistics.mean(ks)
     return {f"{tag}_candidates": st["candidates"], f"{tag}_evaluated_slots": st["evaluated"],
             f"{tag}_search_ms": ms, f"{tag}_prep_ms": statistics.mean(kp),

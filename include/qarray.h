@@ -111,10 +111,11 @@ typedef struct {
     long long resolved;        /* near ties settled by exact double-float    */
     int team;                  /* lanes per pixel used by the search kernel   */
     int inner_bits;            /* unrolled inner / middle bits of the search  */
-    int middle_bits;
+    int middle_bits;           /* (both 0: the sphere search has none)        */
     int timed;                 /* 1 when the ms_* fields below are valid      */
     double ms_prep;            /* device time of each kernel of the last call */
-    double ms_search;          /* (qa_model_set_timing)                       */
+    double ms_search;          /* (qa_model_set_timing); a kernel that prepares
+                                  and searches counts as the search           */
     double ms_recheck;
     double ms_soft;
 } qa_stats;

@@ -484,6 +484,14 @@ int choose_search(const qa_model* m, const qa::ArrayDesc& d, long long P) {
   return kexp < (P >= 30000 ? 9.4 : 4.6) ? qa::kSearchMixed : qa::kSearchTiles;
 }
 
+// Lanes and slots of the search that runs, for the statistics: the sphere
+// search has no inner or middle slots, the enumeration no middle ones.
+qa::SearchCfg search_shape(const qa::ArrayDesc& d) {
+  if (d.search == qa::kSearchTiles) return d.cfg;
+  const int lanes = d.prep_team;
+  return {d.search == qa::kSearchSphere ? 0 : qa::dense_inner(lanes), 0, lanes};
+}
+
 // The same for a single-array call; its close list takes the block counts' room
 // beyond the grid's entries (at most ceil(P / 8) of P + 1).
 void set_search(const qa_model* m, qa::GsLaunch* a) {
@@ -646,7 +654,7 @@ int run_ground_state(qa_model* m, const ScanIn& in, double t, int closed,
   a.one.out_n16 = out_n16;
   a.one.out_U = out_U;
   a.one.out_flags = out_flags;
-  m->last_cfg = a.one.cfg;
+  m->last_cfg = search_shape(a.one);
   m->last_P = P;
   a.ev = m->timing ? m->ev : nullptr;
   m->last_kind = 1;

@@ -1072,7 +1072,7 @@ __device__ __forceinline__ unsigned dense_search(const float* sM, int n, int lt,
                                                  float* sv, unsigned* lst, int& close,
                                                  unsigned& evaluated) {
   constexpr int LB = W == 16 ? 4 : W == 8 ? 3 : 2;
-  constexpr int kIn = W == 4 ? 2 : 4, NI = 1 << kIn;
+  constexpr int kIn = dense_inner(W), NI = 1 << kIn;
   const unsigned hw = threadIdx.x & 31u & ~(unsigned)(W - 1);
   constexpr unsigned kW = W == 32 ? 0xffffffffu : (1u << W) - 1u;
   auto team = [&](bool pred) { return (__ballot_sync(kFull, pred) >> hw) & kW; };

@@ -301,8 +301,8 @@ static cudaError_t run(const GsLaunch& L, cudaStream_t st) {
   constexpr bool kBnb = bnb_search(L1, L2);
   const bool tf = L.one.cfg.T >= kTeamFinishMin;
   if (L.one.search != kSearchTiles) {
-    e = launch_pixels(L, st);
     if (L.ev) cudaEventRecord(L.ev[1], st);
+    e = launch_pixels(L, st);
   } else if (fused_tiles(L)) {
     if (L.ev) cudaEventRecord(L.ev[1], st);
     if (kBnb && tf)

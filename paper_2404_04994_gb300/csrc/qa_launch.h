@@ -21,6 +21,9 @@ struct SearchCfg {
 // pixel's ambiguous dots.
 enum : int { kSearchTiles = 0, kSearchSphere = 1, kSearchDense = 2, kSearchMixed = 3 };
 
+// The enumeration's inner slots, by lanes per pixel.
+__host__ __device__ constexpr int dense_inner(int lanes) { return lanes == 4 ? 2 : 4; }
+
 // One array of a ground-state call: its model, voltages, method settings,
 // scratch records and outputs.
 struct ArrayDesc {

@@ -82,7 +82,7 @@ API int cudaStreamSynchronize(void*) { return 0; }
 API int cudaEventCreate(void** e) { *e = &dev; return 0; }
 API int cudaEventCreateWithFlags(void** e, unsigned) { *e = &dev; return 0; }
 API int cudaEventDestroy(void*) { return 0; }
-API int cudaEventRecord(void*, void*) { return 0; }
+API int cudaEventRecord(void*, void*) { log_ += "event "; return 0; }
 API int cudaEventSynchronize(void*) { return 0; }
 API int cudaEventElapsedTime(float* t, void*, void*) { *t = 0.f; return 0; }
 API void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
@@ -173,3 +173,35 @@ for n in (3, 5, 8, 11, 12, 16):
 """)
     pairs = set(zip(out[::2], out[1::2]))
     assert pairs == {("0", "1")} if team else ("1", "0") in pairs
+
+
+@pytest.mark.parametrize("n,t,closed,kernel,shape", [
+    (2, 1.0, 0, "k_ground_state", (1, 2, 0)), (3, 1.0, 1, "k_pixels", (4, 2, 0)),
+    (4, 0.5, 0, "k_pixels", (4, 2, 0)), (8, 1.0, 0, "k_pixels", (8, 4, 0)),
+    (9, 0.5, 1, "k_pixels", (16, 4, 0)), (16, 0.5, 0, "k_pixels", (16, 4, 0)),
+    (16, 1.0, 1, "k_pixels", (16, 0, 0)), (16, 1.0, 0, "k_pixels", (16, 0, 0))])
+def test_stats_describe_the_search_that_ran(library, n, t, closed, kernel, shape):
+    # lanes and slots of the kernel of the call, and its time as the search's:
+    # the kernel lies between the second and the third of four events
+    out = _run(library, f"""
+import ctypes
+import numpy as np
+from paper_2404_04994_gb300 import api, inputs
+lib, n = api.load(), {n}
+lib.launched.restype = ctypes.c_char_p
+r = np.random.Generator(np.random.PCG64(2))
+m = api.qa_model_create(inputs.chain_cdd(r, n), inputs.dense_cgd(r, n))
+api.qa_model_set_timing(m, True)
+ras = api.make_raster(inputs.raster(n, 0, 1, np.ones(n), W=300, H=200), n)
+out = np.zeros((60000, n), dtype=np.int8)
+if {closed}:
+    rc = lib.qa_ground_state_closed(m, ctypes.byref(ras), {t}, n, out.ctypes.data, None, None, None)
+else:
+    rc = lib.qa_ground_state_open(m, ctypes.byref(ras), {t}, out.ctypes.data, None, None, None)
+s = api.qa_model_stats(m, 0)
+print(rc, s["team"], s["inner_bits"], s["middle_bits"], lib.launched().decode())
+""")
+    assert tuple(int(v) for v in out[:4]) == (0, *shape)
+    chain = out[4:]
+    assert [i for i, v in enumerate(chain) if v == "event"] == [0, 1, 3, 5]
+    assert kernel in chain[2] and "k_lists" in chain[4]
