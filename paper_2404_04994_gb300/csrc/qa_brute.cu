@@ -51,7 +51,8 @@ struct BruteShared {
   unsigned long long code[kBrutePix];  // the answer
   unsigned char tie[kBrutePix];        // 1: near tie, 2: no state
   int nv[kBruteVec];                   // its charges
-  unsigned long long list[kBruteThreads * kBruteList];  // per team: shortlisted lines
+  unsigned long long list[kBruteThreads * kBruteList];  // per team: shortlisted lines (from
+                                                        // bit 8), the minimum's digit below
   unsigned cnt[kBruteThreads];
 };
 
@@ -411,8 +412,7 @@ __global__ void __launch_bounds__(kBruteThreads, 6) k_brute(BruteLaunch L) {
             if (E <= lim) {
               const unsigned at = atomicAdd(&sh.cnt[team], 1u);
               const unsigned long long line = (unsigned long long)(hs * (ID)Rm) + (unsigned)v;
-              if (at < (unsigned)(T * kBruteList))
-                list[at] = line * (unsigned long long)(topl + 1) + (unsigned long long)(int)qq;
+              if (at < (unsigned)(T * kBruteList)) list[at] = (line << 8) | (unsigned)(int)qq;
             }
           }
         }
@@ -424,22 +424,23 @@ __global__ void __launch_bounds__(kBruteThreads, 6) k_brute(BruteLaunch L) {
       unsigned long long c1 = ~0ull;
       if (ok) {
         for (unsigned e = lt; e < 3 * cnt; e += T) {
-          const unsigned long long cc = list[e / 3];
-          const int st = (int)(e % 3) - 1;
-          const int qd = (int)(cc % (unsigned long long)(topl + 1)) + st;
+          const unsigned long long cc = list[e / 3] >> 8;
+          const int qd = (int)(list[e / 3] & 255u) + (int)(e % 3) - 1;
           // the line's range: its other digits leave the last one nhat - sum
           int top = topl;
           if (closed) {
-            unsigned long long w = cc / (unsigned long long)(topl + 1);
+            ID w = (ID)cc;
             int s = 0;
             for (int j = 0; j < nfree - 1; ++j) {
-              s += (int)(w % (unsigned long long)R);
-              w /= (unsigned long long)R;
+              const ID q1 = w / (ID)R;
+              s += (int)(w - q1 * (ID)R);
+              w = q1;
             }
             top = min(top, nhat - s);
           }
           if (qd < 0 || qd > top) continue;
-          const unsigned long long cs = cc + (unsigned long long)(long long)st;
+          const unsigned long long cs =
+              cc * (unsigned long long)(topl + 1) + (unsigned long long)qd;
           brute_keep(brute_energy_f64(L, sh.M, sh.d + q * n, cs), cs, e1, c1, e2);
         }
       } else {
@@ -521,6 +522,13 @@ cudaError_t launch_brute(const BruteLaunch& L0, cudaStream_t st) {
   L.pix = kBruteThreads / L.team * 8;
   while (L.pix > kBrutePix || L.pix * L.a.n > kBruteVec) L.pix /= 2;
   while (L.pix > 4 && (L.a.sc.P + L.pix - 1) / L.pix < 4LL * L.num_sms) L.pix /= 2;
+  // a block's threads beyond its pixels' teams help the shortlist: one lane of
+  // a 1- or 2-dot array otherwise forms its up to 3 x 8 states in FP64 one
+  // after another, and the one block in a hundred with such a pixel sets the
+  // call's time (2 dots closed, 40 x 30 pixels, 12 or 30 charges: 16.1 ->
+  // 14.2 us, the shortlist's entries by shifts instead of 64-bit divisions
+  // included)
+  while (L.team < 32 && 2 * L.team * L.pix <= kBruteThreads) L.team *= 2;
   const long long blocks = (L.a.sc.P + L.pix - 1) / L.pix;
   if (L.nhi * (unsigned long long)L.radix < 0x7fffffffull)
     k_brute<unsigned><<<(unsigned)blocks, kBruteThreads, 0, st>>>(L);

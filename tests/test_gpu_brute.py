@@ -151,3 +151,15 @@ def test_line_search_exact_ties(qa, n, closed):
     want = [1] * (n - n // 2) + [2] * (n // 2) if closed else [1] * n
     np.testing.assert_array_equal(nn[0], want)
     assert f[0] & 1 and abs(U[0] - 0.125 * n) < 1e-14
+
+
+@pytest.mark.parametrize("n,closed,bound,W,H", [
+    (1, False, 30, 40, 30), (2, True, 30, 40, 30), (2, False, 7, 40, 30), (3, False, 1, 4, 1),
+    (2, False, 12, 153, 4), (3, True, 9, 19, 32)])
+def test_teams_wider_than_the_hi_states(qa, n, closed, bound, W, H):
+    # small rasters: lanes without a leading-digit state of their own
+    r = np.random.Generator(np.random.PCG64(600 + n))
+    Cdd, Cgd = inputs.random_model(r, n)
+    gx, gy = (0, 0) if n == 1 else inputs.swept_gates(n)
+    ras = inputs.raster(n, gx, gy, inputs.offsets(r, n, (gx, gy)), W=W, H=H, hi=5.0)
+    _check(qa, Cdd, Cgd, ras, closed, bound, f"N={n} closed={closed} bound={bound}")
