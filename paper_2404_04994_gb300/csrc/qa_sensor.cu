@@ -21,7 +21,7 @@
 // since every run draws its row's telegraph gaps from the start (32 a step).
 // 200 x 200 pixels, 4 dots and a sensor with all noises: 118 us with a
 // block per row, every normal drawn per pixel and c formed gate by gate;
-// about 45 us so (the whole diagram, ground state included, 162 -> 90 us).
+// about 43 us so.
 #include <algorithm>
 
 #include "qa_launch.h"
@@ -87,10 +87,15 @@ struct SensorShared {
   int status;
 };
 
+// S: sensors.  Known when compiled, because an FP64 operation whose predicate
+// is off takes the pipe all the same: with loops over the four possible places
+// 2 dots and a sensor on 601 x 700 pixels took 87 us without noise (76 with a
+// block per row and c formed gate by gate), 49 so.
+template <int S>
 __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
   __shared__ SensorShared sh;
   const ArrayDesc& a = L.a;
-  const int nf = a.n, S = L.S, nd = nf - S;
+  const int nf = a.n, nd = nf - S;
   const int W = a.sc.W;
   const unsigned row = blockIdx.x;
   const int first = (int)blockIdx.y * L.run;
@@ -175,11 +180,13 @@ __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
     return;
   }
   const bool white = L.white_sigma > 0.0, pink = L.pink_sigma > 0.0;
+  // (without noise the chunks share nothing, and need no barriers)
+  const bool noise = white || pink, jump = L.jump_prob > 0.0;
   const int room = kSensorChunk + octaves_room(L.K);
   for (int b0 = first; b0 < last; b0 += kSensorChunk) {
     const int b1 = min(b0 + kSensorChunk, last);
     // the chunk's normals: white, then the octaves' values
-    if (white || pink)
+    if (noise)
       for (int e = threadIdx.x; e < S * room; e += blockDim.x) {
         const int s = e / room;
         int r = e - s * room;
@@ -196,52 +203,46 @@ __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
                                           (unsigned)((b0 >> k) + r));
         }
       }
-    __syncthreads();
+    if (noise) __syncthreads();
     const int col = b0 + threadIdx.x;
     if (col < b1) {
       const long long p = (long long)row * W + col;
       const double x = a.sc.x0 + col * a.sc.dx;
       // g_s = (M_SD (n_D - c_D))_s, the dots one after another
-      double g[kSensorMax] = {0.0, 0.0, 0.0, 0.0};
+      double g[S] = {};
       for (int j = 0; j < nd; ++j) {
         const double r = (double)L.n_dots[p * nd + j] - a.mt.carrier * (sh.c0[j] + x * sh.cu[j]);
 #pragma unroll
-        for (int s = 0; s < kSensorMax; ++s)
-          if (s < S) g[s] += sh.M[(nd + s) * nf + j] * r;
+        for (int s = 0; s < S; ++s) g[s] += sh.M[(nd + s) * nf + j] * r;
       }
-      double cs[kSensorMax], bvec[kSensorMax], xs[kSensorMax];
+      double cs[S], bvec[S], xs[S];
 #pragma unroll
-      for (int s = 0; s < kSensorMax; ++s)
-        cs[s] = s < S ? a.mt.carrier * (sh.c0[nd + s] + x * sh.cu[nd + s]) : 0.0;
+      for (int s = 0; s < S; ++s) cs[s] = a.mt.carrier * (sh.c0[nd + s] + x * sh.cu[nd + s]);
       // b_s = g_s - (M_SS c_S)_s : E(n_S) = 1/2 n_S M_SS n_S + n_S . b
 #pragma unroll
-      for (int s = 0; s < kSensorMax; ++s) {
-        if (s >= S) break;
+      for (int s = 0; s < S; ++s) {
         double mc = 0.0, acc = 0.0;
 #pragma unroll
-        for (int t = 0; t < kSensorMax; ++t) {
-          if (t >= S) break;
+        for (int t = 0; t < S; ++t) {
           mc += sh.M[(nd + s) * nf + nd + t] * cs[t];
           acc += sh.Mssi[s * S + t] * g[t];
         }
         bvec[s] = g[s] - mc;
         xs[s] = cs[s] - acc;
       }
-      int best[kSensorMax] = {0, 0, 0, 0};
+      int best[S] = {};
       double bestE = 0.0;
       for (int m = 0; m < (1 << S); ++m) {
-        int cand[kSensorMax] = {0, 0, 0, 0};
+        int cand[S];
 #pragma unroll
-        for (int s = 0; s < kSensorMax; ++s)
-          if (s < S) cand[s] = (int)floor(xs[s] > 0.0 ? xs[s] : 0.0) + ((m >> s) & 1);
+        for (int s = 0; s < S; ++s)
+          cand[s] = (int)floor(xs[s] > 0.0 ? xs[s] : 0.0) + ((m >> s) & 1);
         double E = 0.0;
 #pragma unroll
-        for (int s = 0; s < kSensorMax; ++s) {
-          if (s >= S) break;
+        for (int s = 0; s < S; ++s) {
           double q = 0.0;
 #pragma unroll
-          for (int t = 0; t < kSensorMax; ++t)
-            if (t < S) q += sh.M[(nd + s) * nf + nd + t] * (double)cand[t];
+          for (int t = 0; t < S; ++t) q += sh.M[(nd + s) * nf + nd + t] * (double)cand[t];
           E += (double)cand[s] * (0.5 * q + bvec[s]);
         }
         bool better = (m == 0) || E < bestE;
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
           better = false;
           bool equal = true;
 #pragma unroll
-          for (int s = 0; s < kSensorMax; ++s) {
+          for (int s = 0; s < S; ++s) {
             if (equal && cand[s] != best[s]) {
               better = cand[s] < best[s];
               equal = false;
@@ -260,17 +261,15 @@ __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
         if (better) {
           bestE = E;
 #pragma unroll
-          for (int s = 0; s < kSensorMax; ++s) best[s] = cand[s];
+          for (int s = 0; s < S; ++s) best[s] = cand[s];
         }
       }
 #pragma unroll
-      for (int s = 0; s < kSensorMax; ++s) {
-        if (s >= S) break;
+      for (int s = 0; s < S; ++s) {
         const int q = nd + s;
         double V = g[s];  // the dots' part of (M (n - c))_s
 #pragma unroll
-        for (int t = 0; t < kSensorMax; ++t)
-          if (t < S) V += sh.M[q * nf + nd + t] * ((double)best[t] - cs[t]);
+        for (int t = 0; t < S; ++t) V += sh.M[q * nf + nd + t] * ((double)best[t] - cs[t]);
         const double y = (0.5 * sh.M[q * nf + q] - fabs(V)) / L.width;
         double v = L.shape == 1 ? exp(-0.5 * y * y) : 1.0 / (1.0 + y * y);
         if (white) v += L.white_sigma * sh.white[s][threadIdx.x];
@@ -283,7 +282,7 @@ __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
           }
           v += L.pink_sigma * acc / sqrt((double)L.K);
         }
-        if (L.jump_prob > 0.0) {
+        if (jump) {
           // telegraph state = parity of the switch points at or before col
           unsigned par = (unsigned)sh.par0[s];
           const int rel = col - first, wlast = rel >> 5;
@@ -297,16 +296,16 @@ __global__ void __launch_bounds__(kSensorThreads) k_sensor(SensorLaunch L) {
         if (L.out_potential) L.out_potential[p * S + s] = V;
       }
     }
-    __syncthreads();
+    if (noise || jump) __syncthreads();
     // the next chunk starts from this one's parity
-    if (threadIdx.x < S && L.jump_prob > 0.0) {
+    if (threadIdx.x < S && jump) {
       int par = sh.par0[threadIdx.x];
       const int w0 = (b0 - first) >> 5;
       for (int w = w0; w < w0 + kSensorChunk / 32 && w < words; ++w)
         par ^= __popc(sh.flips[threadIdx.x][w]) & 1;
       sh.par0[threadIdx.x] = par;
     }
-    __syncthreads();
+    if (jump) __syncthreads();
   }
 }
 
@@ -319,7 +318,11 @@ cudaError_t launch_sensor(const SensorLaunch& L0, cudaStream_t st) {
   const int runs = (int)std::min<long long>((W + kSensorChunk - 1) / kSensorChunk, want);
   L.run = ((W + runs - 1) / runs + kSensorChunk - 1) / kSensorChunk * kSensorChunk;
   const unsigned cols = (unsigned)((W + L.run - 1) / L.run);
-  k_sensor<<<dim3((unsigned)H, cols), kSensorThreads, 0, st>>>(L);
+  const dim3 grid((unsigned)H, cols);
+  if (L.S == 1) k_sensor<1><<<grid, kSensorThreads, 0, st>>>(L);
+  else if (L.S == 2) k_sensor<2><<<grid, kSensorThreads, 0, st>>>(L);
+  else if (L.S == 3) k_sensor<3><<<grid, kSensorThreads, 0, st>>>(L);
+  else k_sensor<4><<<grid, kSensorThreads, 0, st>>>(L);
   return cudaGetLastError();
 }
 

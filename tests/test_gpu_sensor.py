@@ -125,3 +125,31 @@ def test_row_runs_match_oracle(qa, W, H, p):
     np.testing.assert_array_equal(ns[clear], ref["n_sensor"][clear])
     np.testing.assert_allclose(pot[clear], ref["potential"][clear], atol=1e-10)
     np.testing.assert_allclose(sig[clear], ref["signal"][clear], atol=2e-6, rtol=1e-6)
+
+
+# One kernel per number of sensors, each with and without the barriers that
+# noise and the telegraph's parity need.
+@pytest.mark.parametrize("S", [1, 2, 3, 4])
+@pytest.mark.parametrize("noise", [{}, dict(white_sigma=0.05), dict(jump_amplitude=0.2, jump_prob=0.2),
+                                   NOISY])
+def test_every_number_of_sensors(qa, S, noise):
+    r = np.random.Generator(np.random.PCG64(S))
+    n = 2 + S
+    Cdd = np.eye(n)
+    Cdd[2:, :2] = -r.uniform(0.02, 0.08, (S, 2))
+    Cdd[:2, 2:] = Cdd[2:, :2].T
+    Cdd[0, 1] = Cdd[1, 0] = -0.2
+    Cgd = np.diag(r.uniform(0.7, 1.0, n)) + r.uniform(0.0, 0.05, (n, n))
+    ras = {"V0": np.concatenate([[0.0, 0.0], r.uniform(2.0, 3.0, S)]), "u": np.eye(n)[0],
+           "w": np.eye(n)[1], "x0": -0.5, "x1": 4.0, "y0": -0.5, "y1": 4.0, "W": 150, "H": 21}
+    nd = oracle.ground_state(Cdd[:2, :2], Cgd[:2, :], raster=ras, t=1.0)["n"][:, :2]
+    kw = dict(dict(white_sigma=0.0, pink_sigma=0.0, jump_amplitude=0.0, jump_prob=0.0, seed=5),
+              **noise)
+    sig, ns, pot = _gpu_epilogue(qa, Cdd, Cgd, ras, nd, S, width=0.05, **kw)
+    ref = oracle.charge_sensor(Cdd, Cgd, ras, nd, n_sensor=S, width=0.05, **kw)
+    eps = 0.5 * np.diag(np.linalg.inv(Cdd))[2:] - np.abs(ref["potential"])
+    clear = (eps > 1e-9).all(1)
+    assert clear.mean() > 0.95
+    np.testing.assert_array_equal(ns[clear], ref["n_sensor"][clear])
+    np.testing.assert_allclose(pot[clear], ref["potential"][clear], atol=1e-10)
+    np.testing.assert_allclose(sig[clear], ref["signal"][clear], atol=2e-6, rtol=1e-6)
