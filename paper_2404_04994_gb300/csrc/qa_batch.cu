@@ -54,6 +54,7 @@ __device__ __forceinline__ void search_batch_units(const GsLaunch& L, int v) {
   int staged = -1;
   SearchAcc acc;
   const int first = L.var_first[v], count = L.var_count[v];
+  grid_dep_signal();
   for (;;) {
     __syncthreads();
     if (threadIdx.x == 0) s_unit = (int)atomicAdd(&L.cnt->q_var[v], 1u);
@@ -79,6 +80,7 @@ __device__ __forceinline__ void search_batch_units(const GsLaunch& L, int v) {
     o.boundary = acc.boundary;
     o.overflow = acc.overflow;
   }
+  grid_dep_wait();  // ends after the variants before it
 }
 
 template <int L1, int L2, bool CLOSED, bool TF>
@@ -130,15 +132,24 @@ void batch_occupancy(int* prep_per_sm, int* search_per_sm) {
 cudaError_t launch_ground_state_batch(const GsLaunch& L, cudaStream_t st) {
   if (L.ev) cudaEventRecord(L.ev[0], st);
   cudaMemsetAsync(L.cnt, 0, sizeof(Counters), st);
-  // each stage's own error: a launcher that reports one has cleared it
-  cudaError_t e = launch_pixels_batch(L, st);
-  if (e != cudaSuccess) return e;
+  // The first search grid waits for the records of the whole prep; the others
+  // and the one-pass grids each start while the one before runs, and end after
+  // it.  Each stage's own error: a launcher that reports one has cleared it.
+  cudaError_t e = cudaSuccess;
   if (L.n_prep_units > 0) k_prep_batch<<<L.grid_prep, kPrepThreads, 0, st>>>(L);
   if (L.ev) cudaEventRecord(L.ev[1], st);
-  for (int v = 0; v < kBatchVariants; ++v)
-    if (L.var_count[v] > 0) batch_search_kernel(v)<<<L.var_grid[v], kSearchThreads, 0, st>>>(L, v);
+  bool first = true;
+  for (int v = 0; v < kBatchVariants && e == cudaSuccess; ++v) {
+    if (L.var_count[v] == 0) continue;
+    if (first)
+      batch_search_kernel(v)<<<L.var_grid[v], kSearchThreads, 0, st>>>(L, v);
+    else
+      e = launch_dependent(batch_search_kernel(v), (unsigned)L.var_grid[v], kSearchThreads, st, L, v);
+    first = false;
+  }
+  if (e == cudaSuccess) e = launch_pixels_batch(L, st);
   if (L.ev) cudaEventRecord(L.ev[2], st);
-  e = launch_lists(L, st);
+  if (e == cudaSuccess) e = launch_lists(L, st);
   if (L.ev) cudaEventRecord(L.ev[3], st);
   const cudaError_t last = cudaGetLastError();
   return e != cudaSuccess ? e : last;

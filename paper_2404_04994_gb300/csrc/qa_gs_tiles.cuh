@@ -102,6 +102,24 @@ __device__ __forceinline__ U block_sum(U v, U* red) {
   return t;
 }
 
+// Launch with programmatic stream serialisation (the kernel waits for its
+// predecessor's results with grid_dep_wait).
+template <typename... KArgs>
+inline cudaError_t launch_dependent(void (*kern)(KArgs...), unsigned grid, unsigned block,
+                                    cudaStream_t st, KArgs... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = 0;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // ---------------------------------------------------------------------------
 // prep stage: shared state of a block and the per-array set-up
 // ---------------------------------------------------------------------------

@@ -256,24 +256,6 @@ int search_blocks(const GsLaunch& L) {
   return (int)((L.one.sc.P + teams - 1) / teams);
 }
 
-// Launch with programmatic stream serialisation (the kernel waits for its
-// predecessor's results with grid_dep_wait).
-template <typename... KArgs>
-static cudaError_t launch_dependent(void (*kern)(KArgs...), unsigned grid, unsigned block,
-                                    cudaStream_t st, KArgs... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 cudaError_t launch_lists(const GsLaunch& L, cudaStream_t st) {
   // (of a batch, only where an array is searched pixel by pixel)
   bool close = L.one.search != kSearchTiles;

@@ -62,7 +62,10 @@ API int __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* s, void* st) {
 API int __cudaGetKernel(void** k, const void* f) { *k = (void*)f; return 0; }
 API int __cudaLaunchKernel(void* k, dim3, dim3, void**, size_t s, void*) { return launch(k, s); }
 struct Config { dim3 g, b; size_t s; };
-API int cudaLaunchKernelExC(const Config* c, const void* f, void**) { return launch(f, c->s); }
+API int cudaLaunchKernelExC(const Config* c, const void* f, void**) {
+  log_ += "overlapped:";
+  return launch(f, c->s);
+}
 API int cudaGetLastError() { int e = last; last = 0; return e; }
 API const char* cudaGetErrorString(int) { return "error"; }
 API int cudaMalloc(void** p, size_t n) { *p = calloc(n, 1); return 0; }
@@ -205,3 +208,32 @@ print(rc, s["team"], s["inner_bits"], s["middle_bits"], lib.launched().decode())
     chain = out[4:]
     assert [i for i, v in enumerate(chain) if v == "event"] == [0, 1, 3, 5]
     assert kernel in chain[2] and "k_lists" in chain[4]
+
+
+def test_grids_of_a_batch_overlap(library):
+    # arrays of every kind: after the prep and the first search grid, which
+    # waits for it, each grid may start while the one before runs
+    out = _run(library, """
+import ctypes
+import numpy as np
+from paper_2404_04994_gb300 import api, inputs
+lib = api.load()
+lib.launched.restype = ctypes.c_char_p
+kinds = [(n, c, t) for n in (2, 3, 8, 9, 11, 12, 16) for c in (0, 1) for t in (0.5, 1.0)]
+items, keep = (api.qa_batch_item * len(kinds))(), []
+for it, (n, closed, t) in zip(items, kinds):
+    r = np.random.Generator(np.random.PCG64(2))
+    m = api.qa_model_create(inputs.chain_cdd(r, n), inputs.dense_cgd(r, n))
+    out = np.zeros((32, n), dtype=np.int8)
+    ras = api.make_raster(inputs.raster(n, 0, 1, np.ones(n), W=8, H=4), n)
+    keep += [m, out, ras]
+    it.model, it.out_n, it.raster = m.value, out.ctypes.data, ras
+    it.threshold, it.closed, it.n_charges = t, closed, n
+b = ctypes.c_void_p()
+assert lib.qa_batch_create(items, len(kinds), ctypes.byref(b)) == 0
+assert lib.qa_batch_run(b, None) == 0
+print(lib.launched().decode())
+""")
+    assert "k_prep_batch" in out[0] and "k_lists" in out[-1]
+    assert sum("k_pixels_batch" in v for v in out) >= 8
+    assert [v.startswith("overlapped:") for v in out] == [False, False] + [True] * (len(out) - 2)
