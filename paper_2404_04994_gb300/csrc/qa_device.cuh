@@ -113,8 +113,9 @@ struct __align__(16) ModelConsts {
   int pad2[2];
 };
 
-// Arrays of at least this many dots may take the sphere search (qa_sphere.cuh).
-constexpr int kSphereMinDot = 9;
+// Arrays of at least this many dots may take the sphere search (qa_sphere.cuh):
+// the dispatch's line for it lies above 11 expected ambiguous dots.
+constexpr int kSphereMinDot = 12;
 
 // Factor of M for the sphere search, formed on the host with the model: with
 // Cdd = L L^T in the order `ord` (at each step the dot of the smallest
@@ -126,8 +127,8 @@ struct __align__(16) SphereConsts {
   unsigned char ord[kMaxDot];           // dot of each level
   unsigned char pos[kMaxDot];           // level of each dot
   float ysq;                            // sum_k (sum_l |W_kl|)^2
-  float msum;                           // sum_ij |M_ij| (any number of dots)
-  int valid;                            // 0: updated on the device, or no factor
+  float msum;                           // sum_ij |M_ij| (any number of dots; +inf: none)
+  int valid;                            // the factor: 0 if updated on the device, or none
   int pad;
 };
 

@@ -1008,7 +1008,8 @@ struct PixelShared {
   PrepShared p;
   unsigned long long cand[kTeams], ev[kTeams];
   unsigned qp[kTeams], doubled[kTeams], boundary[kTeams], overflow[kTeams];
-  int valid;
+  int valid;  // sum |M|
+  int factor;
 };
 struct SphereShared : PixelShared<kSphT> {
   SphereModel m;
@@ -1038,7 +1039,10 @@ __device__ inline void pixel_stage_search(const ArrayDesc&, PixelShared<W>&) {}
 template <typename SH>
 __device__ inline void pixel_stage_array(const ArrayDesc& a, SH& sh) {
   pixel_stage_search(a, sh);
-  if (threadIdx.x == 0) sh.valid = a.md->s.valid;
+  if (threadIdx.x == 0) {
+    sh.valid = a.md->s.msum < kInf;
+    sh.factor = a.md->s.valid;
+  }
   prep_stage_array(a, sh.p);  // ends with a barrier
 }
 template <int W>
@@ -1326,7 +1330,7 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
     // no factor, or a centre outside [-1, 1] (an unsettled QP): left to the
     // FP32 search
     const bool far = ((__ballot_sync(kFull, !(fabsf(f) <= 1.f)) >> hw) & kW) != 0u;
-    bits = sphere_search<CLOSED>(a.md->s, sh.m, n, lt, active && sh.valid && !far, f, a1, q.mask,
+    bits = sphere_search<CLOSED>(a.md->s, sh.m, n, lt, active && sh.factor && !far, f, a1, q.mask,
                                  q.w, bound, neg, &sh.p.qx[tq], &sh.p.qz[tq], sh.lev[team],
                                  reinterpret_cast<uint2*>(&sh.p.qK[tq][0]), close, ev);
   }

@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
       md->gen = 0u;
       md->k.model_bad = 1;
       md->s.valid = 0;
+      md->s.msum = __int_as_float(0x7f800000);
     }
     return;
   }
@@ -102,9 +103,10 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
         sc += fabs(C[q * n + tid]);
         sm += fabs(Ms[q * n + tid]);
       }
-    double tot = r, n1c = sc, n1m = sm;
+    double tot = r, n1c = sc, n1m = sm, sum = sm;
     for (int off = 16; off > 0; off >>= 1) {
       tot += __shfl_xor_sync(0xffffffffu, tot, off);
+      sum += __shfl_xor_sync(0xffffffffu, sum, off);
       n1c = fmax(n1c, __shfl_xor_sync(0xffffffffu, n1c, off));
       n1m = fmax(n1m, __shfl_xor_sync(0xffffffffu, n1m, off));
     }
@@ -140,6 +142,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
       kc.pad2[0] = kc.pad2[1] = 0;
       kc.model_bad = 0;
       md->s.valid = 0;  // the sphere search's factor is the host's
+      md->s.msum = __double2float_rn(sum * (1.0 + 1e-6));
       kc.pad = 0;
     }
   }
