@@ -233,7 +233,7 @@ void fill_consts(int n, qa::ModelData* md) {
   fill_sphere(n, md);
 }
 
-// ModelData::gen of the host copy that makes a model's generation `gen`.
+// ModelConsts::gen of the host copy that makes a model's generation `gen`.
 unsigned host_gen(unsigned long long gen) { return (unsigned)(gen % 0xffffffffull) + 1u; }
 
 // Validate + convert host matrices into a ModelData (Maxwell form).
@@ -434,7 +434,8 @@ qa::SearchCfg choose_cfg(int n, double t, long long P, int num_sms, bool closed)
 
 // c0 = s Cgd (V0 + x0 u + y0 w), du = s Cgd u dx, dw = s Cgd w dy in FP64 on
 // the host, split into double-float; only when the host copy is current.
-qa::RasterK raster_constants(const qa_model* m, const qa::Scan& sc) {
+// current: for a launch on this stream now (not one that is captured or kept).
+qa::RasterK raster_constants(const qa_model* m, const qa::Scan& sc, bool current) {
   qa::RasterK rk;
   std::memset(&rk, 0, sizeof(rk));
   if (sc.kind != 0 || m->host_stale) return rk;
@@ -451,7 +452,8 @@ qa::RasterK raster_constants(const qa_model* m, const qa::Scan& sc) {
     rk.du[i] = split(b);
     rk.dw[i] = split(c);
   }
-  rk.gen = m->host.gen;
+  rk.gen = m->host.k.gen;
+  rk.current = current;
   return rk;
 }
 
@@ -474,6 +476,14 @@ int prep_team(int n) {
   int t = 1;
   while (t < n) t <<= 1;
   return t;
+}
+
+// Whether work enqueued on a stream now runs once, after what is enqueued already.
+bool runs_once(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s == cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
 }
 
 // The search of an array whose other fields are set (P: the pixels that decide
@@ -651,7 +661,7 @@ int run_ground_state(qa_model* m, const ScanIn& in, double t, int closed,
   a.one.cfg = choose_cfg(m->n, t, P, m->num_sms, closed);
   a.one.klass = qa::search_klass(a.one.cfg);
   a.one.prep_team = prep_team(m->n);
-  a.one.rk = raster_constants(m, sc);
+  a.one.rk = raster_constants(m, sc, runs_once(st));
   a.one.bx_analytic = 4.0e-7f;
   a.one.bx_qp_scale = 0.f;  // derived from the device model's condition number
   a.one.recs = (qa::PixRec*)(ws + off_recs);
@@ -744,7 +754,7 @@ int run_soft(qa_model* m, const qa_raster* r, double kT, double t, int closed,
   g.one.cfg = cfg;
   g.one.klass = qa::search_klass(cfg);
   g.one.prep_team = prep_team(m->n);
-  g.one.rk = raster_constants(m, sc);
+  g.one.rk = raster_constants(m, sc, runs_once(st));
   g.one.bx_analytic = 4.0e-7f;
   g.one.recs = (qa::PixRec*)(ws + off_recs);
   g.flag_list = (qa::ListEntry*)(ws + off_list);
@@ -832,7 +842,7 @@ int qa_model_create(const double* Cdd, const double* Cgd, int n_dot, int n_gate,
   qa_model* m = new qa_model();
   int rc = build_model(n_dot, n_gate, form, Cdd, Cgd, &m->host);
   if (rc) { delete m; return rc; }
-  m->host.gen = host_gen(m->gen);
+  m->host.k.gen = host_gen(m->gen);
   m->n = n_dot;
   m->ng = n_gate;
   m->form = form;
@@ -857,7 +867,7 @@ int qa_model_update(qa_model* m, const double* Cdd, const double* Cgd) {
   qa::ModelData md;
   int rc = build_model(m->n, m->ng, m->form, Cdd, Cgd, &md);
   if (rc) return rc;
-  md.gen = host_gen(m->gen + 1);
+  md.k.gen = host_gen(m->gen + 1);
   if ((rc = select_device(m))) return rc;
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess)
@@ -883,7 +893,7 @@ int qa_model_update_async(qa_model* m, const double* Cdd, const double* Cgd, voi
     if (e != cudaSuccess) return cuda_fail(e, "staging buffer");
   }
   if ((rc = build_model(m->n, m->ng, m->form, Cdd, Cgd, m->staging))) return rc;
-  m->staging->gen = host_gen(m->gen + 1);
+  m->staging->k.gen = host_gen(m->gen + 1);
   e = cudaMemcpyAsync(m->d_md, m->staging, sizeof(qa::ModelData), cudaMemcpyHostToDevice,
                       (cudaStream_t)stream);
   if (e == cudaSuccess) e = cudaEventRecord(m->staged, (cudaStream_t)stream);
@@ -1335,7 +1345,7 @@ extern "C" int qa_ground_state_open_static(qa_model* m, const qa_raster* r,
   a.one.cfg = choose_cfg(m->n, threshold, P, m->num_sms, false);
   a.one.klass = qa::search_klass(a.one.cfg);
   a.one.prep_team = prep_team(m->n);
-  a.one.rk = raster_constants(m, sc);
+  a.one.rk = raster_constants(m, sc, runs_once(st));
   a.one.bx_analytic = 4.0e-7f;
   a.one.bx_qp_scale = 0.f;
   a.one.recs = (qa::PixRec*)(ws + kStOffRecs);
@@ -1408,7 +1418,7 @@ int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out) {
     d.n = m->n;
     d.ng = m->ng;
     d.sc = sc;
-    d.rk = raster_constants(m, sc);
+    d.rk = raster_constants(m, sc, false);
     d.mt.t = it.threshold;
     d.mt.closed = it.closed ? 1 : 0;
     d.mt.n_charges = it.closed ? it.n_charges : 0;

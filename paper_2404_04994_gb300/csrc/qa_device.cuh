@@ -104,7 +104,7 @@ struct __align__(16) ModelConsts {
   float s_s;                   // 1^T Cdd 1
   float bx_qp_scale;           // QP decision margin per unit of (1+|c|+N_hat)
   int model_bad;               // device inverse of an updated Cdd failed (not PD)
-  int pad;
+  unsigned gen;                // which host copy this is; 0: updated on the device
   float CddLo[kMaxDot * kLdM]; // Cdd - hi part (Cdd as double-float with Cdd above)
   df sv2[kMaxDot];             // Cdd 1 as double-float
   float absl[kMaxDot];         // M_ii / 2 + sum_{j < i} |M_ij| (FP32 hi parts, j increasing)
@@ -140,7 +140,7 @@ struct __align__(16) ModelData {
   double vs[kMaxDot];                 // Cdd 1 / (1^T Cdd 1)   (Appendix D)
   double cond;                        // ||Cdd||_1 ||M||_1
   int status;                         // 0 ok; nonzero: Cdd not PD on update
-  unsigned gen;                       // which host copy this is; 0: updated on the device
+  int pad;
   ModelConsts k;                      // FP32 forms of the above
   SphereConsts s;
 };
@@ -160,8 +160,8 @@ struct Scan {
 // the model changed (a batch's next run, the replay of a graph) finds another
 // `gen` in the model and forms them from the device copy instead.
 struct RasterK {
-  unsigned gen;  // ModelData::gen of the host copy they come from; 0: none
-  int pad;
+  unsigned gen;  // ModelConsts::gen of the host copy they come from; 0: none
+  int current;   // the model cannot change before the launch runs: no check of gen
   df c0[kMaxDot], du[kMaxDot], dw[kMaxDot];
 };
 

@@ -145,7 +145,6 @@ struct PrepShared {
 // Stage an array's FP32 model constants and raster constants (all threads);
 // one thread converts the FP64 threshold for the whole block.
 __device__ inline void prep_stage_array(const ArrayDesc& a, PrepShared& sh) {
-  const bool rk = a.rk.gen != 0u && a.rk.gen == a.md->gen;
   stage_consts(&a.md->k, &sh.cs);
   if (threadIdx.x == 0) {
     sh.th0 = __double2float_rn(0.5 * a.mt.t);
@@ -157,22 +156,22 @@ __device__ inline void prep_stage_array(const ArrayDesc& a, PrepShared& sh) {
       sh.sG[i][g] = df_from_double(a.mt.carrier * a.md->Cgd[i * a.ng + g]);
     }
   }
-  if (a.sc.kind == 0) {
-    if (rk) {
-      if (threadIdx.x < kMaxDot) {
-        sh.sc0[threadIdx.x] = a.rk.c0[threadIdx.x];
-        sh.sdu[threadIdx.x] = a.rk.du[threadIdx.x];
-        sh.sdw[threadIdx.x] = a.rk.dw[threadIdx.x];
-      }
-    } else {
-      // (its voltage vectors in the QP rows, which no pixel uses yet)
-      static_assert(sizeof(sh.qK) >= 3 * kMaxGate * sizeof(df), "room for V0, u, w");
-      df* v = reinterpret_cast<df*>(&sh.qK[0][0]);
-      raster_consts(a.md, a.n, a.ng, a.sc, a.mt.carrier, v, v + kMaxGate, v + 2 * kMaxGate,
-                    sh.sc0, sh.sdu, sh.sdw);
-    }
+  if (a.sc.kind == 0 && threadIdx.x < kMaxDot) {
+    sh.sc0[threadIdx.x] = a.rk.c0[threadIdx.x];
+    sh.sdu[threadIdx.x] = a.rk.du[threadIdx.x];
+    sh.sdw[threadIdx.x] = a.rk.dw[threadIdx.x];
   }
   __syncthreads();
+  // of another host copy than the model's?  (Looked up among the constants; a
+  // load of its own cost a call 0.6 - 1.5 us.)
+  if (a.sc.kind == 0 && !a.rk.current && (a.rk.gen == 0u || a.rk.gen != sh.cs.gen)) {
+    // (its voltage vectors in the QP rows, which no pixel uses yet)
+    static_assert(sizeof(sh.qK) >= 3 * kMaxGate * sizeof(df), "room for V0, u, w");
+    df* v = reinterpret_cast<df*>(&sh.qK[0][0]);
+    raster_consts(a.md, a.n, a.ng, a.sc, a.mt.carrier, v, v + kMaxGate, v + 2 * kMaxGate, sh.sc0,
+                  sh.sdu, sh.sdw);
+    __syncthreads();
+  }
 }
 
 // c of a point-list pixel by its team (out of line: the raster kernels carry
@@ -1008,12 +1007,11 @@ struct PixelShared {
   PrepShared p;
   unsigned long long cand[kTeams], ev[kTeams];
   unsigned qp[kTeams], doubled[kTeams], boundary[kTeams], overflow[kTeams];
-  int valid;  // sum |M|
-  int factor;
 };
 struct SphereShared : PixelShared<kSphT> {
   SphereModel m;
   float4 lev[kTeams][kMaxDot / 2];
+  int factor;  // the model has one
 };
 // The search of a kernel's pixels: the enumeration, the sphere search, or the
 // one that a pixel's ambiguous dots call for (a warp's pixels alike: the
@@ -1033,16 +1031,13 @@ static_assert(kSphT * sizeof(float) * kQPRow >= kSphStack * sizeof(uint2),
 // Block set-up (all threads), once per array.
 __device__ inline void pixel_stage_search(const ArrayDesc& a, SphereShared& sh) {
   sphere_stage(a.md->s, sh.m);
+  if (threadIdx.x == 0) sh.factor = a.md->s.valid;
 }
 template <int W>
 __device__ inline void pixel_stage_search(const ArrayDesc&, PixelShared<W>&) {}
 template <typename SH>
 __device__ inline void pixel_stage_array(const ArrayDesc& a, SH& sh) {
   pixel_stage_search(a, sh);
-  if (threadIdx.x == 0) {
-    sh.valid = a.md->s.msum < kInf;
-    sh.factor = a.md->s.valid;
-  }
   prep_stage_array(a, sh.p);  // ends with a barrier
 }
 template <int W>
@@ -1290,18 +1285,17 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
 #pragma unroll
   for (int off = W / 2; off > 0; off >>= 1) S += __shfl_xor_sync(kFull, S, off);
   const unsigned any_qp = __any_sync(kFull, qp);
-  // max_j |base_j - c_j|, |x_j - c_j|, which scales the rounding of M r: at most
-  // 1 on an open pixel without active constraints (x = c), but a closed one
-  // moves every dot by lambda v
+  // max_j |base_j - c_j|, which scales the rounding of M r: at most 1 on an open
+  // pixel without active constraints (x = c), but a closed one moves every dot
+  // by lambda v
   float rmax = 1.f;
   if (CLOSED || any_qp) {
-    rmax = fmaxf(fabsf(r0), fabsf(sh.p.qz[threadIdx.x]));
+    rmax = fmaxf(fabsf(r0), 1.f);
 #pragma unroll
     for (int off = W / 2; off > 0; off >>= 1)
       rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
-    rmax = fmaxf(rmax, 1.f);
   }
-  const float ez = u24 * a.md->s.msum * rmax;  // u sum |M| |r|
+  const float msum = a.md->s.msum;
   int close = 0;
   unsigned ev = 0, bits = 0u;
   const bool sphere =
@@ -1312,6 +1306,7 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
     float a1 = 0.f, neg = 0.f;
     if (any_qp) {
       float z = 0.f;
+      rmax = fmaxf(rmax, fabsf(sh.p.qz[threadIdx.x]));
 #pragma unroll
       for (int j = 0; j < W; ++j) z = fmaf(Mrow[j], sh.p.qz[tq + j], z);
       if (CLOSED) {  // the multiple of 1: the least entry, a free dot's
@@ -1323,8 +1318,12 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
       a1 = (qp && amb) ? fmaxf(z, 0.f) : 0.f;
       neg = (qp && amb) ? fmaxf(-z, 0.f) : 0.f;
 #pragma unroll
-      for (int off = W / 2; off > 0; off >>= 1) neg += __shfl_xor_sync(kFull, neg, off);
+      for (int off = W / 2; off > 0; off >>= 1) {
+        neg += __shfl_xor_sync(kFull, neg, off);
+        rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
+      }
     }
+    const float ez = u24 * msum * rmax;  // u sum |M| |r|
     const float bound = pixel_bound(a, S * 1.00001f + 20.f * ez, k);
     neg += (qp ? 24.f : 2.f) * ez;
     // no factor, or a centre outside [-1, 1] (an unsettled QP): left to the
@@ -1339,11 +1338,12 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
   unsigned* lst =
       reinterpret_cast<unsigned*>(MODE == kPixDense ? &sh.p.qK[tq][0] : &sh.p.qz[tq]);
   if constexpr (MODE != kPixSphere) if (!sphere) {
+    const float ez = u24 * msum * rmax;
     // twice the near-tie bound as in the sphere search, once more for this
     // search's own sums (at most 2 k + 8 additions), and the error of the
     // plain h on both sides
     const float G = 3.f * pixel_bound(a, S * 1.00001f + 20.f * ez, k) + 40.f * ez;
-    bits = dense_search<W, CLOSED>(sh.p.cs.Mhi, n, lt, active && sh.valid, v, q.mask, q.w, G,
+    bits = dense_search<W, CLOSED>(sh.p.cs.Mhi, n, lt, active && msum < kInf, v, q.mask, q.w, G,
                                    &sh.p.qa[tq], &sh.p.qc[tq], lst, close, ev);
   }
   const bool done = active && close == 1;

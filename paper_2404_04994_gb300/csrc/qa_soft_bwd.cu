@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
   if (!ok) {
     if (tid == 0) {
       md->status = 1;
-      md->gen = 0u;
+      md->k.gen = 0u;
       md->k.model_bad = 1;
       md->s.valid = 0;
       md->s.msum = __int_as_float(0x7f800000);
@@ -133,7 +133,6 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
     if (tid == 0) {
       md->cond = cond;
       md->status = 0;
-      md->gen = 0u;
       kc.s_s = __double2float_rn(tot);
       const double e1 = cond * (n + 1) * 5.9604644775390625e-8;
       kc.bx_qp_scale = __double2float_rn(8.0 * e1);
@@ -143,7 +142,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_model_update(ModelData* md, int
       kc.model_bad = 0;
       md->s.valid = 0;  // the sphere search's factor is the host's
       md->s.msum = __double2float_rn(sum * (1.0 + 1e-6));
-      kc.pad = 0;
+      kc.gen = 0u;
     }
   }
 }

@@ -228,3 +228,27 @@ def test_batch_reports_the_error_of_each_stage(tmp_path, launcher):
     r = subprocess.run([sys.executable, "-c", code], env=env, cwd=root, capture_output=True,
                        text=True, timeout=300)
     assert r.stdout.strip() == "code -7", r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("n", [2, 5, 12])
+def test_captured_call_sees_a_model_update(qa, n):
+    # a single-array call replayed from a graph after its model changed
+    import torch
+    r = np.random.Generator(np.random.PCG64(n))
+    Cdd, Cgd = inputs.chain_cdd(r, n), inputs.dense_cgd(r, n)
+    ras = inputs.raster(n, *inputs.swept_gates(n), np.ones(n), W=60, H=50)
+    m = qa.Model(Cdd, Cgd)
+    out = torch.zeros((3000, n), dtype=torch.int8, device="cuda")
+    qa.qa_ground_state_open(m.handle, ras, 1.0, out)  # (the workspace, before the capture)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        qa.qa_ground_state_open(m.handle, ras, 1.0, out)
+    Cgd = Cgd * r.uniform(0.6, 1.4, Cgd.shape)
+    qa.qa_model_update(m.handle, Cdd, Cgd)
+    g.replay()
+    torch.cuda.synchronize()
+    m2 = qa.Model(Cdd, Cgd)
+    want, _, _ = m2.ground_state_open(ras)
+    assert bool((out == want.view(-1, n)).all())
+    m.close()
+    m2.close()

@@ -82,6 +82,7 @@ API int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const voi
 API int cudaGetSymbolAddress(void** p, const void* s) { *p = (void*)s; return 0; }
 API int cudaDeviceSynchronize() { return 0; }
 API int cudaStreamSynchronize(void*) { return 0; }
+API int cudaStreamIsCapturing(void*, int* status) { *status = 0; return 0; }
 API int cudaEventCreate(void** e) { *e = &dev; return 0; }
 API int cudaEventCreateWithFlags(void** e, unsigned) { *e = &dev; return 0; }
 API int cudaEventDestroy(void*) { return 0; }
