@@ -457,21 +457,6 @@ qa::RasterK raster_constants(const qa_model* m, const qa::Scan& sc, bool current
   return rk;
 }
 
-// Whether an array takes the sphere search (cfg: the FP32 search it would
-// take).  Its cost per pixel hardly depends on the candidates' number, 2^kexp
-// expected, the exhaustive walk's doubles with every dot: the line lies where
-// they cross, kexp just above 11 (300 x 200 rasters, exhaustive / sphere, us:
-// 11 dots t = 1 81 / 98, 13 dots t = 0.8 136 / 112, 12 dots t = 1 126 / 107;
-// closed 11 dots 154 / 167, 13 dots t = 0.8 291 / 189, 12 dots 252 / 174).  An
-// open raster too small to fill the GPU walks its candidates in wider teams
-// while the sphere search's few close pixels take a longer list kernel, so
-// there the line is 13 dots (100 x 100: 12 dots 33 / 45, 13 dots 41 / 41, 14
-// dots 53 / 49, 16 dots 58 / 43; closed 12 dots 60 / 53).
-bool use_sphere(int n, double kexp, long long P, bool closed, const qa::SearchCfg& cfg) {
-  return n >= qa::kSphereMinDot && cfg.T >= qa::kTeamFinishMin && cfg.L1 == 5 &&
-         kexp >= (closed || P >= 30000 ? 11.01 : 12.6);
-}
-
 int prep_team(int n) {
   int t = 1;
   while (t < n) t <<= 1;
@@ -487,23 +472,54 @@ bool runs_once(cudaStream_t st) {
 }
 
 // The search of an array whose other fields are set (P: the pixels that decide
-// how full the GPU is).
+// how full the GPU is).  Times below are whole calls on 8 to 240,000 pixels,
+// one-pass search / tiles; kexp: the expected number of ambiguous dots.
+//   3 to 8 dots: the enumeration, 0.31 - 0.99 at any size and threshold.
+//   9 to 11: its cost doubles with every dot while the tiles spread a pixel
+// over more lanes; they cross just above kexp = 9.5 where the pixels fill the
+// GPU (10,000 pixels and more: open 9.3 0.90 - 1.02, 10 0.93 - 1.06, 11 1.07 -
+// 1.20; closed 9.3 0.83 - 0.97, 10 0.82 - 1.07, 11 0.97 - 1.14).  Smaller
+// rasters leave lanes idle either way, and one kernel beats two: 0.41 - 0.98
+// below 3,000 pixels, so there it is taken up to 11.
+//   12 and more: the sphere search from kexp = 11 on (its cost hardly depends on
+// the candidates' number; 10,000 pixels and more 0.30 - 1.04, at 11.0 0.71 -
+// 1.0, at 16 0.33 - 0.70), below it either search by the pixel's dots: closed
+// 0.73 - 1.09; open to 9.4 from 30,000 pixels on (0.32 - 0.94; 9.5 to 10.9 0.89
+// - 1.07), to 4.6 on smaller ones (0.62 - 1.08; 5 to 10.9 at 10,000 pixels 0.81
+// - 1.05, at 600 0.69 - 1.20).  A closed array at t = 0 takes t = 1 wherever its
+// set misses the total: either search from 13 dots on (0.35 - 0.97; 12 dots
+// 1.00 - 1.10 from 10,000 pixels on, 0.65 - 1.01 below).
+//   Close pixels make small open rasters of 12 dots and more a case of their
+// own.  A pixel that the one-pass search cannot settle costs the list kernel 4
+// to 8 us however few they are, which a large raster hides and one of a few
+// pixels does not meet: below 64 pixels 0.61 - 0.83, but at 600 and 2,400 the
+// sphere search takes 0.96 - 1.46 (closed, where tiles cost more, 0.93 - 1.22
+// and 0.79 - 1.0).  Tiles there, unless they would be the pruned search (0.80 -
+// 0.93).
 int choose_search(const qa_model* m, const qa::ArrayDesc& d, long long P) {
   if (m->host_stale || !std::isfinite(m->host.s.msum)) return qa::kSearchTiles;
   const int n = m->n;
   if (n >= qa::kSphereMinDot && !m->host.s.valid) return qa::kSearchTiles;
   const double t = d.mt.t;
-  const bool closed = d.mt.closed != 0;
-  // (a closed array at t = 0 takes t = 1 wherever its set misses the total)
-  const double kexp = t >= 1.0 || (closed && t <= 0.0) ? (double)n : (double)n * std::log2(1.0 + t);
-  if (use_sphere(n, kexp, P, closed, d.cfg)) return qa::kSearchSphere;
+  const bool closed = d.mt.closed != 0, all = closed && t <= 0.0;
+  const double kexp = t >= 1.0 || all ? (double)n : (double)n * std::log2(1.0 + t);
   // the list kernel repeats the sums of these configurations of the FP32 search
+  const bool bnb = qa::bnb_search(d.cfg.L1, d.cfg.L2);
   const bool listed = d.cfg.L1 >= 4 && (d.cfg.T < qa::kTeamFinishMin || d.cfg.L2 == 4);
-  if (n < 3 || !listed) return qa::kSearchTiles;
-  if (n <= 8) return qa::kSearchDense;
-  if (n < 12) return kexp < (closed ? 9.5 : 8.9) ? qa::kSearchDense : qa::kSearchTiles;
-  if (closed) return kexp < 11.01 || t <= 0.0 ? qa::kSearchMixed : qa::kSearchTiles;
-  return kexp < (P >= 30000 ? 9.4 : 4.6) ? qa::kSearchMixed : qa::kSearchTiles;
+  const bool full = P >= 32LL * m->num_sms;
+  if (n < 3) return qa::kSearchTiles;
+  if (n < qa::kSphereMinDot) {
+    const bool dense = n <= 8 || kexp < (full ? 9.5 : 11.01);
+    return dense && listed ? qa::kSearchDense : qa::kSearchTiles;
+  }
+  if (kexp >= 11.01 && !all) {
+    const bool close_hidden = closed || full || P < 64;
+    const bool has_sums = d.cfg.L1 == 5 && d.cfg.T >= qa::kTeamFinishMin;
+    return has_sums && (close_hidden || bnb) ? qa::kSearchSphere : qa::kSearchTiles;
+  }
+  const bool mixed = all ? n > 12 || !full
+                         : closed || kexp < (P >= 192LL * m->num_sms ? 9.4 : 4.6);
+  return mixed && listed ? qa::kSearchMixed : qa::kSearchTiles;
 }
 
 // Lanes and slots of the search that runs, for the statistics: the sphere

@@ -167,3 +167,21 @@ def test_closed_far_from_the_induced_charge(qa, n, a, N, t):
     np.testing.assert_array_equal(x[2], y[2])
     mag = np.abs(np.linalg.inv(Cdd)).sum() * (2.0 * N / n) ** 2
     np.testing.assert_allclose(x[1], y[1], rtol=0, atol=2.0 ** -44 * mag)
+
+
+@pytest.mark.parametrize("n,closed,t,W,H,N", [
+    # either side of the dispatch's lines: the sizes where a small raster's rule
+    # ends, 9 to 11 dots around 9.5 expected ambiguous ones
+    (9, False, 1.0, 100, 60, 0), (10, False, 1.0, 60, 40, 0), (10, False, 1.0, 152, 32, 0),
+    (11, False, 1.0, 9, 7, 0), (11, False, 0.8, 120, 90, 0), (11, True, 1.0, 60, 40, 11),
+    (10, True, 1.0, 60, 40, 7), (12, False, 1.0, 9, 7, 0), (12, False, 1.0, 8, 8, 0),
+    (12, False, 1.0, 128, 38, 0), (12, False, 1.0, 127, 38, 0), (13, False, 0.6, 100, 100, 0),
+    (14, False, 0.7, 100, 100, 0), (15, False, 0.4, 60, 40, 0), (13, True, 1.0, 40, 30, 13),
+    (13, True, 1.0, 38, 32, 13), (12, True, 0.0, 30, 20, 5), (13, True, 0.0, 30, 20, 5),
+    (16, True, 0.7, 40, 31, 16), (16, False, 0.95, 30, 20, 0)])
+def test_either_side_of_the_lines(qa, n, closed, t, W, H, N):
+    Cdd, Cgd, gx, gy, V = _model(n, 3 * n + W)
+    ras = inputs.raster(n, gx, gy, V, lo=-1.0, hi=6.0, W=W, H=H)
+    a, b = _both(qa, Cdd, Cgd, lambda m: (m.ground_state_closed(ras, N, threshold=t) if closed
+                                          else m.ground_state_open(ras, threshold=t)))
+    _same(a, b, f"N={n} closed={closed} t={t} {W} x {H}")

@@ -238,3 +238,30 @@ print(lib.launched().decode())
     assert "k_prep_batch" in out[0] and "k_lists" in out[-1]
     assert sum("k_pixels_batch" in v for v in out) >= 8
     assert [v.startswith("overlapped:") for v in out] == [False, False] + [True] * (len(out) - 2)
+
+
+def test_a_small_raster_of_many_dots_takes_tiles(library):
+    # one-pass searches leave close pixels to the list kernel, which an open
+    # raster of 64 to 4863 pixels does not hide
+    out = _run(library, """
+import ctypes
+import numpy as np
+from paper_2404_04994_gb300 import api, inputs
+lib = api.load()
+lib.launched.restype = ctypes.c_char_p
+for n, closed, t, W in ((14, 0, 1.0, 63), (14, 0, 1.0, 64), (14, 0, 1.0, 4863), (14, 0, 1.0, 4864),
+                        (14, 1, 1.0, 64), (14, 1, 1.0, 4863),
+                        (16, 0, 1.0, 600), (16, 1, 1.0, 600), (13, 0, 0.25, 600), (13, 0, 0.4, 600),
+                        (12, 1, 0.0, 999), (12, 1, 0.0, 9999), (13, 1, 0.0, 9999), (10, 0, 1.0, 4863),
+                        (10, 0, 1.0, 4864), (9, 0, 1.0, 99999)):
+    r = np.random.Generator(np.random.PCG64(2))
+    m = api.qa_model_create(inputs.chain_cdd(r, n), inputs.dense_cgd(r, n))
+    ras = api.make_raster(inputs.raster(n, 0, 1, np.ones(n), W=W, H=1), n)
+    out = np.zeros((W, n), dtype=np.int8)
+    if closed:
+        lib.qa_ground_state_closed(m, ctypes.byref(ras), t, n, out.ctypes.data, None, None, None)
+    else:
+        lib.qa_ground_state_open(m, ctypes.byref(ras), t, out.ctypes.data, None, None, None)
+    print(int("k_pixels" in lib.launched().decode()))
+""")
+    assert "".join(out) == "1001" + "11" + "11" + "10" + "101" + "10" + "1"
