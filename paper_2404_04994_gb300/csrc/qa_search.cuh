@@ -528,15 +528,14 @@ __device__ __forceinline__ void search_lane(const float* __restrict__ sM,
 // (at 1 + L1 + m).  Team-cooperative (lane lt of T); sync after.
 template <int L1, int L2>
 __device__ __forceinline__ void iter_build(const float* sM, const SlotView& sv, int lt, int T,
-                                           float* itab, int step = 0) {
+                                           float* itab) {
   const int k = sv.k;
   const int nmid = min(max(k - L1, 0), L2);
   const int nout = max(k - L1 - L2, 0);
   const int nlb = min(__ffs(T) - 1, nout);
   const int nit = nout - nlb;
   const int s0 = L1 + L2 + nlb;  // the first iteration slot
-  if (step == 0) step = T;  // the lanes that build it
-  for (int e = lt; e < (1 << nit) * kItStride; e += step) {
+  for (int e = lt; e < (1 << nit) * kItStride; e += T) {
     const unsigned it = (unsigned)(e / kItStride);
     const int v = e % kItStride;
     float acc = 0.f;

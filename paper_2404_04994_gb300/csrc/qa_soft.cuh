@@ -767,7 +767,7 @@ struct WideSmem {  // bytes from the start of the dynamic buffer; per team, kSof
         qs(cls + sizeof(unsigned) * kTeams * 8),
         qd(qs + (bwd ? al16(sizeof(float) * kTeams * (tri(K) + K + 1)) : 0)),
         gf(qd + al16(sizeof(float) * kTeams * (bwd ? wide_moments(K) : 1 + K))),
-        red(gf + (bwd ? sizeof(float) * kTeams * 2 * kMaxDot : 0)),
+        red(gf + (bwd ? sizeof(float) * kTeams * kMaxDot : 0)),
         contrib(red + sizeof(float) * kTeams * kWideRow * (bwd ? wide_rows(NIT) : 6 + NIT)),
         total(contrib + (bwd ? al16(sizeof(float) * kTeams * L) : 0)) {}
 };
@@ -941,7 +941,7 @@ template <bool CLOSED, int MODE, int NIT>
 __global__ void __launch_bounds__(kSoftThreads) k_soft_wide(SoftLaunch a) {
   constexpr bool BWD = MODE != kDenseFwd;
   constexpr bool use_ctx = MODE == kDenseBwdCtx;
-  constexpr bool fit = MODE == kDenseFit;
+  static_assert(MODE != kDenseFit, "the fit step beyond 8 dots is k_soft_fit");
   constexpr int K = wide_slots(NIT);
   constexpr int kTeams = kSoftThreads / 32;
   static_assert(kWideIn == 5 && kWideOut == 10, "a warp's lane bits are slots 5..9");
@@ -960,7 +960,7 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_wide(SoftLaunch a) {
   unsigned* cls = reinterpret_cast<unsigned*>(s_dyn + lay.cls) + team * 8;
   float* q_s = reinterpret_cast<float*>(s_dyn + lay.qs) + team * (tri(K) + K + 1);
   float* qd = reinterpret_cast<float*>(s_dyn + lay.qd) + team * (BWD ? wide_moments(K) : 1 + K);
-  float* gf = reinterpret_cast<float*>(s_dyn + lay.gf) + team * 2 * kMaxDot;
+  float* gam = reinterpret_cast<float*>(s_dyn + lay.gf) + team * kMaxDot;
   float* red = reinterpret_cast<float*>(s_dyn + lay.red) +
                team * kWideRow * (BWD ? wide_rows(NIT) : 6 + NIT);
   float* s_contrib = reinterpret_cast<float*>(s_dyn + lay.contrib);
@@ -972,7 +972,6 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_wide(SoftLaunch a) {
   const long long p = (long long)blockIdx.x * kTeams + team;
   const bool active = p < a.sc.P;  // the same for the whole warp
   const float kT = (float)a.kT;
-  float lossp = 0.f;
   soft_setup_team<CLOSED>(a, ts, p, lane, 32, active);
   if (active) {
     const int k = ts.k;
@@ -1198,10 +1197,8 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_wide(SoftLaunch a) {
       if (lane == 0 && a.ctx_out) a.ctx_out[p] = make_uint2(b1, __float_as_uint(logf(Z)));
     } else {
       if (use_ctx) Z = expf(__uint_as_float(a.ctx_in[p].y));
-      if (fit) lossp = fit_loss_grad_team(a, ts, accb, Z, p, gf, lane, 32, true);
-      const float* g = fit ? gf : a.grad_mean + p * n;
+      const float* g = a.grad_mean + p * n;
       // gam_s = sg_s g_s in shared memory, c0 = g . n* - g . <n>
-      float* gam = gf + kMaxDot;
       float c0 = 0.f;
       if (lane < kMaxDot) gam[lane] = 0.f;
       __syncwarp();
@@ -1330,7 +1327,7 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_wide(SoftLaunch a) {
   }
   if (BWD)
     soft_contrib<K>(a, ts, q_s, s_contrib + team * L, s_contrib, sMh, 32, lane, kTeams, active, p,
-                    lossp);
+                    0.f);
 }
 
 // The chain rule through M = Cdd^-1 and c = s Cgd V, from the summed

@@ -13,17 +13,15 @@ namespace qa {
 
 // D(b) = E(b) - E(b*) from the slots that differ from b*: the first-order
 // terms gp / gm of each and the pair terms between them, read from the team's
-// slot-ordered copy of M (Ms[s * KMAX + s2] = M of the dots of slots s, s2).
-template <int KMAX>
-__device__ __forceinline__ float delta_energy(const TeamSlots& ts, const float* Ms,
-                                              unsigned b) {
+// slot-ordered copy of M (Ms[s * 16 + s2] = M of the dots of slots s, s2).
+__device__ __forceinline__ float delta_energy(const TeamSlots& ts, const float* Ms, unsigned b) {
   const unsigned d = b ^ ts.bstar;
   float D = 0.f;
   for (unsigned m = d; m; m &= m - 1u) {
     const int s = __ffs(m) - 1;
     const bool add = (b >> s) & 1u;
     D += add ? ts.gp[s] : ts.gm[s];
-    const float* row = Ms + s * KMAX;
+    const float* row = Ms + s * kMaxDot;
     for (unsigned q = d & ((1u << s) - 1u); q; q &= q - 1u) {
       const int s2 = __ffs(q) - 1;
       const bool add2 = (b >> s2) & 1u;
@@ -35,25 +33,23 @@ __device__ __forceinline__ float delta_energy(const TeamSlots& ts, const float* 
 }
 
 // <n>, loss and the per-block gradient partials of a fit step.
-template <int L1, int L2, bool CLOSED, int KMAX>
+template <bool CLOSED>
 __global__ void __launch_bounds__(kSoftThreads) k_soft_fit(SoftLaunch a) {
+  constexpr int KMAX = kMaxDot, T = 32;  // slots; lanes per pixel
+  constexpr int kTeams = kSoftThreads / T;
   __shared__ ModelConsts cs;
-  __shared__ TeamSlots tsm[kSoftThreads / 4 > 0 ? kSoftThreads / 4 : 1];
-  // slot-ordered M per team (teams of >= 4 lanes for KMAX 8, 32 lanes beyond)
-  constexpr int kMaxTeams = kSoftThreads / (KMAX > 8 ? 32 : 4);
-  __shared__ float slotM[kMaxTeams][KMAX * KMAX];
-  __shared__ float sQa[kMaxTeams][tri(KMAX) + KMAX + 1];  // Qa, va, sa of a team
-  __shared__ float sGf[kMaxTeams][kMaxDot];                 // g of a team
+  __shared__ TeamSlots tsm[kTeams];
+  __shared__ float slotM[kTeams][KMAX * KMAX];         // slot-ordered M of a team
+  __shared__ float sQa[kTeams][tri(KMAX) + KMAX + 1];  // Qa, va, sa of a team
+  __shared__ float sGf[kTeams][kMaxDot];               // g of a team
   extern __shared__ float s_contrib[];  // [teams][contrib_len]
   const int n = a.n;
   stage_consts(&a.md->k, &cs);
   __syncthreads();
   const float* sM = cs.Mhi;
   const float* sMlo = cs.Mlo;
-  const int T = a.cfg.T;  // >= 4
   const int team = threadIdx.x / T, lt = threadIdx.x % T;
-  const int teams = blockDim.x / T;
-  const long long p = (long long)blockIdx.x * teams + team;
+  const long long p = (long long)blockIdx.x * kTeams + team;
   const bool active = p < a.sc.P;
   TeamSlots& ts = tsm[team];
   const float kT = (float)a.kT;
@@ -73,7 +69,7 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_fit(SoftLaunch a) {
   unsigned long long ev = 0;
   if (active) {
     SlotView sv{ts.dot, ts.h, ts.k, ts.w};
-    search_lane<L1, L2, CLOSED, false>(sM, sv, lt, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev);
+    search_lane<5, 4, CLOSED, false>(sM, sv, lt, T, 0.f, nullptr, nullptr, 0u, m1, b1, m2, ev);
   }
   for (int off = 1; off < T; off <<= 1) {
     const float om1 = __shfl_xor_sync(kFullS, m1, off);
@@ -94,7 +90,7 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_fit(SoftLaunch a) {
   if (active) {
     for (unsigned b = (unsigned)lt; b < total; b += (unsigned)T) {
       if (CLOSED && __popc(b) != ts.w) continue;
-      const float wgt = expf(-delta_energy<KMAX>(ts, Ms, b) * inv_kT);
+      const float wgt = expf(-delta_energy(ts, Ms, b) * inv_kT);
       Z += wgt;
 #pragma unroll
       for (int s = 0; s < KMAX; ++s)
@@ -138,7 +134,7 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_fit(SoftLaunch a) {
   if (active) {
     for (unsigned b = (unsigned)lt; b < total; b += (unsigned)T) {
       if (CLOSED && __popc(b) != ts.w) continue;
-      const float wgt = expf(-delta_energy<KMAX>(ts, Ms, b) * inv_kT) * invZ;
+      const float wgt = expf(-delta_energy(ts, Ms, b) * inv_kT) * invZ;
       float gn = 0.f;
 #pragma unroll
       for (int s = 0; s < KMAX; ++s)
@@ -175,21 +171,21 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_fit(SoftLaunch a) {
     q_s[tri(KMAX) + KMAX] = sa;
   }
   __syncwarp();
-  soft_contrib<KMAX>(a, ts, q_s, my, s_contrib, sM, T, lt, teams, active, p, lossp);
+  soft_contrib<KMAX>(a, ts, q_s, my, s_contrib, sM, T, lt, kTeams, active, p, lossp);
 }
 
 template <bool CLOSED>
 static cudaError_t run_soft_fit(const SoftLaunch& a, cudaStream_t st) {
-  const int teams = kSoftThreads / a.cfg.T;
+  constexpr int teams = kSoftThreads / 32;
   const unsigned grid = (unsigned)((a.sc.P + teams - 1) / teams);
   const size_t smem = (size_t)teams * contrib_len(a.n) * sizeof(float);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_soft_fit<5, 4, CLOSED, 16>,
+    cudaError_t e = cudaFuncSetAttribute(k_soft_fit<CLOSED>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   if (a.ev) cudaEventRecord(a.ev[0], st);
-  k_soft_fit<5, 4, CLOSED, 16><<<grid, kSoftThreads, smem, st>>>(a);
+  k_soft_fit<CLOSED><<<grid, kSoftThreads, smem, st>>>(a);
   k_soft_reduce<<<contrib_len(a.n), 256, 0, st>>>(a, (int)grid);
   if (a.ev) cudaEventRecord(a.ev[1], st);
   return cudaGetLastError();
