@@ -156,22 +156,30 @@ __device__ inline void prep_stage_array(const ArrayDesc& a, PrepShared& sh) {
       sh.sG[i][g] = df_from_double(a.mt.carrier * a.md->Cgd[i * a.ng + g]);
     }
   }
-  if (a.sc.kind == 0 && threadIdx.x < kMaxDot) {
-    sh.sc0[threadIdx.x] = a.rk.c0[threadIdx.x];
-    sh.sdu[threadIdx.x] = a.rk.du[threadIdx.x];
-    sh.sdw[threadIdx.x] = a.rk.dw[threadIdx.x];
+  if (a.sc.kind == 0) {
+    bool form = a.rk.gen == 0u;  // on the device
+    if (!form) {
+      if (threadIdx.x < kMaxDot) {
+        sh.sc0[threadIdx.x] = a.rk.c0[threadIdx.x];
+        sh.sdu[threadIdx.x] = a.rk.du[threadIdx.x];
+        sh.sdw[threadIdx.x] = a.rk.dw[threadIdx.x];
+      }
+      // of another host copy than the model's?  (Looked up among the constants;
+      // a load of its own cost a call 0.6 - 1.5 us.)
+      if (!a.rk.current) {
+        __syncthreads();
+        form = a.rk.gen != sh.cs.gen;
+      }
+    }
+    if (form) {
+      // (its voltage vectors in the QP rows, which no pixel uses yet)
+      static_assert(sizeof(sh.qK) >= 3 * kMaxGate * sizeof(df), "room for V0, u, w");
+      df* v = reinterpret_cast<df*>(&sh.qK[0][0]);
+      raster_consts(a.md, a.n, a.ng, a.sc, a.mt.carrier, v, v + kMaxGate, v + 2 * kMaxGate,
+                    sh.sc0, sh.sdu, sh.sdw);
+    }
   }
   __syncthreads();
-  // of another host copy than the model's?  (Looked up among the constants; a
-  // load of its own cost a call 0.6 - 1.5 us.)
-  if (a.sc.kind == 0 && !a.rk.current && (a.rk.gen == 0u || a.rk.gen != sh.cs.gen)) {
-    // (its voltage vectors in the QP rows, which no pixel uses yet)
-    static_assert(sizeof(sh.qK) >= 3 * kMaxGate * sizeof(df), "room for V0, u, w");
-    df* v = reinterpret_cast<df*>(&sh.qK[0][0]);
-    raster_consts(a.md, a.n, a.ng, a.sc, a.mt.carrier, v, v + kMaxGate, v + 2 * kMaxGate, sh.sc0,
-                  sh.sdu, sh.sdw);
-    __syncthreads();
-  }
 }
 
 // c of a point-list pixel by its team (out of line: the raster kernels carry
@@ -1007,11 +1015,11 @@ struct PixelShared {
   PrepShared p;
   unsigned long long cand[kTeams], ev[kTeams];
   unsigned qp[kTeams], doubled[kTeams], boundary[kTeams], overflow[kTeams];
+  int factor;  // sphere search: the model has one
 };
 struct SphereShared : PixelShared<kSphT> {
   SphereModel m;
   float4 lev[kTeams][kMaxDot / 2];
-  int factor;  // the model has one
 };
 // The search of a kernel's pixels: the enumeration, the sphere search, or the
 // one that a pixel's ambiguous dots call for (a warp's pixels alike: the
@@ -1285,28 +1293,28 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
 #pragma unroll
   for (int off = W / 2; off > 0; off >>= 1) S += __shfl_xor_sync(kFull, S, off);
   const unsigned any_qp = __any_sync(kFull, qp);
-  // max_j |base_j - c_j|, which scales the rounding of M r: at most 1 on an open
-  // pixel without active constraints (x = c), but a closed one moves every dot
-  // by lambda v
+  int close = 0;
+  unsigned ev = 0, bits = 0u;
+  const bool sphere =
+      MODE == kPixSphere || (MODE == kPixMixed && __any_sync(kFull, active && k >= kMixedDots));
+  // max_j |base_j - c_j| (and |x_j - c_j| for the gradient below), which scales
+  // the rounding of M r: at most 1 on an open pixel without active constraints
+  // (x = c), but a closed one moves every dot by lambda v.  (The sphere search
+  // with active constraints takes it along with the gradient's sums.)
   float rmax = 1.f;
-  if (CLOSED || any_qp) {
+  if (sphere ? CLOSED && !any_qp : CLOSED || any_qp) {
     rmax = fmaxf(fabsf(r0), 1.f);
 #pragma unroll
     for (int off = W / 2; off > 0; off >>= 1)
       rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
   }
-  const float msum = a.md->s.msum;
-  int close = 0;
-  unsigned ev = 0, bits = 0u;
-  const bool sphere =
-      MODE == kPixSphere || (MODE == kPixMixed && __any_sync(kFull, active && k >= kMixedDots));
   if constexpr (MODE != kPixDense) if (sphere) {
     // the gradient M (x - c) where a constraint is active (else zero, closed: a
     // multiple of 1)
     float a1 = 0.f, neg = 0.f;
     if (any_qp) {
       float z = 0.f;
-      rmax = fmaxf(rmax, fabsf(sh.p.qz[threadIdx.x]));
+      rmax = fmaxf(rmax, fmaxf(fabsf(r0), fabsf(sh.p.qz[threadIdx.x])));
 #pragma unroll
       for (int j = 0; j < W; ++j) z = fmaf(Mrow[j], sh.p.qz[tq + j], z);
       if (CLOSED) {  // the multiple of 1: the least entry, a free dot's
@@ -1323,7 +1331,7 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
         rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
       }
     }
-    const float ez = u24 * msum * rmax;  // u sum |M| |r|
+    const float ez = u24 * a.md->s.msum * rmax;  // u sum |M| |r|
     const float bound = pixel_bound(a, S * 1.00001f + 20.f * ez, k);
     neg += (qp ? 24.f : 2.f) * ez;
     // no factor, or a centre outside [-1, 1] (an unsettled QP): left to the
@@ -1338,7 +1346,7 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
   unsigned* lst =
       reinterpret_cast<unsigned*>(MODE == kPixDense ? &sh.p.qK[tq][0] : &sh.p.qz[tq]);
   if constexpr (MODE != kPixSphere) if (!sphere) {
-    const float ez = u24 * msum * rmax;
+    const float msum = a.md->s.msum, ez = u24 * msum * rmax;
     // twice the near-tie bound as in the sphere search, once more for this
     // search's own sums (at most 2 k + 8 additions), and the error of the
     // plain h on both sides
