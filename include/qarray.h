@@ -384,8 +384,9 @@ typedef struct qa_batch qa_batch;
 /* Prepare a batch of `count` independent arrays of any dot count, raster size
  * and open/closed form: validates every item (as the single-array calls do),
  * uploads one descriptor per array, builds the work-unit queues (runs of
- * pixels of one array, ordered by estimated cost, largest first) and
- * allocates the scratch (per-pixel records for all pixels, the recheck lists).
+ * pixels of one array; those of the search by tiles ordered by estimated cost,
+ * largest first) and allocates the scratch (per-pixel records for all pixels,
+ * the lists).
  * Synchronous; *out is owned by the caller (qa_batch_destroy).  The models
  * and output buffers must outlive the batch; model capacitances may change
  * between runs only through qa_model_update (same shapes).
@@ -393,10 +394,13 @@ typedef struct qa_batch qa_batch;
  * different devices. */
 int qa_batch_create(const qa_batch_item* items, int count, qa_batch** out);
 
-/* Run the batch on `stream`: one persistent prep launch and one persistent
- * search launch whose blocks take work units from a device queue, then the
- * list kernel (near-tie resolve, FP64 recheck) over all arrays.  Asynchronous, allocates
- * nothing and synchronises nothing, so it can be captured in a CUDA graph.
+/* Run the batch on `stream`: persistent grids whose blocks take work units from
+ * device queues -- for the arrays searched by tiles one that prepares and one
+ * per kind of search, for the others one per kind of one-pass search (team
+ * width, open or closed) -- overlapping where they are independent, then the
+ * list kernel (close candidates, near-tie resolve, FP64 recheck) over all
+ * arrays.  Asynchronous, allocates nothing and synchronises nothing, so it can
+ * be captured in a CUDA graph.
  * Runs of one batch must not overlap on the GPU. */
 int qa_batch_run(qa_batch* b, void* stream);
 

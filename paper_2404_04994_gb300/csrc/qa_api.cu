@@ -580,7 +580,7 @@ int make_scan(const qa_model* m, const ScanIn& in, qa::Scan* sc) {
 }
 
 // Brute force (Table I): every state of the box (open) or every composition
-// of N_hat (closed), FP64, one warp per pixel.
+// of N_hat (closed), exact in FP64.
 int run_brute(qa_model* m, const qa_raster* r, int closed, int bound, int8_t* out_n,
               double* out_U, uint8_t* out_flags, void* stream) {
   if (!m) return fail(QA_ERR_INVALID, "null model");

@@ -1,6 +1,7 @@
 // qa_batch.cu -- the batched ground state: many arrays (any N, raster size,
-// open or closed) in one persistent prep launch and one persistent search
-// launch per kernel variant present (split, form, team finish).  Blocks take
+// open or closed).  Those searched by tiles take one persistent prep launch and
+// one persistent search launch per kernel variant present (split, form, team
+// finish), the others the one-pass grids of qa_pixels_batch.cu.  Blocks take
 // work units -- a run of pixels of one array -- from a device queue (an
 // atomic counter over a unit table ordered largest first), stage that array's
 // constants when it changes, and run the same tile code as the single-array

@@ -1005,9 +1005,9 @@ __device__ __forceinline__ df team_energy(const ModelConsts& cs, int n, int lt, 
 // in doubt gets its record and goes on the FP64 list.
 // What bounds it: instruction issue (1,430 warp instructions per 16-dot pixel
 // of the sphere search, 2.4 - 3 a cycle; the tile kernels' 3,061, three
-// quarters of them in the FP32 search).  Whole calls, before / after: 16 dots
-// 100 x 100 57 / 42 us (closed 93 / 60), 16-dot list of 10^4 vectors 71 / 54
-// us, 12 dots 400 x 301 241 / 172 us.
+// quarters of them in the FP32 search).  Whole calls, tiles / so: 16 dots
+// 100 x 100 60 / 43 us (closed 94 / 52), 16-dot list of 10^4 vectors 76 / 57
+// us, 12 dots 400 x 301 243 / 168 us.
 // ---------------------------------------------------------------------------
 template <int W>
 struct PixelShared {

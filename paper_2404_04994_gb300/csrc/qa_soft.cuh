@@ -883,7 +883,12 @@ __device__ __forceinline__ void wide_block(float A, const float (&q)[kWideIn], c
   }
 }
 
-// 2^x, results below FP32's normal range as zero.
+// 2^x, results below FP32's normal range as zero (2^-126 of the largest
+// weight).  Its own two units in the last place are less than what x's rounding
+// makes of the weight, u |x|: for 9 to 14 dots at kT 0.01 to 0.05 <n> is 0.65 -
+// 1.4e-7 rms off FP64 (0.73 - 1.4e-7 with expf of the unscaled energies, one
+// candidate at a time) and the gradient 0.5 - 4.5e-7 of its largest entry (1.7 -
+// 33e-7).
 __device__ __forceinline__ float wide_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
