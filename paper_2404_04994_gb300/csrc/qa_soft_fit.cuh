@@ -4,7 +4,7 @@
 // FP32 rounding of a small entry reaches the FP64 parameters (1e-7 relative
 // where an entry's gradient is below 1e-6), and a fit's trajectory is kept to
 // the bit instead.  What bounds it: issue of the divergent per-candidate sums
-// and 136 register moments (two blocks per SM): 12 dots, 75 x 60, about 1.5 ms.
+// and 136 register moments (two blocks per SM): 12 dots, 75 x 60, 1.5 - 2.6 ms.
 #pragma once
 
 #include "qa_soft.cuh"
@@ -35,8 +35,8 @@ __device__ __forceinline__ float delta_energy(const TeamSlots& ts, const float* 
 // <n>, loss and the per-block gradient partials of a fit step.
 template <bool CLOSED>
 __global__ void __launch_bounds__(kSoftThreads) k_soft_fit(SoftLaunch a) {
-  constexpr int KMAX = kMaxDot, T = 32;  // slots; lanes per pixel
-  constexpr int kTeams = kSoftThreads / T;
+  constexpr int KMAX = kMaxDot;               // slots
+  constexpr int kTeams = kSoftThreads / 32;   // pixels: a warp each
   __shared__ ModelConsts cs;
   __shared__ TeamSlots tsm[kTeams];
   __shared__ float slotM[kTeams][KMAX * KMAX];         // slot-ordered M of a team
@@ -48,8 +48,13 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_fit(SoftLaunch a) {
   __syncthreads();
   const float* sM = cs.Mhi;
   const float* sMlo = cs.Mlo;
+  // 32 (run_soft_fit sees to it), but read at run time: with T or the block's
+  // teams known when compiled the kernel takes 255 registers instead of 196 and
+  // the step a tenth longer (12 dots, 75 x 60: 2635 -> 2907 us)
+  const int T = a.cfg.T;
   const int team = threadIdx.x / T, lt = threadIdx.x % T;
-  const long long p = (long long)blockIdx.x * kTeams + team;
+  const int teams = blockDim.x / T;
+  const long long p = (long long)blockIdx.x * teams + team;
   const bool active = p < a.sc.P;
   TeamSlots& ts = tsm[team];
   const float kT = (float)a.kT;
@@ -171,11 +176,12 @@ __global__ void __launch_bounds__(kSoftThreads) k_soft_fit(SoftLaunch a) {
     q_s[tri(KMAX) + KMAX] = sa;
   }
   __syncwarp();
-  soft_contrib<KMAX>(a, ts, q_s, my, s_contrib, sM, T, lt, kTeams, active, p, lossp);
+  soft_contrib<KMAX>(a, ts, q_s, my, s_contrib, sM, T, lt, teams, active, p, lossp);
 }
 
 template <bool CLOSED>
 static cudaError_t run_soft_fit(const SoftLaunch& a, cudaStream_t st) {
+  if (a.cfg.T != 32) return cudaErrorInvalidValue;  // the kernel's shared arrays
   constexpr int teams = kSoftThreads / 32;
   const unsigned grid = (unsigned)((a.sc.P + teams - 1) / teams);
   const size_t smem = (size_t)teams * contrib_len(a.n) * sizeof(float);
