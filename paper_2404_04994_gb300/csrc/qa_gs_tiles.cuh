@@ -164,12 +164,9 @@ __device__ inline void prep_stage_array(const ArrayDesc& a, PrepShared& sh) {
         sh.sdu[threadIdx.x] = a.rk.du[threadIdx.x];
         sh.sdw[threadIdx.x] = a.rk.dw[threadIdx.x];
       }
-      // of another host copy than the model's?  (Looked up among the constants;
-      // a load of its own cost a call 0.6 - 1.5 us.)
-      if (!a.rk.current) {
-        __syncthreads();
-        form = a.rk.gen != sh.cs.gen;
-      }
+      // of another host copy than the model's?  (The load costs a call 0.6 - 1.5
+      // us: only where the model may have changed.)
+      if (!a.rk.current) form = a.rk.gen != a.md->k.gen;
     }
     if (form) {
       // (its voltage vectors in the QP rows, which no pixel uses yet)
@@ -1015,7 +1012,6 @@ struct PixelShared {
   PrepShared p;
   unsigned long long cand[kTeams], ev[kTeams];
   unsigned qp[kTeams], doubled[kTeams], boundary[kTeams], overflow[kTeams];
-  int factor;  // sphere search: the model has one
 };
 struct SphereShared : PixelShared<kSphT> {
   SphereModel m;
@@ -1039,7 +1035,6 @@ static_assert(kSphT * sizeof(float) * kQPRow >= kSphStack * sizeof(uint2),
 // Block set-up (all threads), once per array.
 __device__ inline void pixel_stage_search(const ArrayDesc& a, SphereShared& sh) {
   sphere_stage(a.md->s, sh.m);
-  if (threadIdx.x == 0) sh.factor = a.md->s.valid;
 }
 template <int W>
 __device__ inline void pixel_stage_search(const ArrayDesc&, PixelShared<W>&) {}
@@ -1335,9 +1330,10 @@ __device__ inline void search_pixel(const GsLaunch& L, const ArrayDesc& a,
     const float bound = pixel_bound(a, S * 1.00001f + 20.f * ez, k);
     neg += (qp ? 24.f : 2.f) * ez;
     // no factor, or a centre outside [-1, 1] (an unsettled QP): left to the
-    // FP32 search
+    // FP32 search.  (The mark is read here: held in shared memory the kernel
+    // spilled registers, 4 % of 10^4 voltage vectors' time.)
     const bool far = ((__ballot_sync(kFull, !(fabsf(f) <= 1.f)) >> hw) & kW) != 0u;
-    bits = sphere_search<CLOSED>(a.md->s, sh.m, n, lt, active && sh.factor && !far, f, a1, q.mask,
+    bits = sphere_search<CLOSED>(a.md->s, sh.m, n, lt, active && a.md->s.valid && !far, f, a1, q.mask,
                                  q.w, bound, neg, &sh.p.qx[tq], &sh.p.qz[tq], sh.lev[team],
                                  reinterpret_cast<uint2*>(&sh.p.qK[tq][0]), close, ev);
   }
